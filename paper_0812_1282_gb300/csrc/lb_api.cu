@@ -17,6 +17,7 @@
 #include "lb_internal.h"
 #include "lb_geo_persist.h"
 #include "lb_node.cuh"
+#include "lb_node64.cuh"
 
 using lbfe::DomDesc;
 using lbfe::StatsOut;
@@ -79,7 +80,7 @@ struct Layout {
     std::vector<size_t> geo_flags;  // its persistent step's tile flags and counter (ints)
     size_t flags = 0, dep_off = 0, dep_idx = 0;  // persistent schedules (batches)
     size_t descs = 0, items = 0, partials = 0, stats = 0, pts = 0, count = 0, staging = 0, err = 0,
-           sched = 0;
+           sched = 0, c64 = 0;
     size_t total = 0;
     long long item_cap = 0;
     int pts_cap = 0;
@@ -119,7 +120,9 @@ bool build_layout(int precision, int n_dom, const int* nx, const int* ny, Layout
     // at least one full row, so host field output can always go row by row
     L.staging_nodes = std::max(std::min<long long>(max_nodes, kChunk), max_nx);
     L.descs = off;
-    off = align_up(off + sizeof(DomDesc) * n_dom, kAlign);
+    off += sizeof(DomDesc) * n_dom;
+    L.c64 = off;  // FP64 node constants, uploaded with the descriptors
+    off = align_up(off + (precision == LB_FP64 ? sizeof(lbfe::Node64) * n_dom : 0), kAlign);
     L.items = off;
     off = align_up(off + sizeof(WorkItem) * (n_dom > 1 ? item_cap : 1), kAlign);
     L.flags = off;
@@ -928,6 +931,7 @@ int make_handle(const lb_params* per_dom, const int* nx, const int* ny, int n_do
         h->base = static_cast<unsigned char*>(p);
         h->owns = true;
     }
+    std::vector<lbfe::Node64> c64;
     for (int d = 0; d < n_dom; ++d) {
         const lb_params& p = per_dom[d];
         DomDesc D{};
@@ -980,11 +984,22 @@ int make_handle(const lb_params* per_dom, const int* nx, const int* ny, int n_do
             D.hcls[k] = 0.0;
             D.fhcls[k] = 0.0f;
         }
+        D.c64 = nullptr;
+        if (h->precision == LB_FP64) {
+            D.c64 = reinterpret_cast<const double*>(h->base + L.c64 + sizeof(lbfe::Node64) * d);
+            c64.push_back(lbfe::make_node64(D.a, D.kappa, D.gamma, D.omega_phi, D.tau_c0, D.tau_c1,
+                                            D.lut_lo, D.lut_step, D.lut_inv, D.lut_kmax));
+        }
         h->descs.push_back(D);
     }
+    static_assert(sizeof(DomDesc) % alignof(lbfe::Node64) == 0, "constants follow the descriptors");
+    std::vector<unsigned char> tables(sizeof(DomDesc) * n_dom + sizeof(lbfe::Node64) * c64.size());
+    memcpy(tables.data(), h->descs.data(), sizeof(DomDesc) * n_dom);
+    if (!c64.empty())
+        memcpy(tables.data() + sizeof(DomDesc) * n_dom, c64.data(), sizeof(lbfe::Node64) * c64.size());
     if ((e = cudaMemsetAsync(h->base, 0, L.total, h->stream)) != cudaSuccess ||
-        (e = cudaMemcpyAsync(h->d_descs(), h->descs.data(), sizeof(DomDesc) * n_dom,
-                             cudaMemcpyHostToDevice, h->stream)) != cudaSuccess ||
+        (e = cudaMemcpyAsync(h->d_descs(), tables.data(), tables.size(), cudaMemcpyHostToDevice,
+                             h->stream)) != cudaSuccess ||
         (e = cudaStreamSynchronize(h->stream)) != cudaSuccess)
         return bail(fail(LB_ERR_CUDA, "device init failed: %s", cudaGetErrorString(e)));
     // default launch shape: 128 threads (64 with compact storage, whose

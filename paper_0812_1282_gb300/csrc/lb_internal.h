@@ -54,6 +54,7 @@ struct DomDesc {
     const unsigned char* cls;
     double hcls[8];
     float fhcls[8];
+    const double* c64;  // FP64: the node constants (Node64, lb_node64.cuh) in device memory
 };
 
 constexpr int kMaxClass = 7;
@@ -144,8 +145,9 @@ int launch_step_f32(int coll, const DomDesc& d, const DomDesc* d_descs, const Wo
                     int n_items, int n_dom, int parity, int bx, int rows, int band_mul, int grid_p,
                     int* sched, bool one_body, void* stream);
 int launch_step_f64(int coll, const DomDesc& d, const DomDesc* d_descs, const WorkItem* d_items,
-                    int n_items, int n_dom, int parity, int bx, int rows, int band_mul, int grid_p,
-                    int* sched, bool one_body, void* stream);
+                    int n_items, int n_dom, int parity, int bx, int rows, int grid_p, int* sched,
+                    void* stream);
+size_t step_smem_f64(int bx);
 int prepare_step_f32();
 int prepare_step_f64();
 

@@ -18,7 +18,7 @@ size_t step_smem_bytes(int precision, int bx)
 {
     if (bx < 32 || bx > 256 || bx % 32) return 0;
     return precision == 0 ? StageLayout<float>(bx / 32, kStages<float>).total()
-                          : StageLayout<double>(bx / 32, kStages<double>).total();
+                          : step_smem_f64(bx);
 }
 
 int prepare_step_kernels()
@@ -40,7 +40,7 @@ int launch_step(int precision, int coll, const DomDesc& d, const DomDesc* d_desc
                ? launch_step_f32(coll, d, d_descs, d_items, n_items, n_dom, parity, block_x, rows,
                                  band_mul, grid_persistent, sched, one_body, stream)
                : launch_step_f64(coll, d, d_descs, d_items, n_items, n_dom, parity, block_x, rows,
-                                 band_mul, grid_persistent, sched, one_body, stream);
+                                 grid_persistent, sched, stream);
 }
 
 static int step_occupancy(int precision, int coll, int compact, int block_x, int single)
