@@ -281,7 +281,8 @@ int lb_load_state(lb_handle* h, const void* host_buf, size_t bytes);
  * [32, 256], or [32, 288] with compact g storage) and rows each CTA marches
  * through (rows >= 1).  Results do not
  * depend on it.  On a batch it sets a one-class schedule with that shape
- * (lb_schedule).  Invalidates captured graphs. */
+ * (lb_schedule).  Invalidates captured graphs.  A handle starts with a shape
+ * chosen from its domains' sizes. */
 int lb_set_tile(lb_handle* h, int block_x, int rows);
 int lb_get_tile(const lb_handle* h, int* block_x, int* rows);
 

@@ -504,6 +504,113 @@ int build_items(lb_handle* h)
     return LB_OK;
 }
 
+// The schedule a handle starts with (lb_autotune times others): one class,
+// a persistent grid of up to 8 CTAs per SM, and a launch shape from the
+// domains' sizes.  A CTA marches through its rows in series, about 1.05 us a
+// row in FP32 and 4.7 us in FP64 whatever its width, so small lattices want
+// their rows spread over the whole GPU, and large ones rows enough per CTA to
+// carry its lead-in rows:
+//  - the fewest rows with which all CTAs are resident at once (batches: with
+//    5 % more, their last items being small), while that is at most 32 rows
+//    (single domains; 24 and 6 for batches with compact and full storage);
+//  - beyond that single domains take equal waves of at most 12 rows (compact:
+//    16 rows of the wider strips), batches the most.
+//  - FP64 is bound by the FP64 pipe of each SM, so what counts is that the SMs
+//    get equal shares: 64 columns and one wave while that takes at most 4
+//    rows, beyond it 128 columns (more CTAs hide the row barrier) and the most
+//    rows up to 10 (batches 16) that leave each SM eight CTAs; 128 columns too
+//    where every CTA has an SM to itself.
+// Widths else: 128 columns in full storage, four CTAs per SM (1200^2: 20 rows
+// 40.8 us, five CTAs' 16 rows 42.1; 1500^2 30 rows 60, 24 rows 65); compact 96
+// columns for a single domain, and for batches the narrowest strip that holds
+// a domain of mean width (weighted by nodes), so that most are one strip.
+// Items go largest first when one wave holds them (40 drops of 48..200,
+// compact: 24.5 against 25.6 us) and in FP64, in domain order else (256
+// drops, compact: 435 against 445 us).
+// Measured, us per step, with 128 x 32 (compact 64 x 32) and with this rule:
+// FP32 28 x 15 17 -> 4.0, 200 x 100 31 -> 4.4, 512 x 256 32 -> 6.9, 1024^2 39
+// -> 29; compact 200 x 100 40 -> 4.9, 1000 x 500 40 -> 13.7; FP64 200 x 100 158
+// -> 11, 512 x 256 158 -> 35, 1024^2 247 -> 214; 40 drops FP32 43 -> 27, compact
+// 55 -> 25, FP64 248 -> 165.
+lb_schedule default_schedule(const lb_handle* h)
+{
+    const bool compact = h->descs[0].compact != 0, fp64 = h->precision == LB_FP64;
+    const bool single = h->n_dom == 1;
+    double nodes = 0.0, width = 0.0;
+    int max_ny = 1;
+    for (const DomDesc& D : h->descs) {
+        nodes += double(D.nx) * D.ny;
+        width += double(D.nx) * D.ny * D.nx;
+        max_ny = std::max(max_ny, D.ny);
+    }
+    auto strip = [&](int bx) { return compact ? lbfe::compact_strip(bx) : bx; };
+    // CTAs of a shape over all domains; they fall as rows grow
+    auto ctas = [&](int bx, int rows) {
+        long long n = 0;
+        for (const DomDesc& D : h->descs)
+            n += (long long)((D.nx + strip(bx) - 1) / strip(bx)) * ((D.ny + rows - 1) / rows);
+        return n;
+    };
+    // fewest rows of at most `limit` CTAs (max_ny + 1: there are none)
+    auto rows_for = [&](int bx, long long limit) {
+        int lo = 1, hi = max_ny + 1;
+        while (lo < hi) {
+            const int mid = (lo + hi) / 2;
+            if (ctas(bx, mid) <= limit)
+                hi = mid;
+            else
+                lo = mid + 1;
+        }
+        return lo;
+    };
+    auto wave = [&](int bx) {
+        const int occ = single ? lbfe::step_single_occupancy(h->precision, h->coll, compact, bx)
+                               : lbfe::step_batch_occupancy(h->precision, h->coll, compact, bx);
+        const long long per = single && !compact && !fp64 ? std::min(occ, 4) : occ;
+        return std::max<long long>(per, 1) * h->sm_count * (single ? 100 : 105) / 100;
+    };
+    int bx = 128, rows = 1;
+    bool one_wave = true;
+    if (fp64) {
+        const int most = single ? 10 : 16;
+        if (ctas(128, 1) > h->sm_count) {
+            rows = rows_for(64, wave(64));
+            one_wave = rows <= 4;
+            if (one_wave)
+                bx = 64;
+            else
+                rows = std::min(most, std::max(1, rows_for(128, 8LL * h->sm_count - 1) - 1));
+        }
+    } else {
+        if (compact) {
+            bx = single ? 96 : 64;
+            while (!single && bx < 128 && strip(bx) < width / nodes) bx += 32;
+        }
+        const int most = single ? 32 : (compact ? 24 : 6);
+        rows = rows_for(bx, wave(bx));
+        one_wave = rows <= most;
+        if (!one_wave && !single) {
+            rows = most;
+        } else if (!one_wave && compact) {
+            bx = 128;
+            rows = 16;
+        } else if (!one_wave) {
+            const long long w = wave(bx), waves = (ctas(bx, 12) + w - 1) / w;
+            rows = rows_for(bx, waves * w);
+        }
+    }
+    lb_schedule s{};
+    s.n_class = 1;
+    for (int c = 0; c < LB_MAX_SCHED_CLASSES; ++c) {
+        s.block_x[c] = bx;
+        s.rows[c] = rows;
+        s.ctas_per_sm[c] = 8;
+    }
+    s.order = !single && (one_wave || fp64);
+    s.chains = 1;
+    return s;
+}
+
 // Grid of class c's launch: a persistent grid, or one CTA per work item.
 int class_grid(const lb_handle* h, int c)
 {
@@ -1002,18 +1109,7 @@ int make_handle(const lb_params* per_dom, const int* nx, const int* ny, int n_do
                              h->stream)) != cudaSuccess ||
         (e = cudaStreamSynchronize(h->stream)) != cudaSuccess)
         return bail(fail(LB_ERR_CUDA, "device init failed: %s", cudaGetErrorString(e)));
-    // default launch shape: 128 threads (64 with compact storage, whose
-    // threads take two columns each) x 32 rows, one class, a persistent grid
-    // of up to 8 CTAs per SM, items in domain order (tuned by lb_autotune)
-    h->sched.n_class = 1;
-    for (int c = 0; c < LB_MAX_SCHED_CLASSES; ++c) {
-        h->sched.max_nx[c] = 0;
-        h->sched.block_x[c] = h->descs[0].compact ? 64 : 128;
-        h->sched.rows[c] = 32;
-        h->sched.ctas_per_sm[c] = 8;
-    }
-    h->sched.order = 0;
-    h->sched.chains = 1;
+    h->sched = default_schedule(h);
     const int rc = build_items(h);
     if (rc != LB_OK) return bail(rc);
     *out = h;
@@ -1867,7 +1963,7 @@ std::vector<lb_schedule> batch_candidates(const lb_handle* h)
     const bool compact = h->descs[0].compact != 0;
     std::vector<int> widths = compact ? std::vector<int>{64, 96, 128} : std::vector<int>{64, 128, 256};
     if (h->precision == LB_FP64) widths = {64, 128};
-    std::vector<lb_schedule> out;
+    std::vector<lb_schedule> out{default_schedule(h)};
     auto occ = [&](int bx) {
         return std::max(1, lbfe::step_batch_occupancy(h->precision, h->coll, compact, bx));
     };
@@ -1961,6 +2057,14 @@ int lb_autotune(lb_handle* h, int reps, int* block_x, int* rows, double* best_ms
             h->descs[0].compact ? std::vector<int>{32, 64, 96, 128, 160, 192, 224, 256, 288}
                                 : std::vector<int>{64, 128, 256};
         const int rws[] = {4, 8, 16, 32, 64, 128};
+        {
+            const lb_schedule d = default_schedule(h);
+            lb_schedule s = h->sched;
+            s.n_class = 1;
+            s.block_x[0] = d.block_x[0];
+            s.rows[0] = d.rows[0];
+            cands.push_back(s);
+        }
         for (int bx : bxs)
             for (int r : rws) {
                 if (r > max_ny && r != rws[0]) continue;
