@@ -78,6 +78,7 @@ struct Layout {
     std::vector<size_t> dom_bytes;  // bytes of one ping-pong buffer of domain d
     std::vector<size_t> geo_off;    // domain d's obstacle map (nx*ny bytes)
     std::vector<size_t> geo_flags;  // its persistent step's tile flags and counter (ints)
+    std::vector<size_t> geo_tiles;  // its tile list (ints)
     size_t flags = 0, dep_off = 0, dep_idx = 0;  // persistent schedules (batches)
     size_t descs = 0, items = 0, partials = 0, stats = 0, pts = 0, count = 0, staging = 0, err = 0,
            sched = 0, c64 = 0;
@@ -108,6 +109,8 @@ bool build_layout(int precision, int n_dom, const int* nx, const int* ny, Layout
         off = align_up(off + nodes, kAlign);
         L.geo_flags.push_back(off);
         off = align_up(off + sizeof(int) * (size_t(lbfe::geo_tiles(nx[d], ny[d])) + 1), kAlign);
+        L.geo_tiles.push_back(off);
+        off = align_up(off + sizeof(int) * lbfe::geo_tile_capacity(nx[d], ny[d]), kAlign);
         max_nodes = std::max(max_nodes, (long long)nx[d] * ny[d]);
         max_nx = std::max<long long>(max_nx, nx[d]);
         // at most ceil(nx / 28) strips per row (the narrowest strip of any
@@ -225,6 +228,8 @@ struct lb_handle {
     std::map<std::pair<int, int>, cudaGraphExec_t> graphs;  // (length, start parity)
     std::vector<double> host_pts;
     int n_geo = 0;  // domains with an obstacle map
+    // rows of each domain's step tiles and the length of its tile list
+    std::vector<std::pair<int, int>> geo_tiles;
 
     DomDesc* d_descs() const { return reinterpret_cast<DomDesc*>(base + L.descs); }
     WorkItem* d_items() const { return reinterpret_cast<WorkItem*>(base + L.items); }
@@ -704,6 +709,8 @@ int enqueue_geo_steps(lb_handle* h, int len, int parity, bool fixed_parity, cuda
         const DomDesc& D = h->descs[d];
         if (!D.cls) continue;
         int e = 0;
+        const int* tiles = reinterpret_cast<const int*>(h->base + h->L.geo_tiles[d]);
+        const auto [tile_rows, n_tiles] = h->geo_tiles[d];
         if (geo_persistent(h, D)) {
             int* flags = reinterpret_cast<int*>(h->base + h->L.geo_flags[d]);
             e = lbfe::launch_geo_persist(h->precision, h->coll, D, parity, fixed_parity ? 0 : 1, len,
@@ -716,11 +723,13 @@ int enqueue_geo_steps(lb_handle* h, int len, int parity, bool fixed_parity, cuda
                                            fixed_parity ? parity : parity ^ (k & 1), s);
             if (e == 0 && (len & 1))
                 e = lbfe::launch_geo_step(h->precision, h->coll, D,
-                                          fixed_parity ? parity : parity ^ (pairs & 1), s);
+                                          fixed_parity ? parity : parity ^ (pairs & 1),
+                                          tile_rows, tiles, n_tiles, s);
         } else {
             for (int k = 0; k < len && e == 0; ++k)
                 e = lbfe::launch_geo_step(h->precision, h->coll, D,
-                                          fixed_parity ? parity : parity ^ (k & 1), s);
+                                          fixed_parity ? parity : parity ^ (k & 1), tile_rows,
+                                          tiles, n_tiles, s);
         }
         if (e != 0)
             return fail(LB_ERR_CUDA, "obstacle step launch failed: %s", cudaGetErrorString(cudaError_t(e)));
@@ -1001,6 +1010,7 @@ int make_handle(const lb_params* per_dom, const int* nx, const int* ny, int n_do
     h->precision = per_dom[0].precision;
     h->coll = per_dom[0].collision;
     h->params.assign(per_dom, per_dom + n_dom);
+    h->geo_tiles.assign(n_dom, {8, 0});
     h->L = L;
     h->stream = static_cast<cudaStream_t>(stream);
     auto bail = [&](int rc) {
@@ -1521,6 +1531,12 @@ int lb_set_geometry(lb_handle* h, int dom, const unsigned char* cls, const doubl
     const bool had = D.cls != nullptr;
     if (cls) {
         LB_CUDA(cudaMemcpyAsync(dev, cls, size_t(D.nx) * D.ny, cudaMemcpyHostToDevice, h->stream));
+        const lbfe::GeoTiles t =
+            lbfe::make_geo_tiles(h->precision, h->sm_count, cls, D.nx, D.ny, D.walls);
+        LB_CUDA(cudaMemcpyAsync(h->base + h->L.geo_tiles[dom], t.list.data(),
+                                sizeof(int) * t.list.size(), cudaMemcpyHostToDevice, h->stream));
+        LB_CUDA(cudaStreamSynchronize(h->stream));
+        h->geo_tiles[dom] = {t.rows, int(t.list.size())};
         D.cls = dev;
         for (int k = 0; k < 8; ++k) {
             D.hcls[k] = k < n_class ? h_class[k] : 0.0;

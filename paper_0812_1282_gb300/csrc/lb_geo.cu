@@ -23,32 +23,42 @@
 // colliding; its fluid neighbours see phi(x, 0) = phi(x, 1) - h_bot (phi(x,
 // ny-1) = phi(x, ny-2) - h_top) and are Step-2 nodes.
 //
-// A step is one launch.  A CTA owns a tile of kGTX x kGTY nodes (one per
-// thread) and, in shared memory:
-//   1. the class map of the tile and a kGC-node halo;
-//   2. phi of the tile and a kGH-node halo, each fluid node's sum of its
-//      pulled g (Eq. moments): a ghost value at a solid neighbour reads phi
-//      up to three nodes from the fluid node it serves (the solid node, then
-//      twice the direction towards fluid), and the pulls of the halo reach
-//      one node further;
-// then each fluid node of the tile pulls f and g, takes the phi stencil
-// from shared memory (ghost values at solid neighbours), collides (the node
-// arithmetic of the plain step) and stores.  Halo nodes are formed by
-// several CTAs with the same arithmetic, so every tile sees the same phi.
-// Solid nodes are never written by a step; they hold the rest state
-// (f = t, g = 0), so they carry no fluid.
+// A step is one launch over the tiles that hold a fluid or wall node (a list
+// the host makes with the map).  A CTA owns a tile of 32 x TY nodes (one per
+// thread) and, in shared memory, the class map of the tile and a four-node
+// halo.  Then
+//   1. each thread pulls f and g of its node and g of one halo position, and
+//      stores the phi of both (Eq. moments).  A tile needs phi on a one-node
+//      halo, and a tile with a solid neighbour somewhere on a three-node one:
+//      a ghost value reads phi up to two nodes from its solid node;
+//   2. in such a tile each solid node on the tile and its one-node halo gets
+//      its ghost value, once, into the same phi array;
+//   3. each fluid node takes its 3 x 3 phi from shared memory, collides (the
+//      node arithmetic of the plain step) and stores.
+// Halo nodes are formed by several CTAs with the same arithmetic, so every
+// tile sees the same phi.  Solid nodes are never written by a step; they hold
+// the rest state (f = t, g = 0), so they carry no fluid.
 //
 // The obstacle path serves small and medium geometries (the capillary set-up
 // is ~10^5 nodes) whose state stays in L2: a step is bound by launch and L2
 // latency rather than by HBM bandwidth, so it uses plain loads instead of
 // the staged pipeline of the plain step, and one launch with one shared
-// phi field instead of a phi pass through memory.
+// phi field instead of a phi pass through memory.  Measured, us per step:
+// 1000 x 120 channel FP32 7.6 -> 5.3 (a three-node phi halo in every tile,
+// ghost values formed anew for each fluid neighbour, g pulled twice, tiles of
+// solid nodes launched; then as above), 2000 x 200 FP32 18 -> 10.9, 401 x 77
+// FP64 22 -> 10.2 (with the arithmetic of lb_node64.cuh); a single tile 4.2 ->
+// 3.2, of which the launch is about half.
 #include <cuda_runtime.h>
+
+#include <algorithm>
+#include <vector>
 
 #include "lb_async.cuh"
 #include "lb_internal.h"
 #include "lb_geo_persist.h"
 #include "lb_node.cuh"
+#include "lb_node64.cuh"
 
 namespace lbfe {
 
@@ -117,12 +127,14 @@ struct GeoView {
     __device__ __forceinline__ bool solid(int x, int y) const { return cls_at(x, y) != 0; }
 };
 
-// Tile of the fused obstacle step and its halos.
-constexpr int kGTX = 32, kGTY = 8;  // nodes of one CTA (one per thread)
-constexpr int kGH = 3;              // phi halo
-constexpr int kGC = kGH + 1;        // class-map halo
-constexpr int kGCX = kGTX + 2 * kGC, kGCY = kGTY + 2 * kGC;
-constexpr int kGPX = kGTX + 2 * kGH, kGPY = kGTY + 2 * kGH;
+// Tile of a step and its halos: 32 x TY nodes, one per thread.
+constexpr int kGTX = 32;
+constexpr int kGH = 3;        // phi halo
+constexpr int kGC = kGH + 1;  // class-map halo
+constexpr int kGCX = kGTX + 2 * kGC, kGPX = kGTX + 2 * kGH;
+// Rows of the multi-step forms' tiles (persistent, two steps); the per-step
+// form takes 8 or 4 (GeoTiles).
+constexpr int kGTY = 8;
 
 // periodic index for any offset (halos may exceed a small lattice)
 __device__ __forceinline__ int wrap_any(int v, int n)
@@ -134,18 +146,21 @@ __device__ __forceinline__ int wrap_any(int v, int n)
 // Per-CTA tables of a tile: the wrapped halo coordinates and the class map
 // with its halo.  They depend only on the geometry, so the persistent form
 // builds them once per launch.
+template <int TY>
 struct GeoTables {
-    int colx[kGCX];  // wrapped column (+ kXOff) of each halo column
-    int rowo[kGCY];  // offset of each halo row (wrapped row x pitch)
-    int rowc[kGCY];  // the same row in the class map (wrapped row x nx)
-    signed char cl[kGCY][kGCX];  // 0 fluid, k > 0 solid class k, -1 / -2 wall rows
+    int colx[kGCX];          // wrapped column (+ kXOff) of each halo column
+    int rowo[TY + 2 * kGC];  // offset of each halo row (wrapped row x pitch)
+    int rowc[TY + 2 * kGC];  // the same row in the class map (wrapped row x nx)
+    signed char cl[TY + 2 * kGC][kGCX];  // 0 fluid, k > 0 solid class k, -1 / -2 wall rows
 };
 
-__device__ __forceinline__ void geo_tile_setup(const DomDesc& D, int x0, int y0, GeoTables& t)
+template <int TY>
+__device__ __forceinline__ void geo_tile_setup(const DomDesc& D, int x0, int y0, GeoTables<TY>& t)
 {
+    constexpr int CY = TY + 2 * kGC;
     const int nx = D.nx, ny = D.ny;
-    // 0. periodic wrap of the halo coordinates
-    for (int k = threadIdx.x; k < kGCX + kGCY; k += blockDim.x) {
+    // periodic wrap of the halo coordinates
+    for (int k = threadIdx.x; k < kGCX + CY; k += blockDim.x) {
         if (k < kGCX)
             t.colx[k] = wrap_any(x0 - kGC + k, nx) + kXOff;
         else {
@@ -155,8 +170,8 @@ __device__ __forceinline__ void geo_tile_setup(const DomDesc& D, int x0, int y0,
         }
     }
     __syncthreads();
-    // 1. class map (0 fluid, k > 0 solid class k, -1 / -2 bottom / top wall row)
-    for (int k = threadIdx.x; k < kGCX * kGCY; k += blockDim.x) {
+    // class map (0 fluid, k > 0 solid class k, -1 / -2 bottom / top wall row)
+    for (int k = threadIdx.x; k < kGCX * CY; k += blockDim.x) {
         const int cy = k / kGCX, cx = k - cy * kGCX;
         const int y = y0 - kGC + cy;
         int c;
@@ -182,16 +197,216 @@ __device__ __forceinline__ Real geo_ld(const Real* p)
         return *p;
 }
 
-// The step of one fluid or wall node (x, y) of class cme from its pulled
-// populations f, g: cls_l(x, y) reads the class map and phi_l(x, y) phi of
-// the same state around the node (lattice coordinates; ghost values at solid
-// neighbours reach three nodes away); fo, go receive the new populations.
-template <typename Real, bool MRT, class ClsF, class PhiF>
-__device__ __forceinline__ void geo_node_update(const DomDesc& D, int x, int y, int cme,
-                                                const Real (&f)[9], const Real (&g)[9], ClsF cls_l,
-                                                PhiF phi_l, Real (&fo)[9], Real (&go)[9])
+// Wetting ghost value of the solid node at (x, y), or the one-sided value a
+// wall node shows its fluid neighbours; false if no fluid touches it (then
+// nothing reads it).  cls(x, y) and phi(x, y) read the class map and phi around
+// it; y_lat is its lattice row.  The mean over the axis (or, through a corner
+// only, the diagonal) directions d towards fluid of phi(s + k d) - k h, k =
+// D.wet_k.
+template <typename Real, class ClsF, class PhiF>
+__device__ __forceinline__ bool geo_ghost(const DomDesc& D, int x, int y, int y_lat, ClsF cls,
+                                          PhiF phi, Real& value)
 {
-    const int ny = D.ny;
+    const Real h_bot = sizeof(Real) == 4 ? Real(D.fh_bot) : Real(D.h_bot);
+    const Real h_top = sizeof(Real) == 4 ? Real(D.fh_top) : Real(D.h_top);
+    const int k = cls(x, y);
+    if (k == kNodeWall) {
+        value = y_lat == 0 ? phi(x, y + 1) - h_bot : phi(x, y - 1) - h_top;
+        return true;
+    }
+    const Real h = k == -1 ? h_bot : (k == -2 ? h_top : class_h<Real>(D, k));
+    Real sum = Real(0);
+    int n = 0;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const int dx = j == 0 ? 1 : (j == 1 ? -1 : 0);
+        const int dy = j == 2 ? 1 : (j == 3 ? -1 : 0);
+        if (cls(x + dx, y + dy) == 0) {
+            sum += phi(x + D.wet_k * dx, y + D.wet_k * dy);
+            ++n;
+        }
+    }
+    if (n == 0) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int dx = (j == 0 || j == 3) ? 1 : -1;
+            const int dy = (j == 0 || j == 2) ? 1 : -1;
+            if (cls(x + dx, y + dy) == 0) {
+                sum += phi(x + D.wet_k * dx, y + D.wet_k * dy);
+                ++n;
+            }
+        }
+    }
+    if (n == 0) return false;
+    const Real mean =
+        n == 1 ? sum : (n == 2 ? sum * Real(0.5) : (n == 3 ? div_const<3>(sum) : sum * Real(0.25)));
+    value = mean - Real(D.wet_k) * h;
+    return true;
+}
+
+// The node constants of a CTA (FP64 only) and their load.
+template <typename Real>
+struct GeoConst {
+    __device__ __forceinline__ void load(const DomDesc&) {}
+};
+template <>
+struct GeoConst<double> {
+    Node64 c;
+    __device__ __forceinline__ void load(const DomDesc& D)
+    {
+        load_node64(c, D.c64, int(threadIdx.x));
+    }
+};
+
+// Collision of one fluid node from its pulled f, g, its phi c and the phi of
+// its eight neighbours (ghost values at solid ones), directions 1..8 in nb.
+template <typename Real, bool MRT>
+__device__ __forceinline__ void geo_collide(const DomDesc& D, const GeoConst<Real>& K,
+                                            const Real (&f)[9], const Real (&g)[9], Real c,
+                                            const Real (&nb)[9], bool step2, Real (&fo)[9],
+                                            Real (&go)[9])
+{
+    if constexpr (sizeof(Real) == 8) {
+        const Node64& C = K.c;
+        // the stencils of Eq. (best) on scaled values (collide64)
+        const double p = LB64_SUB(nb[5], nb[6]), q = LB64_SUB(nb[8], nb[7]);
+        const double X = __fma_rn(C.four, LB64_SUB(nb[1], nb[2]), LB64_ADD(p, q));
+        const double Y = __fma_rn(C.four, LB64_SUB(nb[3], nb[4]), LB64_SUB(p, q));
+        const double a = LB64_ADD(LB64_ADD(nb[1], nb[2]), LB64_ADD(nb[3], nb[4]));
+        const double d = LB64_ADD(LB64_ADD(nb[5], nb[6]), LB64_ADD(nb[7], nb[8]));
+        const double L = __fma_rn(C.m20, c, __fma_rn(C.four, a, d));
+        collide64<MRT>(C, f, c, LB64_MUL(C.sig, X), LB64_MUL(C.sig, Y), LB64_MUL(C.sig, L), step2,
+                       D.step2_relax_j != 0,
+                       [&](double (&v)[9]) {
+#pragma unroll
+                           for (int i = 0; i < 9; ++i) v[i] = g[i];
+                       },
+                       fo, go);
+    } else {
+        Real dx, dy, lap;
+        // order: centre, E, W, N, S, NE, NW, SE, SW
+        stencils<Real>(c, nb[1], nb[2], nb[3], nb[4], nb[5], nb[7], nb[8], nb[6], dx, dy, lap);
+        const NodeParams<Real> prm = geo_params<Real>(D);
+        collide<Real, MRT>(prm, f, g, c, dx, dy, lap, step2, D.step2_relax_j != 0, fo, go);
+    }
+}
+
+// phi = sum of the pulled g
+template <typename Real>
+__device__ __forceinline__ Real geo_phi(const GeoConst<Real>& K, const Real (&g)[9])
+{
+    if constexpr (sizeof(Real) == 8)
+        return phi64(K.c, g);
+    else
+        return phi_sum<Real>(g);
+}
+
+// Halo position k of a tile, relative to its first node: the one-node ring
+// first (kRing1 positions), then the ring two and three nodes out (kRing3).
+template <int TY>
+struct GeoHalo {
+    static constexpr int kRing1 = 2 * (kGTX + 2) + 2 * TY;
+    static constexpr int kRing3 = 4 * kGPX + 4 * (TY + 2);
+    __device__ __forceinline__ static void at(int k, int& dx, int& dy)
+    {
+        constexpr int W = kGTX + 2;
+        if (k < 2 * W) {
+            dy = k < W ? -1 : TY;
+            dx = (k < W ? k : k - W) - 1;
+            return;
+        }
+        k -= 2 * W;
+        if (k < 2 * TY) {
+            dx = (k & 1) ? kGTX : -1;
+            dy = k >> 1;
+            return;
+        }
+        k -= 2 * TY;
+        if (k < 4 * kGPX) {
+            const int r = k / kGPX;
+            dy = r < 2 ? r - 3 : TY - 1 + r;
+            dx = k - r * kGPX - 3;
+            return;
+        }
+        k -= 4 * kGPX;
+        dy = (k >> 2) - 1;
+        dx = (k & 2) ? kGTX + 1 + (k & 1) : (k & 1) - 3;
+    }
+};
+
+// One time step of the tile at (x0, y0).  near: the tile holds a fluid node
+// with a solid neighbour.  Every thread of the CTA calls it (it holds CTA
+// barriers).
+template <typename Real, bool MRT, int TY, bool L2ONLY>
+__device__ __forceinline__ void geo_tile_step(const DomDesc& D, const GeoConst<Real>& K, int parity,
+                                              int x0, int y0, bool near, const GeoTables<TY>& t,
+                                              Real (&ph)[TY + 2 * kGH][kGPX])
+{
+    constexpr int N = kGTX * TY;
+    const int nx = D.nx, ny = D.ny;
+    const long long P = D.plane;
+    const Real* fs = static_cast<const Real*>(parity ? D.f[1] : D.f[0]);
+    const Real* gs = static_cast<const Real*>(parity ? D.g[1] : D.g[0]);
+    // positions relative to the tile's first node
+    auto cls = [&](int x, int y) -> int { return t.cl[y + kGC][x + kGC]; };
+    auto phi = [&](int x, int y) -> Real& { return ph[y + kGH][x + kGH]; };
+    auto off = [&](int x, int y) -> int { return t.rowo[y + kGC] + t.colx[x + kGC]; };
+    // the nine pulled values of a fluid or wall node; a solid source bounces
+    // back (the node's own reversed population), a wall node streams
+    auto pull = [&](const Real* src, int x, int y, Real (&v)[9]) {
+        const int own = off(x, y);
+#pragma unroll
+        for (int i = 0; i < 9; ++i) {
+            const int sx = x - gex(i), sy = y - gey(i);
+            const int c = i == 0 ? 0 : cls(sx, sy);
+            v[i] = c != 0 && c != kNodeWall ? geo_ld<L2ONLY>(src + gopp(i) * P + own)
+                                            : geo_ld<L2ONLY>(src + i * P + off(sx, sy));
+        }
+    };
+    const int tid = int(threadIdx.x), x = tid % kGTX, y = tid / kGTX;
+    const int cme = (x0 + x < nx && y0 + y < ny) ? cls(x, y) : 1;
+    const bool live = cme == 0 || cme == kNodeWall;
+    // 1. own f and g, and g of halo positions
+    Real f[9], g[9];
+    if (live) {
+        pull(gs, x, y, g);
+        pull(fs, x, y, f);
+    }
+    const int nh = GeoHalo<TY>::kRing1 + (near ? GeoHalo<TY>::kRing3 : 0);
+    for (int k = tid; k < nh; k += N) {
+        int hx, hy;
+        GeoHalo<TY>::at(k, hx, hy);
+        if (cls(hx, hy) == 0) {
+            Real gh[9];
+            pull(gs, hx, hy, gh);
+            phi(hx, hy) = geo_phi<Real>(K, gh);
+        }
+    }
+    // a short last tile's threads beyond the lattice take part in the phi array
+    // too: their columns and rows are the wrapped ones
+    Real c = Real(0);
+    if (live) {
+        c = geo_phi<Real>(K, g);
+        phi(x, y) = c;
+    } else if (cls(x, y) == 0) {
+        pull(gs, x, y, g);
+        phi(x, y) = geo_phi<Real>(K, g);
+    }
+    __syncthreads();
+    // 2. ghost values of the solid nodes on the tile and its one-node halo
+    if (near) {
+        constexpr int GX = kGTX + 2, GY = TY + 2;
+        for (int k = tid; k < GX * GY; k += N) {
+            const int sy = k / GX - 1, sx = k - (sy + 1) * GX - 1;
+            if (cls(sx, sy) == 0) continue;
+            Real v;
+            if (geo_ghost<Real>(D, sx, sy, y0 + sy, cls, phi, v)) phi(sx, sy) = v;
+        }
+        __syncthreads();
+    }
+    // 3. the tile's fluid and wall nodes
+    if (!live) return;
+    Real fo[9], go[9];
     if (cme == kNodeWall) {
         // node bounce-back: every population reversed, no collision
 #pragma unroll
@@ -199,134 +414,19 @@ __device__ __forceinline__ void geo_node_update(const DomDesc& D, int x, int y, 
             fo[i] = f[gopp(i)];
             go[i] = g[gopp(i)];
         }
-        return;
+    } else {
+        Real nb[9];
+        bool next_to_solid = false;
+#pragma unroll
+        for (int i = 1; i < 9; ++i) {
+            nb[i] = phi(x + gex(i), y + gey(i));
+            next_to_solid = next_to_solid || (near && cls(x + gex(i), y + gey(i)) != 0);
+        }
+        geo_collide<Real, MRT>(D, K, f, g, c, nb, D.step2 != 0 && next_to_solid, fo, go);
     }
-    const Real c = phi_sum<Real>(g);
-    // wetting ghost value of solid node (sx, sy): the mean over the axis (or,
-    // through a corner only, the diagonal) directions d towards fluid of
-    // phi(s + k d) - k h, k = D.wet_k
-    auto ghost = [&](int sx, int sy) -> Real {
-        const int k = cls_l(sx, sy);
-        const Real h = k == -1 ? (sizeof(Real) == 4 ? Real(D.fh_bot) : Real(D.h_bot))
-                     : k == -2 ? (sizeof(Real) == 4 ? Real(D.fh_top) : Real(D.h_top))
-                               : class_h<Real>(D, k);
-        Real sum = Real(0);
-        int n = 0;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int dx = j == 0 ? 1 : (j == 1 ? -1 : 0);
-            const int dy = j == 2 ? 1 : (j == 3 ? -1 : 0);
-            if (cls_l(sx + dx, sy + dy) == 0) {
-                sum += phi_l(sx + D.wet_k * dx, sy + D.wet_k * dy);
-                ++n;
-            }
-        }
-        if (n == 0) {
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const int dx = (j == 0 || j == 3) ? 1 : -1;
-                const int dy = (j == 0 || j == 2) ? 1 : -1;
-                if (cls_l(sx + dx, sy + dy) == 0) {
-                    sum += phi_l(sx + D.wet_k * dx, sy + D.wet_k * dy);
-                    ++n;
-                }
-            }
-        }
-        const Real mean = n == 1 ? sum : (n == 2 ? sum * Real(0.5) : (n == 3 ? div_const<3>(sum) : sum * Real(0.25)));
-        return mean - Real(D.wet_k) * h;
-    };
-    // phi at the eight neighbours; ghost values at solid ones
-    Real nb[9];
-    bool next_to_solid = false;
-#pragma unroll
-    for (int i = 1; i < 9; ++i) {
-        const int qx = x + gex(i), qy = y + gey(i);
-        const int cq = cls_l(qx, qy);
-        if (cq == kNodeWall) {
-            // one-sided wetting value from the first fluid row
-            next_to_solid = true;
-            nb[i] = qy == 0 ? phi_l(qx, 1) - (sizeof(Real) == 4 ? Real(D.fh_bot) : Real(D.h_bot))
-                            : phi_l(qx, ny - 2) - (sizeof(Real) == 4 ? Real(D.fh_top) : Real(D.h_top));
-        } else if (cq != 0) {
-            next_to_solid = true;
-            nb[i] = ghost(qx, qy);
-        } else {
-            nb[i] = phi_l(qx, qy);
-        }
-    }
-    Real dx, dy, lap;
-    // order: centre, E, W, N, S, NE, NW, SE, SW
-    stencils<Real>(c, nb[1], nb[2], nb[3], nb[4], nb[5], nb[7], nb[8], nb[6], dx, dy, lap);
-    const NodeParams<Real> prm = geo_params<Real>(D);
-    collide<Real, MRT>(prm, f, g, c, dx, dy, lap, D.step2 != 0 && next_to_solid,
-                       D.step2_relax_j != 0, fo, go);
-}
-
-// One time step of the tile at (x0, y0): phi of the tile and its halo into
-// ph, then the tile's fluid and wall nodes.  Every thread of the CTA calls it
-// (it holds CTA barriers); threads without a node of their own only help
-// with phi.
-template <typename Real, bool MRT, bool L2ONLY>
-__device__ __forceinline__ void geo_tile_step(const DomDesc& D, int parity, int x0, int y0,
-                                              const GeoTables& t, Real (&ph)[kGPY][kGPX])
-{
-    const int nx = D.nx, ny = D.ny;
-    const Real* fs = static_cast<const Real*>(parity ? D.f[1] : D.f[0]);
-    const Real* gs = static_cast<const Real*>(parity ? D.g[1] : D.g[0]);
-    // lattice coordinates (unwrapped, within the halos) to shared memory
-    auto cls_l = [&](int x, int y) -> int { return t.cl[y - y0 + kGC][x - x0 + kGC]; };
-    // a population pulled from a solid node bounces back (wall nodes stream)
-    auto solid_l = [&](int x, int y) {
-        const int c = cls_l(x, y);
-        return c != 0 && c != kNodeWall;
-    };
-    auto phi_l = [&](int x, int y) -> Real { return ph[y - y0 + kGH][x - x0 + kGH]; };
-    auto off_l = [&](int x, int y) -> int { return t.rowo[y - y0 + kGC] + t.colx[x - x0 + kGC]; };
-    // the nine pulled values of fluid node (x, y) from population set src;
-    // a solid source bounces back (the node's own reversed population)
-    const long long P = D.plane;
-    auto pull = [&](const Real* src, int x, int y, Real (&v)[9]) {
-        const int own = off_l(x, y);
-#pragma unroll
-        for (int i = 0; i < 9; ++i) {
-            const int sx = x - gex(i), sy = y - gey(i);
-            if (i != 0 && solid_l(sx, sy))
-                v[i] = geo_ld<L2ONLY>(src + gopp(i) * P + own);
-            else
-                v[i] = geo_ld<L2ONLY>(src + i * P + off_l(sx, sy));
-        }
-    };
-    const int x = x0 + int(threadIdx.x) % kGTX, y = y0 + int(threadIdx.x) / kGTX;
-    const int cme = (x < nx && y < ny) ? cls_l(x, y) : 1;
-    const bool live = cme == 0 || cme == kNodeWall;
-    Real f[9];
-    if (live) pull(fs, x, y, f);
-    // 2. phi of the tile and its halo (solid nodes: unused); a fixed trip
-    // count lets the loads of all of a thread's positions be in flight at once
-    constexpr int kPhiIters = (kGPX * kGPY + kGTX * kGTY - 1) / (kGTX * kGTY);
-#pragma unroll
-    for (int it = 0; it < kPhiIters; ++it) {
-        const int k = int(threadIdx.x) + it * kGTX * kGTY;
-        if (k >= kGPX * kGPY) break;
-        const int py = k / kGPX, px = k - py * kGPX;
-        const int hx = x0 - kGH + px, hy = y0 - kGH + py;
-        Real v = Real(0);
-        if (cls_l(hx, hy) == 0) {
-            Real g[9];
-            pull(gs, hx, hy, g);
-            v = phi_sum<Real>(g);
-        }
-        ph[py][px] = v;
-    }
-    __syncthreads();
-    // 3. the tile's fluid and wall nodes
-    if (!live) return;
     Real* fd = static_cast<Real*>(parity ? D.f[0] : D.f[1]);
     Real* gd = static_cast<Real*>(parity ? D.g[0] : D.g[1]);
-    const int o = off_l(x, y);
-    Real g[9], fo[9], go[9];
-    pull(gs, x, y, g);
-    geo_node_update<Real, MRT>(D, x, y, cme, f, g, cls_l, phi_l, fo, go);
+    const int o = off(x, y);
 #pragma unroll
     for (int i = 0; i < 9; ++i) {
         fd[i * P + o] = fo[i];
@@ -346,16 +446,22 @@ __device__ __forceinline__ void pdl_allow_next()
 }
 __device__ __forceinline__ void pdl_wait_prev() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
-template <typename Real, bool MRT>
-__global__ void __launch_bounds__(kGTX * kGTY) geo_step_kernel(DomDesc D, int parity)
+// tiles: the domain's list (make_geo_tiles).
+template <typename Real, bool MRT, int TY>
+__global__ void __launch_bounds__(kGTX * TY) geo_step_kernel(DomDesc D, int parity,
+                                                             const int* __restrict__ tiles)
 {
-    __shared__ GeoTables t;
-    __shared__ Real ph[kGPY][kGPX];
-    const int x0 = blockIdx.x * kGTX, y0 = blockIdx.y * kGTY;
+    __shared__ GeoTables<TY> t;
+    __shared__ Real ph[TY + 2 * kGH][kGPX];
+    __shared__ GeoConst<Real> K;
     pdl_allow_next();
-    geo_tile_setup(D, x0, y0, t);
+    const int e = tiles[blockIdx.x], ntx = (D.nx + kGTX - 1) / kGTX;
+    const int q = e & kGeoTileIndex;
+    const int x0 = q % ntx * kGTX, y0 = q / ntx * TY;
+    K.load(D);
+    geo_tile_setup<TY>(D, x0, y0, t);
     pdl_wait_prev();
-    geo_tile_step<Real, MRT, false>(D, parity, x0, y0, t, ph);
+    geo_tile_step<Real, MRT, TY, false>(D, K, parity, x0, y0, e < 0, t, ph);
 }
 
 // Two steps per launch (temporal blocking; the state stays in L2, so a step
@@ -376,12 +482,48 @@ constexpr int kFCX = kGTX + 2 * kFC, kFCY = kGTY + 2 * kFC;
 constexpr int kFPX = kGTX + 2 * kFP, kFPY = kGTY + 2 * kFP;
 constexpr int kFAX = kGTX + 2 * kFH, kFAY = kGTY + 2 * kFH;
 
+
+// The step of one fluid or wall node (x, y) of class cme from its pulled
+// populations f, g: cls_l(x, y) reads the class map and phi_l(x, y) phi of
+// the same state around the node (lattice coordinates; ghost values at solid
+// neighbours are formed on the way and reach three nodes away).
+template <typename Real, bool MRT, class ClsF, class PhiF>
+__device__ __forceinline__ void geo_node_update(const DomDesc& D, const GeoConst<Real>& K, int x,
+                                                int y, int cme, const Real (&f)[9],
+                                                const Real (&g)[9], ClsF cls_l, PhiF phi_l,
+                                                Real (&fo)[9], Real (&go)[9])
+{
+    if (cme == kNodeWall) {
+#pragma unroll
+        for (int i = 0; i < 9; ++i) {
+            fo[i] = f[gopp(i)];
+            go[i] = g[gopp(i)];
+        }
+        return;
+    }
+    Real nb[9];
+    bool next_to_solid = false;
+#pragma unroll
+    for (int i = 1; i < 9; ++i) {
+        const int qx = x + gex(i), qy = y + gey(i);
+        if (cls_l(qx, qy) != 0) {
+            next_to_solid = true;
+            geo_ghost<Real>(D, qx, qy, qy, cls_l, phi_l, nb[i]);
+        } else {
+            nb[i] = phi_l(qx, qy);
+        }
+    }
+    geo_collide<Real, MRT>(D, K, f, g, geo_phi<Real>(K, g), nb, D.step2 != 0 && next_to_solid, fo,
+                           go);
+}
+
 template <typename Real>
 struct GeoFused {
     Real fa[9][kFAY][kFAX];  // step-t output on the tile and its kFH halo
     Real ga[9][kFAY][kFAX];
     Real ph0[kFPY][kFPX];    // phi of the state at t
-    Real ph1[kGPY][kGPX];    // phi of the state at t + 1
+    Real ph1[kGTY + 2 * kGH][kGPX];  // phi of the state at t + 1
+    GeoConst<Real> K;
     int colx[kFCX];
     int rowo[kFCY];
     int rowc[kFCY];
@@ -389,13 +531,15 @@ struct GeoFused {
 };
 
 template <typename Real, bool MRT>
-__global__ void __launch_bounds__(kGTX * kGTY) geo_step2_kernel(DomDesc D, int parity)
+__global__ void __launch_bounds__(kGTX * kGTY, sizeof(Real) == 4 ? 4 : 2)
+    geo_step2_kernel(DomDesc D, int parity)
 {
     extern __shared__ __align__(16) unsigned char geo_smem[];
     GeoFused<Real>& S = *reinterpret_cast<GeoFused<Real>*>(geo_smem);
     const int x0 = blockIdx.x * kGTX, y0 = blockIdx.y * kGTY;
     const int nx = D.nx, ny = D.ny;
     const int tid = int(threadIdx.x), nthr = int(blockDim.x);
+    S.K.load(D);
     // 0. wrapped halo coordinates and the class map on the tile + kFC
     for (int k = tid; k < kFCX + kFCY; k += nthr) {
         if (k < kFCX)
@@ -461,7 +605,7 @@ __global__ void __launch_bounds__(kGTX * kGTY) geo_step2_kernel(DomDesc D, int p
         if (cls_l(x, y) == 0) {
             Real g[9];
             pull_g(gs, x, y, g);
-            v = phi_sum<Real>(g);
+            v = geo_phi<Real>(S.K, g);
         }
         S.ph0[py][px] = v;
     }
@@ -479,7 +623,7 @@ __global__ void __launch_bounds__(kGTX * kGTY) geo_step2_kernel(DomDesc D, int p
         Real f[9], g[9], fo[9], go[9];
         pull_g(fs, x, y, f);
         pull_g(gs, x, y, g);
-        geo_node_update<Real, MRT>(D, x, y, cme, f, g, cls_l, phi0_l, fo, go);
+        geo_node_update<Real, MRT>(D, S.K, x, y, cme, f, g, cls_l, phi0_l, fo, go);
 #pragma unroll
         for (int i = 0; i < 9; ++i) {
             S.fa[i][ay][ax] = fo[i];
@@ -489,16 +633,16 @@ __global__ void __launch_bounds__(kGTX * kGTY) geo_step2_kernel(DomDesc D, int p
     __syncthreads();
     // 3. phi of the state at t + 1 on the tile + kGH
 #pragma unroll
-    for (int it = 0; it < (kGPX * kGPY + kT - 1) / kT; ++it) {
+    for (int it = 0; it < (kGPX * (kGTY + 2 * kGH) + kT - 1) / kT; ++it) {
         const int k = tid + it * kT;
-        if (k >= kGPX * kGPY) break;
+        if (k >= kGPX * (kGTY + 2 * kGH)) break;
         const int py = k / kGPX, px = k - py * kGPX;
         const int x = x0 - kGH + px, y = y0 - kGH + py;
         Real v = Real(0);
         if (cls_l(x, y) == 0) {
             Real g[9];
             pull_s(S.ga, x, y, g);
-            v = phi_sum<Real>(g);
+            v = geo_phi<Real>(S.K, g);
         }
         S.ph1[py][px] = v;
     }
@@ -512,7 +656,7 @@ __global__ void __launch_bounds__(kGTX * kGTY) geo_step2_kernel(DomDesc D, int p
     Real f[9], g[9], fo[9], go[9];
     pull_s(S.fa, x, y, f);
     pull_s(S.ga, x, y, g);
-    geo_node_update<Real, MRT>(D, x, y, cme, f, g, cls_l, phi1_l, fo, go);
+    geo_node_update<Real, MRT>(D, S.K, x, y, cme, f, g, cls_l, phi1_l, fo, go);
     Real* fd = static_cast<Real*>(parity ? D.f[0] : D.f[1]);
     Real* gd = static_cast<Real*>(parity ? D.g[0] : D.g[1]);
     const int o = off_l(x, y);
@@ -540,14 +684,16 @@ template <typename Real, bool MRT>
 __global__ void __launch_bounds__(kGTX * kGTY, sizeof(Real) == 4 ? 4 : 2)
     geo_persist_kernel(DomDesc D, int parity0, int flip, int n_steps, int* flags, int* done)
 {
-    __shared__ GeoTables t;
-    __shared__ Real ph[kGPY][kGPX];
+    __shared__ GeoTables<kGTY> t;
+    __shared__ Real ph[kGTY + 2 * kGH][kGPX];
+    __shared__ GeoConst<Real> K;
     __shared__ int nbr[16];
     __shared__ int n_nbr, stop, last_cta;
     const int ntx = int(gridDim.x), nty = int(gridDim.y);
     const int tx = int(blockIdx.x), ty = int(blockIdx.y), me = ty * ntx + tx;
     const int x0 = tx * kGTX, y0 = ty * kGTY;
-    geo_tile_setup(D, x0, y0, t);
+    K.load(D);
+    geo_tile_setup<kGTY>(D, x0, y0, t);
     if (threadIdx.x == 0) {
         // the tiles under the halo (the wrapped columns and rows of the
         // tables; a short last tile can bring a second tile within reach)
@@ -558,7 +704,7 @@ __global__ void __launch_bounds__(kGTX * kGTY, sizeof(Real) == 4 ? 4 : 2)
             for (int j = 0; j < ncx; ++j) seen = seen || cx[j] == q;
             if (!seen) cx[ncx++] = q;
         }
-        for (int k = 0; k < kGCY; ++k) {
+        for (int k = 0; k < kGTY + 2 * kGC; ++k) {
             const int y = y0 - kGC + k;
             if (D.walls && (y < 0 || y >= D.ny)) continue;  // wall rows: no data
             const int q = t.rowc[k] / D.nx / kGTY;
@@ -582,7 +728,7 @@ __global__ void __launch_bounds__(kGTX * kGTY, sizeof(Real) == 4 ? 4 : 2)
             __syncthreads();
             if (stop) break;
         }
-        geo_tile_step<Real, MRT, true>(D, parity0 ^ (s & flip), x0, y0, t, ph);
+        geo_tile_step<Real, MRT, kGTY, true>(D, K, parity0 ^ (s & flip), x0, y0, true, t, ph);
         __syncthreads();
         if (threadIdx.x == 0) {
             __threadfence();
@@ -699,20 +845,28 @@ __global__ void geo_solid_rest_kernel(DomDesc D, int b)
 
 dim3 geo_grid(const DomDesc& d) { return dim3((d.nx + kGeoBlock - 1) / kGeoBlock, d.ny); }
 
-template <typename Real, bool MRT>
-cudaError_t geo_step_t(const DomDesc& d, int parity, cudaStream_t s)
+// A dependent launch, except for FP64 domains of few tiles: the next grid's
+// CTAs are placed while this one's still run, some of them two to an SM, and
+// there the FP64 pipe of the fullest SM is the bound (401 x 77 channel, about
+// one tile per SM: 10.2 us a step without, 20.9 with; 2000 x 200, twelve
+// tiles per SM: 58.0 without, 56.2 with; FP32 1000 x 120: 6.4 without, 5.3
+// with).
+constexpr int kFewTiles = 1024;
+
+template <typename Real, bool MRT, int TY>
+cudaError_t geo_step_t(const DomDesc& d, int parity, const int* tiles, int n_tiles, cudaStream_t s)
 {
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((d.nx + kGTX - 1) / kGTX, (d.ny + kGTY - 1) / kGTY);
-    cfg.blockDim = dim3(kGTX * kGTY);
+    cfg.gridDim = dim3(n_tiles);
+    cfg.blockDim = dim3(kGTX * TY);
     cfg.dynamicSmemBytes = 0;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[0].val.programmaticStreamSerializationAllowed = sizeof(Real) == 4 || n_tiles >= kFewTiles;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, geo_step_kernel<Real, MRT>, d, parity);
+    return cudaLaunchKernelEx(&cfg, geo_step_kernel<Real, MRT, TY>, d, parity, tiles);
 }
 
 template <typename Real, bool MRT>
@@ -799,12 +953,61 @@ int prepare_geo_step2()
     return 0;
 }
 
-int launch_geo_step(int precision, int coll, const DomDesc& d, int parity, void* stream)
+int launch_geo_step(int precision, int coll, const DomDesc& d, int parity, int tile_rows,
+                    const int* tiles, int n_tiles, void* stream)
 {
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    if (precision == 0)
-        return int(coll ? geo_step_t<float, true>(d, parity, s) : geo_step_t<float, false>(d, parity, s));
-    return int(coll ? geo_step_t<double, true>(d, parity, s) : geo_step_t<double, false>(d, parity, s));
+    if (precision != 0)
+        return int(coll ? geo_step_t<double, true, 4>(d, parity, tiles, n_tiles, s)
+                        : geo_step_t<double, false, 4>(d, parity, tiles, n_tiles, s));
+    if (tile_rows == 8)
+        return int(coll ? geo_step_t<float, true, 8>(d, parity, tiles, n_tiles, s)
+                        : geo_step_t<float, false, 8>(d, parity, tiles, n_tiles, s));
+    return int(coll ? geo_step_t<float, true, 4>(d, parity, tiles, n_tiles, s)
+                    : geo_step_t<float, false, 4>(d, parity, tiles, n_tiles, s));
+}
+
+size_t geo_tile_capacity(int nx, int ny)
+{
+    return size_t((nx + kGTX - 1) / kGTX) * size_t((ny + 3) / 4);
+}
+
+static std::vector<int> live_tiles(int ty, const unsigned char* cls, int nx, int ny, int walls)
+{
+    const int ntx = (nx + kGTX - 1) / kGTX, nty = (ny + ty - 1) / ty;
+    std::vector<int> near, plain;
+    auto solid = [&](int x, int y) {
+        if (walls && (y < 0 || y >= ny)) return true;
+        return cls[size_t((y + ny) % ny) * nx + (x + nx) % nx] != 0;
+    };
+    for (int q = 0; q < ntx * nty; ++q) {
+        const int x0 = q % ntx * kGTX, y0 = q / ntx * ty;
+        bool live = false, touches = false;
+        for (int y = y0; y < std::min(y0 + ty, ny); ++y)
+            for (int x = x0; x < std::min(x0 + kGTX, nx); ++x) {
+                const int c = cls[size_t(y) * nx + x];
+                live = live || c == 0 || c == kNodeWall;
+                if (c != 0 || touches) continue;
+                for (int dy = -1; dy <= 1; ++dy)
+                    for (int dx = -1; dx <= 1; ++dx) touches = touches || solid(x + dx, y + dy);
+            }
+        if (live) (touches ? near : plain).push_back(touches ? q | ~kGeoTileIndex : q);
+    }
+    near.insert(near.end(), plain.begin(), plain.end());
+    return near;
+}
+
+GeoTiles make_geo_tiles(int precision, int sm_count, const unsigned char* cls, int nx, int ny,
+                        int walls)
+{
+    GeoTiles t;
+    t.rows = 8;
+    if (precision == 0) t.list = live_tiles(8, cls, nx, ny, walls);
+    if (precision != 0 || t.list.size() > 3 * size_t(sm_count)) {
+        t.rows = 4;
+        t.list = live_tiles(4, cls, nx, ny, walls);
+    }
+    return t;
 }
 
 int launch_geo_init_eq(int precision, const DomDesc& d, const double* phi0, int parity, void* stream)

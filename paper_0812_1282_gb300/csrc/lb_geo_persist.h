@@ -1,9 +1,30 @@
-// Host entry points of the multi-step obstacle steps (lb_geo.cu).
+// Host entry points of the obstacle steps' tile lists and multi-step forms
+// (lb_geo.cu).
 #pragma once
+
+#include <vector>
 
 #include "lb_internal.h"
 
 namespace lbfe {
+
+// Tiles of the per-step form, 32 columns x `rows`: those with a fluid or wall
+// node, the ones whose fluid touches a solid node first and marked by their
+// sign bit (they take longer).  FP32 takes 8 rows while all tiles are
+// resident at once (three to an SM), else 4, of which more fit (us per step:
+// 1000 x 120 channel, 255 tiles of 8 rows, 5.3 with 8 and 6.2 with 4; 2000 x
+// 200, 950 tiles, 13.4 and 10.9).  FP64 takes 4: the FP64 pipe of each SM is
+// the bound and smaller tiles share the work out more evenly (401 x 77: 10.2
+// with 4, 13.9 with 8, 12.6 with 2).  geo_tile_capacity: the most entries a
+// list can have.
+constexpr int kGeoTileIndex = 0x7fffffff;
+struct GeoTiles {
+    int rows;
+    std::vector<int> list;
+};
+GeoTiles make_geo_tiles(int precision, int sm_count, const unsigned char* cls, int nx, int ny,
+                        int walls);
+size_t geo_tile_capacity(int nx, int ny);
 
 // Persistent multi-step obstacle step (a cooperative launch of one CTA per
 // tile for n_steps steps, step s reading buffer parity0 ^ (s & flip));
