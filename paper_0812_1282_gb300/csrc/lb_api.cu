@@ -18,6 +18,7 @@
 #include "lb_geo_persist.h"
 #include "lb_node.cuh"
 #include "lb_node64.cuh"
+#include "lb_small.h"
 
 using lbfe::DomDesc;
 using lbfe::StatsOut;
@@ -213,6 +214,9 @@ struct lb_handle {
     cudaEvent_t fork_ev = nullptr;
     cudaEvent_t join_ev[LB_MAX_SCHED_CLASSES - 1] = {nullptr};
     int n_items = 0;
+    // single domain without obstacles: rows per tile of the small-lattice step
+    // (0: the staged one, whose shape `sched` holds either way)
+    int small_rows = 0;
     // persistent schedules: CTAs of each class's launch
     int pgrid[LB_MAX_SCHED_CLASSES] = {0};
     // single domain: the start order of its row bands (see band_multiplier)
@@ -616,6 +620,50 @@ lb_schedule default_schedule(const lb_handle* h)
     return s;
 }
 
+// Rows per tile of the small-lattice step (lb_small.cu) where a single domain
+// should take it, 0 where the staged step is the faster one.  It is the
+// faster one while the lattice is bound by latency, in FP64 also while it is
+// bound by the FP64 pipe and the tiles still fit the SMs evenly (us per step,
+// staged and small: FP32 28 x 15 4.0 and 2.5, 200 x 100 4.3 and 2.9, 1000 x 500
+// 15.4 and 13.8, 2000 x 350 20.7 and 20.0, but 900^2 24.4 and 27.4; compact
+// 28 x 15 4.5 and 3.4, 200 x 100 4.8 and 3.3, 512 x 256 7.2 and 5.9, but 2000 x
+// 100 7.7 and 8.1; FP64 28 x 15 8.3 and 6.4, 200 x 100 11 and 7.4, 1000 x 500 115
+// and 110, 1200^2 313 and 300, but 2048^2 831 and 850).
+//  - FP32: 4 rows (3 to 7 are within 5 %);
+//  - compact, whose tiles expand a two-node halo: the fewest rows from 4 on
+//    with which every tile has an SM to itself, else 7;
+//  - FP64: a warp's operations take the pipe of its scheduler four times as
+//    long as the SM's, so up to four rows per SM cost the same and beyond that
+//    the SM with the most rows is the bound (200 x 100, us per step with 3, 4,
+//    5, 6, 7 rows: 8.2, 9.9, 7.4, 8.1, 9.0).
+int small_rows(const lb_handle* h)
+{
+    if (h->n_dom != 1) return 0;
+    const DomDesc& D = h->descs[0];
+    const bool fp64 = h->precision == LB_FP64;
+    const long long nodes = (long long)D.nx * D.ny;
+    if (nodes > (fp64 ? 2000000 : (D.compact ? 120000 : 700000))) return 0;
+    auto tiles = [&](int rows) { return (long long)((D.nx + 31) / 32) * ((D.ny + rows - 1) / rows); };
+    if (D.compact) {
+        for (int r = 4; r < 7; ++r)
+            if (tiles(r) <= h->sm_count) return r;
+        return 7;
+    }
+    if (!fp64) return 4;
+    int best = 3;
+    double best_cost = 1e300;
+    for (int r = 3; r <= 7; ++r) {
+        // rows on the fullest SM; a tile's halo costs about a quarter row
+        const long long per_sm = (tiles(r) + h->sm_count - 1) / h->sm_count;
+        const double cost = std::max(double(per_sm) * (r + 0.25), 4.25);
+        if (cost < best_cost) {
+            best_cost = cost;
+            best = r;
+        }
+    }
+    return best;
+}
+
 // Grid of class c's launch: a persistent grid, or one CTA per work item.
 int class_grid(const lb_handle* h, int c)
 {
@@ -748,7 +796,12 @@ int enqueue_geo(lb_handle* h, int parity, cudaStream_t s)
 int enqueue_step(lb_handle* h, int parity, cudaStream_t s)
 {
     if (h->n_dom == 1) {
-        if (h->descs[0].cls == nullptr) {
+        if (h->descs[0].cls == nullptr && h->small_rows > 0) {
+            const int e = lbfe::launch_small_step(h->precision, h->coll, h->descs[0], parity,
+                                                  h->small_rows, s);
+            if (e != 0)
+                return fail(LB_ERR_CUDA, "step launch failed: %s", cudaGetErrorString(cudaError_t(e)));
+        } else if (h->descs[0].cls == nullptr) {
             const int e = lbfe::launch_step(h->precision, h->coll, h->descs[0], h->d_descs(),
                                             nullptr, 0, 1, parity, h->block_x(), h->rows(),
                                             h->band_mul, 0, h->d_sched(0), false, s);
@@ -1120,6 +1173,7 @@ int make_handle(const lb_params* per_dom, const int* nx, const int* ny, int n_do
         (e = cudaStreamSynchronize(h->stream)) != cudaSuccess)
         return bail(fail(LB_ERR_CUDA, "device init failed: %s", cudaGetErrorString(e)));
     h->sched = default_schedule(h);
+    h->small_rows = small_rows(h);
     const int rc = build_items(h);
     if (rc != LB_OK) return bail(rc);
     *out = h;
@@ -1929,6 +1983,7 @@ int lb_set_schedule(lb_handle* h, const lb_schedule* sc)
     }
     v.max_nx[v.n_class - 1] = 0;
     h->sched = v;
+    h->small_rows = 0;  // an explicit shape is the staged step's
     return build_items(h);
 }
 
@@ -2050,6 +2105,7 @@ int lb_autotune(lb_handle* h, int reps, int* block_x, int* rows, double* best_ms
     // with obstacles chooses between per-step and persistent launches
     const bool plain = h->n_dom == 1 ? h->descs[0].cls == nullptr : h->n_items > 0;
     std::vector<lb_schedule> cands;
+    bool small = false;  // candidate 0 is the small-lattice step
     if (!plain) {
         cands.push_back(h->sched);
         if (h->n_dom == 1) {
@@ -2073,14 +2129,14 @@ int lb_autotune(lb_handle* h, int reps, int* block_x, int* rows, double* best_ms
             h->descs[0].compact ? std::vector<int>{32, 64, 96, 128, 160, 192, 224, 256, 288}
                                 : std::vector<int>{64, 128, 256};
         const int rws[] = {4, 8, 16, 32, 64, 128};
-        {
-            const lb_schedule d = default_schedule(h);
-            lb_schedule s = h->sched;
-            s.n_class = 1;
-            s.block_x[0] = d.block_x[0];
-            s.rows[0] = d.rows[0];
-            cands.push_back(s);
-        }
+        // the shape by size, and the small-lattice step where that is the rule
+        lb_schedule def = h->sched;
+        def.n_class = 1;
+        def.block_x[0] = default_schedule(h).block_x[0];
+        def.rows[0] = default_schedule(h).rows[0];
+        small = small_rows(h) > 0;
+        if (small) cands.push_back(def);
+        cands.push_back(def);
         for (int bx : bxs)
             for (int r : rws) {
                 if (r > max_ny && r != rws[0]) continue;
@@ -2095,13 +2151,18 @@ int lb_autotune(lb_handle* h, int reps, int* block_x, int* rows, double* best_ms
     LB_CUDA(cudaEventCreate(&e0));
     LB_CUDA(cudaEventCreate(&e1));
     const lb_schedule old = h->sched;
+    const int old_small = h->small_rows;
     double best = 1e300;
     lb_schedule chosen = old;
-    int rc = LB_OK;
-    // one timing of a candidate (ms per step); negative on failure
-    auto time_candidate = [&](const lb_schedule& c, int len, int r) -> double {
-        if ((rc = lb_set_schedule(h, &c)) != LB_OK) return -1.0;
-        if (h->n_dom > 1 || !plain) return time_graph_steps(h, len, r, e0, e1);
+    int chosen_small = old_small, rc = LB_OK;
+    // single launches of a small lattice would time the host's launch rate
+    const bool graphs =
+        h->n_dom > 1 || !plain || (long long)h->descs[0].nx * h->descs[0].ny <= 200000;
+    // one timing of candidate k (ms per step); negative on failure
+    auto time_candidate = [&](size_t k, int len, int r) -> double {
+        if ((rc = lb_set_schedule(h, &cands[k])) != LB_OK) return -1.0;
+        if (small && k == 0) h->small_rows = small_rows(h);
+        if (graphs) return time_graph_steps(h, len, r, e0, e1);
         // warm-up, then time `r` launches that read the current buffer and
         // write the idle one (the state itself does not advance)
         if ((rc = enqueue_step(h, h->parity, h->stream)) != LB_OK) return -1.0;
@@ -2115,23 +2176,23 @@ int lb_autotune(lb_handle* h, int reps, int* block_x, int* rows, double* best_ms
             return -1.0;
         return double(t) / r;
     };
-    // a batch: graphs of 16 steps, so that chains and tails show; then the
-    // fastest eight again over graphs of the length the steps run in (the
+    // a batch or a small lattice: graphs of 16 steps, so that chains and tails
+    // show; then the fastest eight again over graphs of the length the steps run in (the
     // leading candidates are within a few percent of each other)
     std::vector<std::pair<double, size_t>> scored;
     for (size_t k = 0; k < cands.size(); ++k) {
-        const double ms = time_candidate(cands[k], h->n_dom > 1 || !plain ? 16 : 4, reps);
+        const double ms = time_candidate(k, 16, reps);
         if (ms < 0.0) {
             if (rc == LB_OK) rc = LB_ERR_CUDA;
             break;
         }
         scored.emplace_back(ms, k);
     }
-    if (rc == LB_OK && (h->n_dom > 1 || !plain) && scored.size() > 1) {
+    if (rc == LB_OK && graphs && scored.size() > 1) {
         std::sort(scored.begin(), scored.end());
         const size_t top = std::min<size_t>(8, scored.size());
         for (size_t t = 0; t < top && rc == LB_OK; ++t) {
-            const double ms = time_candidate(cands[scored[t].second], kGraphBig, reps + 3);
+            const double ms = time_candidate(scored[t].second, kGraphBig, reps + 3);
             if (ms < 0.0) {
                 if (rc == LB_OK) rc = LB_ERR_CUDA;
                 break;
@@ -2144,11 +2205,13 @@ int lb_autotune(lb_handle* h, int reps, int* block_x, int* rows, double* best_ms
         if (sc.first < best) {
             best = sc.first;
             chosen = cands[sc.second];
+            chosen_small = small && sc.second == 0 ? small_rows(h) : 0;
         }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     if (rc == LB_OK) rc = sync_and_check(h);
     const int rc2 = lb_set_schedule(h, rc == LB_OK ? &chosen : &old);
+    h->small_rows = rc == LB_OK ? chosen_small : old_small;
     if (rc != LB_OK) return rc;
     if (rc2 != LB_OK) return rc2;
     if (block_x) *block_x = h->block_x();

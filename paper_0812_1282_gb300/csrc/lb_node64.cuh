@@ -7,9 +7,11 @@
 // DMUL or has a constant among its operands (measured on independent
 // chains, 1 to 16 warps).  So what counts is the number of operations, and
 // each is best a DFMA on registers:
-//  - the constants, among them 1 and -0, come from shared memory (Node64),
+//  - the constants, among them 1, -1 and -0, come from shared memory (Node64),
 //    where the compiler cannot fold them: add(x, y) is x * 1 + y and
-//    mul(x, y) is x * y + (-0), exactly the sum and the product;
+//    mul(x, y) is x * y + (-0), exactly the sum and the product (2048^2, MRT:
+//    832 us a step; 907 with plain sums and products; all constants held in
+//    registers for a whole tile, two CTAs per SM instead of three: 996);
 //  - opposite directions share their even part (E) and differ in the sign of
 //    the odd one, which MRT leaves at its equilibrium;
 //  - the two reciprocals 1/rho and 1/tau come from one of rho tau;
@@ -29,7 +31,7 @@ namespace lbfe {
 // Constants of one domain, computed once on the host (DomDesc::c64) and read
 // from shared memory.  s = sqrt(kappa).
 struct Node64 {
-    double one, nzero;         // 1, -0
+    double one, mone, nzero;   // 1, -1, -0
     double two, four, m4, m20;
     double q25, c3, c9, c12, m24;  // 1/4, 1/3, 1/9, 1/12, -1/24
     double sig;                // s / 12: scale of the phi values the stencils read
@@ -49,6 +51,7 @@ inline Node64 make_node64(double a, double kappa, double gamma, double omega_phi
     const double s = std::sqrt(kappa);
     Node64 c;
     c.one = 1.0;
+    c.mone = -1.0;
     c.nzero = -0.0;
     c.two = 2.0;
     c.four = 4.0;
@@ -84,7 +87,7 @@ __device__ __forceinline__ void load_node64(Node64& dst, const double* src, int 
 
 // x + y, x - y, x y and x y + z as one DFMA each (C: a Node64)
 #define LB64_ADD(x, y) __fma_rn((x), C.one, (y))
-#define LB64_SUB(x, y) __fma_rn((y), -C.one, (x))
+#define LB64_SUB(x, y) __fma_rn((y), C.mone, (x))
 #define LB64_MUL(x, y) __fma_rn((x), (y), C.nzero)
 
 // 1 / x: the hardware's seed (about 20 bits) and one third-order Newton-
@@ -96,6 +99,14 @@ __device__ __forceinline__ double rcp64(const Node64& C, double x)
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
     const double e = __fma_rn(-x, r, C.one);
     return __fma_rn(r, __fma_rn(e, e, e), r);
+}
+
+// m of a wall ghost row (lb_step64.cuh) from the m of the row it mirrors: phi
+// less wet_k h, 4 + 1 + 1 times, on the scaled phi.  (As one fused operation
+// it costs the row loop 8 %: the compiler keeps fewer constants.)
+__device__ __forceinline__ double ghost_m64(const Node64& C, double m, int wet_k, double h)
+{
+    return __dsub_rn(m, __dmul_rn(6.0 * wet_k * h, C.sig));
 }
 
 // phi = sum of the nine pulled g

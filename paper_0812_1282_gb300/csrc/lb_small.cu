@@ -1,0 +1,352 @@
+// Fused step of small lattices without obstacles: one launch per step, one
+// node per thread, plain loads.
+//
+// A lattice whose CTAs all fit the GPU at once is bound by latency: a
+// dependent launch costs 0.6 us, a global load and a store 0.5 us more, and
+// then every stage of a pipeline adds to the step.  The staged kernels
+// (lb_step.cuh and its FP64 and compact forms), made for bandwidth, put a
+// bulk copy (0.7 us more than plain loads), its barriers and the phi of three
+// rows in series in front of a row.  Here a CTA takes 32 columns x TY rows
+// and has all its loads in flight at once:
+//  - FP32 and FP64 full storage: a thread pulls f and g of its node and g of
+//    a position of the one-node halo (those with the highest index first);
+//    phi of both goes to shared memory, the CTA meets, and each thread
+//    collides its node from the 3 x 3 phi around it.
+//  - compact g storage: a thread loads the four compact values of positions
+//    on the tile and a two-node halo, expands them to g' in shared memory;
+//    then phi(t+1) of the tile and a one-node halo is formed from the g' that
+//    arrive there; then the nodes collide.
+// The arithmetic is that of the staged kernels, operation for operation, and
+// so are the stored populations and ghost columns, bit for bit.
+#include <cuda_runtime.h>
+
+#include "lb_internal.h"
+#include "lb_node.cuh"
+#include "lb_node64.cuh"
+#include "lb_node_x2.cuh"
+#include "lb_small.h"
+#include "lb_step.cuh"
+
+namespace lbfe {
+
+namespace {
+
+constexpr int kTX = 32;          // columns of a tile
+constexpr int kPW = kTX + 2;     // phi array: one halo column on each side
+constexpr int kEW = kTX + 4;     // g' array (compact): two
+
+// The tile of a CTA: node columns [x0, x0 + wc), rows [y0, y0 + hc).
+struct SmallTile {
+    int x0, y0, wc, hc;
+    __device__ __forceinline__ SmallTile(const DomDesc& D, int ty)
+        : x0(int(blockIdx.x) * kTX), y0(int(blockIdx.y) * ty), wc(min(kTX, D.nx - x0)),
+          hc(min(ty, D.ny - y0))
+    {
+    }
+};
+
+// The nine pulled values of the node at column x (-1 .. nx: ghost columns
+// included) and row y of population set src; a link through a wall gives the
+// node's own reversed population.
+template <typename Real>
+__device__ __forceinline__ void pull9(const Real* __restrict__ src, int P, int pitch, int ny,
+                                      bool walls, int x, int y, Real (&v)[9])
+{
+    const int o = y * pitch + x + kXOff;
+    const bool blo = walls && y == 0, bhi = walls && y == ny - 1;
+    const int om = y == 0 ? o + (ny - 1) * pitch : o - pitch;       // row below
+    const int op = y == ny - 1 ? o - (ny - 1) * pitch : o + pitch;  // row above
+    v[0] = src[o];
+    v[1] = src[P + o - 1];
+    v[2] = src[2 * P + o + 1];
+    v[3] = src[blo ? 4 * P + o : 3 * P + om];
+    v[4] = src[bhi ? 3 * P + o : 4 * P + op];
+    v[5] = src[blo ? 6 * P + o : 5 * P + om - 1];
+    v[6] = src[bhi ? 5 * P + o : 6 * P + op + 1];
+    v[7] = src[blo ? 8 * P + o : 7 * P + om + 1];
+    v[8] = src[bhi ? 7 * P + o : 8 * P + op - 1];
+}
+
+// Store one value of a plane at offset o and its periodic ghost copies:
+// logical columns 0, 1 also at nx, nx + 1 and nx - 2, nx - 1 also at -2, -1.
+template <typename Real>
+__device__ __forceinline__ void store_ghosts(Real* __restrict__ p, int o, int x, int nx, Real v)
+{
+    p[o] = v;
+    if (x < 2) p[o + nx] = v;
+    if (x >= nx - 2) p[o - nx] = v;
+}
+
+// Position k of the one-node halo of a tile, relative to its first node;
+// false if the tile or the lattice has none there.
+__device__ __forceinline__ bool halo_at(int k, const SmallTile& T, bool walls, int ny, int& hx,
+                                        int& hy)
+{
+    if (k < 2 * kPW) {
+        const bool low = k < kPW;
+        hx = (low ? k : k - kPW) - 1;
+        hy = low ? -1 : T.hc;
+        return hx <= T.wc && !(walls && (low ? T.y0 == 0 : T.y0 + T.hc == ny));
+    }
+    k -= 2 * kPW;
+    hx = (k & 1) ? T.wc : -1;
+    hy = k >> 1;
+    return hy < T.hc;
+}
+
+// Full storage.  blockDim.x = 32 TY (a multiple of a warp; every thread has
+// at most a node of its own); phi: (TY + 2) x 34 values of shared memory.
+template <typename Real, bool MRT>
+__global__ void __launch_bounds__(kSmallMaxThreads) small_step_kernel(DomDesc D, int parity)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    Real* ph = reinterpret_cast<Real*>(smem);
+    __shared__ Node64 C;  // FP64 only
+    const int TY = int(blockDim.x) / kTX;
+    const SmallTile T(D, TY);
+    const int nx = D.nx, ny = D.ny, pitch = D.pitch, P = int(D.plane);
+    const bool walls = D.walls != 0;
+    const Real* __restrict__ fs = static_cast<const Real*>(parity ? D.f[1] : D.f[0]);
+    const Real* __restrict__ gs = static_cast<const Real*>(parity ? D.g[1] : D.g[0]);
+    const int tid = int(threadIdx.x), tx = tid % kTX, ty = tid / kTX;
+    const int x = T.x0 + tx, y = T.y0 + ty;
+    const bool live = tx < T.wc && ty < T.hc;
+    // all loads of the thread's node and of its halo position
+    Real f[9], g[9], gh[9];
+    int hx = 0, hy = 0;
+    const int nh = 2 * kPW + 2 * TY;
+    int k = int(blockDim.x) - 1 - tid;
+    auto row = [&](int r) { return r < 0 ? r + ny : (r >= ny ? r - ny : r); };
+    bool halo = k < nh && halo_at(k, T, walls, ny, hx, hy);
+    if (live) pull9<Real>(gs, P, pitch, ny, walls, x, y, g);
+    if (halo) pull9<Real>(gs, P, pitch, ny, walls, T.x0 + hx, row(T.y0 + hy), gh);
+    if (live) pull9<Real>(fs, P, pitch, ny, walls, x, y, f);
+    if constexpr (sizeof(Real) == 8) {
+        if (tid < kNode64) reinterpret_cast<double*>(&C)[tid] = D.c64[tid];
+        __syncthreads();
+    }
+    // the stored value: phi, in FP64 scaled for the stencils (lb_step64.cuh)
+    auto put = [&](int cx, int cy, const Real (&v)[9], Real& phi) {
+        if constexpr (sizeof(Real) == 8) {
+            phi = phi64(C, v);
+            ph[(cy + 1) * kPW + cx + 1] = LB64_MUL(C.sig, phi);
+        } else {
+            phi = phi_sum<Real>(v);
+            ph[(cy + 1) * kPW + cx + 1] = phi;
+        }
+    };
+    Real c = Real(0), dump;
+    if (live) put(tx, ty, g, c);
+    for (;;) {
+        if (halo) put(hx, hy, gh, dump);
+        k += int(blockDim.x);
+        if (k >= nh) break;
+        halo = halo_at(k, T, walls, ny, hx, hy);
+        if (halo) pull9<Real>(gs, P, pitch, ny, walls, T.x0 + hx, row(T.y0 + hy), gh);
+    }
+    __syncthreads();
+    if (!live) return;
+    const bool blo = walls && y == 0, bhi = walls && y == ny - 1;
+    const bool s2 = D.step2 && (blo || bhi);
+    // the row of a ghost row's phi: row k - 1 (ny - k), see DomDesc::wet_k
+    const Real* r0 = ph + (ty + 1) * kPW + tx + 1;
+    const Real* rp = r0 + kPW;
+    const Real* rm = r0 - kPW;
+    Real fo[9], go[9];
+    if constexpr (sizeof(Real) == 8) {
+        struct Row {
+            double k, h, m;
+        };
+        auto row_of = [&](const double* r) {
+            Row v;
+            v.k = LB64_SUB(r[1], r[-1]);
+            v.h = LB64_ADD(r[1], r[-1]);
+            v.m = __fma_rn(C.four, r[0], v.h);
+            return v;
+        };
+        const Row cur = row_of(r0);
+        Row up = cur, dn = cur;
+        if (!bhi) up = row_of(rp);
+        if (!blo) dn = row_of(rm);
+        if (blo) {
+            const Row& v = D.wet_k == 2 ? up : cur;
+            dn.k = v.k;
+            dn.m = ghost_m64(C, v.m, D.wet_k, D.h_bot);
+        }
+        if (bhi) {
+            const Row& v = D.wet_k == 2 ? dn : cur;
+            up.k = v.k;
+            up.m = ghost_m64(C, v.m, D.wet_k, D.h_top);
+        }
+        const double X = __fma_rn(C.four, cur.k, LB64_ADD(up.k, dn.k));
+        const double Y = LB64_SUB(up.m, dn.m);
+        const double L = __fma_rn(C.m20, r0[0], __fma_rn(C.four, cur.h, LB64_ADD(up.m, dn.m)));
+        collide64<MRT>(C, f, c, X, Y, L, s2, D.step2_relax_j != 0,
+                       [&](double (&v)[9]) {
+#pragma unroll
+                           for (int i = 0; i < 9; ++i) v[i] = g[i];
+                       },
+                       fo, go);
+    } else {
+        const NodeParams<Real> prm = node_params<Real>(D);
+        Real dx, dy, lap, n[3], s[3];
+        const Real* gp = bhi ? r0 - (D.wet_k - 1) * kPW : rp;
+        const Real* gm = blo ? r0 + (D.wet_k - 1) * kPW : rm;
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            n[j] = gp[j - 1];
+            s[j] = gm[j - 1];
+        }
+        if (bhi) {
+            const Real h2 = Real(D.wet_k) * prm.h_top;
+#pragma unroll
+            for (int j = 0; j < 3; ++j) n[j] = n[j] - h2;
+        }
+        if (blo) {
+            const Real h2 = Real(D.wet_k) * prm.h_bot;
+#pragma unroll
+            for (int j = 0; j < 3; ++j) s[j] = s[j] - h2;
+        }
+        stencils<Real>(c, r0[1], r0[-1], n[1], s[1], n[2], n[0], s[2], s[0], dx, dy, lap);
+        collide<Real, MRT>(prm, f, g, c, dx, dy, lap, s2, D.step2_relax_j != 0, fo, go);
+    }
+    Real* __restrict__ fd = static_cast<Real*>(parity ? D.f[0] : D.f[1]);
+    Real* __restrict__ gd = static_cast<Real*>(parity ? D.g[0] : D.g[1]);
+    const int o = y * pitch + x + kXOff;
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+        store_ghosts(fd + i * P, o, x, nx, fo[i]);
+        store_ghosts(gd + i * P, o, x, nx, go[i]);
+    }
+}
+
+// Compact g storage.  Shared memory: nine values (g'_1..g'_8 and their sum)
+// and the phi word of (TY + 4) x 36 positions, then phi of (TY + 2) x 34.
+template <bool MRT>
+__global__ void __launch_bounds__(kSmallMaxThreads) small_compact_kernel(DomDesc D, int parity)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    const int TY = int(blockDim.x) / kTX;
+    const int ne = (TY + 4) * kEW;
+    float* E = reinterpret_cast<float*>(smem);  // E[i * ne + position], i = 0: the sum, 9: the word
+    float* ph = E + 10 * ne;
+    const SmallTile T(D, TY);
+    const int nx = D.nx, ny = D.ny, pitch = D.pitch, P = int(D.plane);
+    const bool walls = D.walls != 0;
+    const float* __restrict__ fs = static_cast<const float*>(parity ? D.f[1] : D.f[0]);
+    const float* __restrict__ cs = static_cast<const float*>(parity ? D.g[1] : D.g[0]);
+    const int tid = int(threadIdx.x), tx = tid % kTX, ty = tid / kTX;
+    const int x = T.x0 + tx, y = T.y0 + ty;
+    const bool live = tx < T.wc && ty < T.hc;
+    auto row = [&](int r) { return r < 0 ? r + ny : (r >= ny ? r - ny : r); };
+    auto inside = [&](int r) { return !walls || (r >= 0 && r < ny); };
+    const NodeParams<float> prm = node_params<float>(D);
+    float f[9];
+    if (live) pull9<float>(fs, P, pitch, ny, walls, x, y, f);
+    // 1. expand the compact values of the tile and two nodes around it
+    for (int k = tid; k < ne; k += int(blockDim.x)) {
+        const int cy = k / kEW, cx = k - cy * kEW;
+        const int r = T.y0 + cy - 2;
+        if (cx - 2 > T.wc + 1 || cy - 2 > T.hc + 1 || !inside(r)) continue;
+        const float* s = cs + row(r) * pitch + T.x0 + cx - 2 + kXOff;
+        const f2 word(s[0]), G(s[P]), ux(s[2 * P]), uy(s[3 * P]);
+        f2 ge[9];
+        g_equilibria2(g0_value2(word), G, ux, uy, ge);
+        E[k] = g_tail_sum2(ge).lane(0);
+#pragma unroll
+        for (int i = 1; i < 9; ++i) E[i * ne + k] = ge[i].lane(0);
+        E[9 * ne + k] = word.lane(0);
+    }
+    __syncthreads();
+    // 2. phi(t+1) = word + [(U + H) + D - sum] of the tile and one node around
+    //    it (lb_step_compact.cuh); the node's own word for its store
+    auto phi_at = [&](int cx, int cy, f2& word) -> f2 {
+        const int q = (cy + 2) * kEW + cx + 2, r = T.y0 + cy;
+        auto e = [&](int i, int dx, int dy) { return f2(E[i * ne + q + dy * kEW + dx]); };
+        const f2 u = walls && r == 0 ? (e(4, 0, 0) + e(6, 0, 0)) + e(8, 0, 0)
+                                     : (e(3, 0, -1) + e(5, -1, -1)) + e(7, 1, -1);
+        const f2 h = e(1, -1, 0) + e(2, 1, 0);
+        const f2 d = walls && r == ny - 1 ? (e(3, 0, 0) + e(5, 0, 0)) + e(7, 0, 0)
+                                          : (e(4, 0, 1) + e(6, 1, 1)) + e(8, -1, 1);
+        word = g0_advance2(e(9, 0, 0), ((u + h) + d) - e(0, 0, 0));
+        return g0_value2(word);
+    };
+    f2 word(0.f), c(0.f), dump(0.f);
+    if (live) {
+        c = phi_at(tx, ty, word);
+        ph[(ty + 1) * kPW + tx + 1] = c.lane(0);
+    }
+    for (int k = int(blockDim.x) - 1 - tid; k < 2 * kPW + 2 * TY; k += int(blockDim.x)) {
+        int hx, hy;
+        if (!halo_at(k, T, walls, ny, hx, hy)) continue;
+        // a periodic halo row is the row across the lattice's edge
+        ph[(hy + 1) * kPW + hx + 1] = phi_at(hx, hy, dump).lane(0);
+    }
+    __syncthreads();
+    // 3. collide
+    if (!live) return;
+    const bool blo = walls && y == 0, bhi = walls && y == ny - 1;
+    const float* r0 = ph + (ty + 1) * kPW + tx + 1;
+    const float* gp = bhi ? r0 - (D.wet_k - 1) * kPW : r0 + kPW;
+    const float* gm = blo ? r0 + (D.wet_k - 1) * kPW : r0 - kPW;
+    f2 n[3], s[3];
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+        n[j] = f2(gp[j - 1]);
+        s[j] = f2(gm[j - 1]);
+    }
+    if (bhi) {
+        const f2 h(float(D.wet_k) * prm.h_top);
+#pragma unroll
+        for (int j = 0; j < 3; ++j) n[j] = n[j] - h;
+    }
+    if (blo) {
+        const f2 h(float(D.wet_k) * prm.h_bot);
+#pragma unroll
+        for (int j = 0; j < 3; ++j) s[j] = s[j] - h;
+    }
+    f2 dx, dy, lap, fi[9], fo[9], ux, uy;
+#pragma unroll
+    for (int i = 0; i < 9; ++i) fi[i] = f2(f[i]);
+    stencils2(c, f2(r0[1]), f2(r0[-1]), n[1], s[1], n[2], n[0], s[2], s[0], dx, dy, lap);
+    collide_f2<MRT>(prm, fi, c, dx, dy, lap, D.step2 && (blo || bhi), D.step2_relax_j != 0, fo, ux,
+                    uy);
+    const f2 gmu = gamma_mu2(prm, c, lap);
+    float* __restrict__ fd = static_cast<float*>(parity ? D.f[0] : D.f[1]);
+    float* __restrict__ cd = static_cast<float*>(parity ? D.g[0] : D.g[1]);
+    const int o = y * pitch + x + kXOff;
+#pragma unroll
+    for (int i = 0; i < 9; ++i) store_ghosts(fd + i * P, o, x, nx, fo[i].lane(0));
+    store_ghosts(cd, o, x, nx, word.lane(0));
+    store_ghosts(cd + P, o, x, nx, gmu.lane(0));
+    store_ghosts(cd + 2 * P, o, x, nx, ux.lane(0));
+    store_ghosts(cd + 3 * P, o, x, nx, uy.lane(0));
+}
+
+template <bool MRT>
+cudaError_t launch_t(int precision, const DomDesc& d, int parity, int rows, cudaStream_t s)
+{
+    const dim3 grid((d.nx + kTX - 1) / kTX, (d.ny + rows - 1) / rows);
+    const int threads = kTX * rows;
+    const size_t phi = size_t(rows + 2) * kPW;
+    if (precision != 0)
+        small_step_kernel<double, MRT><<<grid, threads, phi * 8, s>>>(d, parity);
+    else if (d.compact)
+        small_compact_kernel<MRT>
+            <<<grid, threads, (size_t(rows + 4) * kEW * 10 + phi) * 4, s>>>(d, parity);
+    else
+        small_step_kernel<float, MRT><<<grid, threads, phi * 4, s>>>(d, parity);
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+int launch_small_step(int precision, int coll, const DomDesc& d, int parity, int rows, void* stream)
+{
+    if (rows < 1 || rows > kSmallMaxThreads / kTX) return int(cudaErrorInvalidValue);
+    cudaStream_t s = static_cast<cudaStream_t>(stream);
+    return int(coll ? launch_t<true>(precision, d, parity, rows, s)
+                    : launch_t<false>(precision, d, parity, rows, s));
+}
+
+}  // namespace lbfe

@@ -148,12 +148,12 @@ __device__ __forceinline__ void consume_tile64(const DomDesc& D, const Node64& C
             if (blo) {
                 const bool mirror = D.wet_k == 2;
                 km = mirror ? nxt.k : cur.k;
-                mm = (mirror ? nxt.m : cur.m) - 6.0 * D.wet_k * D.h_bot * C.sig;
+                mm = ghost_m64(C, mirror ? nxt.m : cur.m, D.wet_k, D.h_bot);
             }
             if (bhi) {
                 const bool mirror = D.wet_k == 2;
                 nxt.k = mirror ? km : cur.k;
-                nxt.m = (mirror ? mm : cur.m) - 6.0 * D.wet_k * D.h_top * C.sig;
+                nxt.m = ghost_m64(C, mirror ? mm : cur.m, D.wet_k, D.h_top);
             }
             const double dx = __fma_rn(C.four, cur.k, LB64_ADD(nxt.k, km));
             const double dy = LB64_SUB(nxt.m, mm);
