@@ -57,6 +57,8 @@ constexpr int kGraphBig = 64;
 // strips.
 constexpr int kMaxDeps = 15;
 constexpr int kGraphSmall = 2;
+constexpr size_t kPtsHeader = 16;  // bytes before the interface points (their count)
+constexpr int kPtsFirst = 1024;    // interface points fetched together with their count
 constexpr int kChunk = 1 << 20;  // nodes per staging chunk for host field output
 
 // rest-state weights of f (deviation storage): t_0 = 4/9, t_1..4 = 1/9, t_5..8 = 1/36
@@ -82,7 +84,7 @@ struct Layout {
     std::vector<size_t> geo_tiles;  // its tile list (ints)
     size_t flags = 0, dep_off = 0, dep_idx = 0;  // persistent schedules (batches)
     size_t descs = 0, items = 0, partials = 0, stats = 0, pts = 0, count = 0, staging = 0, err = 0,
-           sched = 0, c64 = 0;
+           sched = 0, c64 = 0, done = 0;
     size_t total = 0;
     long long item_cap = 0;
     int pts_cap = 0;
@@ -138,14 +140,13 @@ bool build_layout(int precision, int n_dom, const int* nx, const int* ny, Layout
     L.partials = off;
     off = align_up(off + sizeof(double) * lbfe::kStatsFields * lbfe::max_partials_needed(0, 0),
                    kAlign);
-    L.stats = off;
-    off = align_up(off + sizeof(StatsOut), kAlign);
-    L.pts = off;
-    off = align_up(off + sizeof(double) * 2 * pts_cap, kAlign);
-    L.count = off;
-    off = align_up(off + sizeof(int), kAlign);
-    L.err = off;
-    off = align_up(off + sizeof(unsigned), kAlign);
+    L.stats = off;  // the statistics, then the error word: one copy reads both
+    L.err = off + sizeof(StatsOut);
+    L.done = off + sizeof(StatsOut) + 2 * sizeof(unsigned);
+    off = align_up(off + sizeof(StatsOut) + 4 * sizeof(unsigned), kAlign);
+    L.count = off;  // the number of interface points, then the points
+    L.pts = off + kPtsHeader;
+    off = align_up(off + kPtsHeader + sizeof(double) * 2 * pts_cap, kAlign);
     L.sched = off;
     off = align_up(off + 2 * sizeof(int) * LB_MAX_SCHED_CLASSES, kAlign);
     L.staging = off;
@@ -245,6 +246,7 @@ struct lb_handle {
     double* d_pts() const { return reinterpret_cast<double*>(base + L.pts); }
     int* d_count() const { return reinterpret_cast<int*>(base + L.count); }
     double* d_staging() const { return reinterpret_cast<double*>(base + L.staging); }
+    int* d_done() const { return reinterpret_cast<int*>(base + L.done); }
     unsigned* d_err() const { return reinterpret_cast<unsigned*>(base + L.err); }
     // two device ints per schedule class (tile counter, finished CTAs)
     int* d_sched(int c) const { return reinterpret_cast<int*>(base + L.sched) + 2 * c; }
@@ -963,12 +965,22 @@ int use_device(const lb_handle* h)
 }
 
 // Synchronise the stream and report a device-side timeout recorded by a
-// bounded wait (the word is cleared once reported).
-int sync_and_check(lb_handle* h)
+// bounded wait (the word is cleared once reported).  With `so`, the statistics
+// come in the same copy.
+int sync_and_check(lb_handle* h, StatsOut* so = nullptr)
 {
-    unsigned err = 0;
-    LB_CUDA(cudaMemcpyAsync(&err, h->d_err(), sizeof(err), cudaMemcpyDeviceToHost, h->stream));
+    struct {
+        StatsOut stats;
+        unsigned err;
+    } got{};
+    static_assert(offsetof(decltype(got), err) == sizeof(StatsOut), "as laid out on the device");
+    const size_t skip = so ? 0 : sizeof(StatsOut);
+    LB_CUDA(cudaMemcpyAsync(reinterpret_cast<unsigned char*>(&got) + skip, h->base + h->L.stats + skip,
+                            sizeof(StatsOut) + sizeof(unsigned) - skip, cudaMemcpyDeviceToHost,
+                            h->stream));
     LB_CUDA(cudaStreamSynchronize(h->stream));
+    if (so) *so = got.stats;
+    const unsigned err = got.err;
     if (err != 0) {
         cudaMemsetAsync(h->d_err(), 0, sizeof(unsigned), h->stream);
         cudaStreamSynchronize(h->stream);
@@ -1312,6 +1324,35 @@ int check_geometry(const unsigned char* cls, int nx, int ny, int walls)
     return LB_OK;
 }
 
+// The phi = 0 points of a domain, (x, y) pairs in arbitrary order.  Their
+// number and the first kPtsFirst of them come in one copy.
+int interface_points(lb_handle* h, const DomDesc& D, std::vector<double>& raw)
+{
+    const int cap = 16 * (D.nx + D.ny);
+    const int e = lbfe::launch_crossings(h->precision, D, h->parity, h->d_pts(), h->d_count(), cap,
+                                         h->stream);
+    if (e != 0) return fail(LB_ERR_CUDA, "crossings launch failed: %s", cudaGetErrorString(cudaError_t(e)));
+    h->launches += 1;
+    static_assert(kPtsHeader == 2 * sizeof(double), "the count fills one point's place");
+    const int first = std::min(cap, kPtsFirst);
+    raw.resize(2 * size_t(first) + 2);
+    LB_CUDA(cudaMemcpyAsync(raw.data(), h->d_count(), kPtsHeader + sizeof(double) * 2 * first,
+                            cudaMemcpyDeviceToHost, h->stream));
+    LB_CUDA(cudaStreamSynchronize(h->stream));
+    int count = 0;
+    memcpy(&count, raw.data(), sizeof(int));
+    if (count > cap) return fail(LB_ERR_CAPACITY, "%d interface points exceed capacity %d", count, cap);
+    raw.erase(raw.begin(), raw.begin() + 2);
+    raw.resize(2 * size_t(count));
+    if (count > first) {
+        LB_CUDA(cudaMemcpyAsync(raw.data() + 2 * size_t(first), h->d_pts() + 2 * size_t(first),
+                                sizeof(double) * 2 * (count - first), cudaMemcpyDeviceToHost,
+                                h->stream));
+        LB_CUDA(cudaStreamSynchronize(h->stream));
+    }
+    return LB_OK;
+}
+
 // The device address of a page-locked host buffer (nullptr if the buffer is
 // pageable or not known to CUDA).
 double* device_alias(double* p)
@@ -1453,30 +1494,24 @@ int lb_moments(lb_handle* h, int dom, int on_device, double* rho, double* phi, d
     int rc = check_dom(h, dom);
     if (rc != LB_OK) return rc;
     const DomDesc& D = h->descs[dom];
-    if (stats) {
-        const int e = lbfe::launch_moments(h->precision, D, h->parity, 0, D.ny, nullptr, nullptr,
-                                           nullptr, nullptr, D.nx, h->d_partials(),
-                                           lbfe::max_partials_needed(0, 0), h->d_stats(), h->stream);
-        if (e != 0) return fail(LB_ERR_CUDA, "moments launch failed: %s", cudaGetErrorString(cudaError_t(e)));
-        h->launches += 2;
-    }
     double* outs[4] = {rho, phi, ux, uy};
     const bool any = rho || phi || ux || uy;
-    if (any && on_device) {
-        const int e = lbfe::launch_moments(h->precision, D, h->parity, 0, D.ny, rho, phi, ux, uy,
-                                           D.nx, nullptr, 0, nullptr, h->stream);
+    // page-locked host buffers are mapped into the device's address space:
+    // the kernel writes them directly
+    const bool mapped = any && !on_device && host_mapped(outs);
+    const bool direct = any && (on_device || mapped);
+    if (stats || direct) {
+        double* dev[4] = {nullptr, nullptr, nullptr, nullptr};
+        if (direct)
+            for (int k = 0; k < 4; ++k) dev[k] = outs[k] && mapped ? device_alias(outs[k]) : outs[k];
+        const int e = lbfe::launch_moments(
+            h->precision, D, h->parity, 0, D.ny, dev[0], dev[1], dev[2], dev[3], D.nx,
+            h->d_partials(), lbfe::max_partials_needed(0, 0), stats ? h->d_stats() : nullptr,
+            h->d_done(), h->stream);
         if (e != 0) return fail(LB_ERR_CUDA, "moments launch failed: %s", cudaGetErrorString(cudaError_t(e)));
         h->launches += 1;
-    } else if (any && host_mapped(outs)) {
-        // page-locked host buffers are mapped into the device's address
-        // space: the kernel writes them directly, in one pass
-        double* dev[4];
-        for (int k = 0; k < 4; ++k) dev[k] = outs[k] ? device_alias(outs[k]) : nullptr;
-        const int e = lbfe::launch_moments(h->precision, D, h->parity, 0, D.ny, dev[0], dev[1],
-                                           dev[2], dev[3], D.nx, nullptr, 0, nullptr, h->stream);
-        if (e != 0) return fail(LB_ERR_CUDA, "moments launch failed: %s", cudaGetErrorString(cudaError_t(e)));
-        h->launches += 1;
-    } else if (any) {
+    }
+    if (any && !direct) {
         const int chunk_rows = int(std::max<long long>(1, h->L.staging_nodes / D.nx));
         double* st = h->d_staging();
         const long long sn = h->L.staging_nodes;
@@ -1485,7 +1520,8 @@ int lb_moments(lb_handle* h, int dom, int on_device, double* rho, double* phi, d
             double* dev[4];
             for (int k = 0; k < 4; ++k) dev[k] = outs[k] ? st + k * sn : nullptr;
             const int e = lbfe::launch_moments(h->precision, D, h->parity, r0, nr, dev[0], dev[1],
-                                               dev[2], dev[3], D.nx, nullptr, 0, nullptr, h->stream);
+                                               dev[2], dev[3], D.nx, nullptr, 0, nullptr, nullptr,
+                                               h->stream);
             if (e != 0) return fail(LB_ERR_CUDA, "moments launch failed: %s", cudaGetErrorString(cudaError_t(e)));
             h->launches += 1;
             for (int k = 0; k < 4; ++k)
@@ -1496,9 +1532,7 @@ int lb_moments(lb_handle* h, int dom, int on_device, double* rho, double* phi, d
         }
     }
     StatsOut so{};
-    if (stats)
-        LB_CUDA(cudaMemcpyAsync(&so, h->d_stats(), sizeof(StatsOut), cudaMemcpyDeviceToHost, h->stream));
-    rc = sync_and_check(h);
+    rc = sync_and_check(h, stats ? &so : nullptr);
     if (rc != LB_OK) return rc;
     if (stats) {
         stats->mass = so.mass;
@@ -1521,21 +1555,10 @@ int lb_contact_angle(lb_handle* h, int dom, double exclude, double* theta_deg, d
     if (rc != LB_OK) return rc;
     if (!std::isfinite(exclude)) return fail(LB_ERR_INVALID_ARG, "exclude must be finite");
     const DomDesc& D = h->descs[dom];
-    const int cap = 16 * (D.nx + D.ny);
-    const int e = lbfe::launch_crossings(h->precision, D, h->parity, h->d_pts(), h->d_count(), cap,
-                                         h->stream);
-    if (e != 0) return fail(LB_ERR_CUDA, "crossings launch failed: %s", cudaGetErrorString(cudaError_t(e)));
-    h->launches += 1;
-    int count = 0;
-    LB_CUDA(cudaMemcpyAsync(&count, h->d_count(), sizeof(int), cudaMemcpyDeviceToHost, h->stream));
-    LB_CUDA(cudaStreamSynchronize(h->stream));
-    if (count > cap) return fail(LB_ERR_CAPACITY, "%d interface points exceed capacity %d", count, cap);
-    std::vector<double> raw(2 * size_t(count));
-    if (count > 0) {
-        LB_CUDA(cudaMemcpyAsync(raw.data(), h->d_pts(), sizeof(double) * 2 * count,
-                                cudaMemcpyDeviceToHost, h->stream));
-        LB_CUDA(cudaStreamSynchronize(h->stream));
-    }
+    std::vector<double> raw;
+    rc = interface_points(h, D, raw);
+    if (rc != LB_OK) return rc;
+    const int count = int(raw.size() / 2);
     std::vector<std::pair<double, double>> pts;
     const double wall = -0.5;
     for (int i = 0; i < count; ++i)
@@ -1692,21 +1715,10 @@ int lb_meniscus(lb_handle* h, int dom, int x_lo, int x_hi, int y_lo, int y_hi, d
     if (x_lo < 0 || x_hi > D.nx || x_lo + 2 > x_hi || y_lo < 0 || y_hi > D.ny || y_lo + 2 > y_hi ||
         !std::isfinite(exclude))
         return fail(LB_ERR_INVALID_ARG, "bad meniscus box");
-    const int cap = 16 * (D.nx + D.ny);
-    const int e = lbfe::launch_crossings(h->precision, D, h->parity, h->d_pts(), h->d_count(), cap,
-                                         h->stream);
-    if (e != 0) return fail(LB_ERR_CUDA, "crossings launch failed: %s", cudaGetErrorString(cudaError_t(e)));
-    h->launches += 1;
-    int count = 0;
-    LB_CUDA(cudaMemcpyAsync(&count, h->d_count(), sizeof(int), cudaMemcpyDeviceToHost, h->stream));
-    LB_CUDA(cudaStreamSynchronize(h->stream));
-    if (count > cap) return fail(LB_ERR_CAPACITY, "%d interface points exceed capacity %d", count, cap);
-    std::vector<double> raw(2 * size_t(count));
-    if (count > 0) {
-        LB_CUDA(cudaMemcpyAsync(raw.data(), h->d_pts(), sizeof(double) * 2 * count,
-                                cudaMemcpyDeviceToHost, h->stream));
-        LB_CUDA(cudaStreamSynchronize(h->stream));
-    }
+    std::vector<double> raw;
+    rc = interface_points(h, D, raw);
+    if (rc != LB_OK) return rc;
+    const int count = int(raw.size() / 2);
     // points on links with both ends in the box, away from the walls
     const double wb = y_lo - 0.5, wt = y_hi - 0.5;
     std::vector<std::pair<double, double>> pts;

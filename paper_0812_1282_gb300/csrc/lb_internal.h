@@ -122,9 +122,11 @@ int launch_init_eq(int precision, const DomDesc& d, const double* phi0, int pari
                    void* stream);
 // phi0 rows (nx per row, contiguous, device-addressable) into the pitched field.
 int launch_copy_rows(const DomDesc& d, const double* src, double* phi0, void* stream);
+// Fields (each may be nullptr) and, with out, the statistics: partials holds
+// max_partials block partials, done one int, zero between launches.
 int launch_moments(int precision, const DomDesc& d, int parity, int row0, int nrows,
                    double* rho, double* phi, double* ux, double* uy, long long ld,
-                   double* partials, int max_partials, StatsOut* out, void* stream);
+                   double* partials, int max_partials, StatsOut* out, int* done, void* stream);
 int launch_crossings(int precision, const DomDesc& d, int parity, double* pts, int* count,
                      int cap, void* stream);
 int launch_fill_ghosts(int precision, const DomDesc& d, int parity, void* stream);

@@ -288,39 +288,100 @@ int launch_init_eq(int precision, const DomDesc& d, const double* phi0, int pari
 // ------------------------------------------------------------- moments
 // Moments of the stored populations (Eq. moments) on rows
 // [row0, row0 + nrows): optional FP64 field outputs (leading dimension ld,
-// row-relative), and per-block partial sums for the diagnostics.
+// row-relative) and the diagnostics, in one pass over the state.
 // Reductions: fixed grid, per-thread serial accumulation, warp shuffles,
-// one partial per block, then a single-block pass in fixed order, so the
-// result is deterministic.
+// one partial per block, which the last block to finish combines in a fixed
+// order, so the result is deterministic.  A reading of a small lattice is a
+// handful of latencies: fields and statistics as two passes, the partials
+// combined by a launch of their own, and the results and the error word
+// fetched by a copy each took 43 us on 200 x 100 (FP32; 53 in FP64, whose
+// divisions and root are one reciprocal per node and one root now), 28 as one
+// launch and one copy, 10 of them the copy and the wait.
 constexpr int kMomBlock = 256;
 constexpr int kMaxMomBlocks = 4096;  // ~27 blocks of 256 per SM: enough loads in flight
 
 int max_partials_needed(int, int) { return kMaxMomBlocks; }
 
-__device__ __forceinline__ void warp_reduce(double (&v)[kStatsFields])
+// A thread's share of the statistics: the four sums, max |u|^2 (compared as
+// bits: it is never negative) and the non-finite nodes.
+struct MomAcc {
+    double s[4];
+    unsigned long long u2;
+    unsigned bad;
+};
+
+__device__ __forceinline__ void take_max(unsigned long long& a, unsigned long long b)
 {
+    a = a > b ? a : b;
+}
+
+// Reduction over a block of kMomBlock threads; the result is in threads 0..3
+// (the sums, in `sum`) and thread 0 (u2, bad).  An FP64 add takes its
+// scheduler's pipe for 64 cycles, so the four sums of a warp halve their
+// number with each exchange (2 + 1 + 1 + 1 + 1 adds instead of 4 x 5), and
+// the maximum and the count use integers.
+__device__ __forceinline__ void block_reduce(MomAcc v, double& sum, unsigned long long& u2,
+                                             unsigned& bad)
+{
+    constexpr unsigned kAll = 0xffffffffu;
+    constexpr int kWarps = kMomBlock / 32;
+    static_assert(kWarps * 4 == 32, "one warp combines the warps' sums");
+    __shared__ double red[kWarps][4];
+    __shared__ unsigned long long red_u2[kWarps];
+    __shared__ unsigned red_bad[kWarps];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const bool h16 = lane & 16, h8 = lane & 8;
+    const double a =
+        (h16 ? v.s[2] : v.s[0]) + __shfl_xor_sync(kAll, h16 ? v.s[0] : v.s[2], 16);
+    const double b =
+        (h16 ? v.s[3] : v.s[1]) + __shfl_xor_sync(kAll, h16 ? v.s[1] : v.s[3], 16);
+    double c = (h8 ? b : a) + __shfl_xor_sync(kAll, h8 ? a : b, 8);
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
+    for (int off = 4; off > 0; off >>= 1) c += __shfl_xor_sync(kAll, c, off);
 #pragma unroll
-        for (int k = 0; k < kStatsFields; ++k) {
-            const double o = __shfl_xor_sync(0xffffffffu, v[k], off);
-            v[k] = (k == 4) ? fmax(v[k], o) : v[k] + o;
-        }
+    for (int off = 16; off > 0; off >>= 1) take_max(v.u2, __shfl_xor_sync(kAll, v.u2, off));
+    v.bad = __reduce_add_sync(kAll, v.bad);
+    __syncthreads();  // an earlier reduction of this block is read
+    if ((lane & 7) == 0) red[wid][(h16 ? 2 : 0) + (h8 ? 1 : 0)] = c;
+    if (lane == 0) {
+        red_u2[wid] = v.u2;
+        red_bad[wid] = v.bad;
     }
+    __syncthreads();
+    sum = 0.0;
+    if (wid == 0) {
+        sum = red[lane >> 2][lane & 3];
+#pragma unroll
+        for (int off = 16; off > 2; off >>= 1) sum += __shfl_xor_sync(kAll, sum, off);
+        u2 = lane < kWarps ? red_u2[lane] : 0ull;
+        bad = lane < kWarps ? red_bad[lane] : 0u;
+#pragma unroll
+        for (int off = 4; off > 0; off >>= 1) take_max(u2, __shfl_xor_sync(kAll, u2, off));
+        bad = __reduce_add_sync(kAll, bad);
+    }
+}
+
+// j / r to the last bit or so from one reciprocal of r: the product, and its
+// residual's correction.
+__device__ __forceinline__ double div_by(double j, double r, double inv)
+{
+    const double q = j * inv;
+    return fma(fma(-q, r, j), inv, q);
 }
 
 template <typename Real>
 __global__ void __launch_bounds__(kMomBlock) moments_kernel(DomDesc D, int parity, int row0,
                                                             int nrows, double* rho, double* phi,
                                                             double* ux, double* uy, long long ld,
-                                                            double* partials)
+                                                            double* partials, StatsOut* out,
+                                                            int* done)
 {
     const Real* fs = static_cast<const Real*>((parity ? D.f[1] : D.f[0]));
     const Real* gs = static_cast<const Real*>((parity ? D.g[1] : D.g[0]));
     const long long P = D.plane;
-    const int nx = D.nx, pitch = D.pitch;
-    const long long n = (long long)nx * nrows;
-    double acc[kStatsFields] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+    const unsigned nx = unsigned(D.nx), pitch = unsigned(D.pitch);
+    const unsigned n = nx * unsigned(nrows);  // 9 planes stay below 2^31 elements
+    MomAcc acc{{0.0, 0.0, 0.0, 0.0}, 0ull, 0u};
     if constexpr (sizeof(Real) == 4) {
         // FP32 storage: per-node arithmetic in FP32 and per-thread sums of the
         // small quantities (rho - 1, rho u, the g tail) in FP32, of the phi
@@ -328,10 +389,8 @@ __global__ void __launch_bounds__(kMomBlock) moments_kernel(DomDesc D, int parit
         // FP64 pipe runs at 1/64 of the FP32 rate)
         float s_drho = 0.f, s_jx = 0.f, s_jy = 0.f, s_tail = 0.f, s_um = 0.f;
         long long s_word = 0, s_n = 0;
-        int s_bad = 0;
-        for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n;
-             k += (long long)gridDim.x * blockDim.x) {
-            const int yr = int(k / nx), x = int(k - (long long)yr * nx);
+        for (unsigned k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
+            const unsigned yr = k / nx, x = k - yr * nx;
             const long long q = (long long)yr * ld + x;
             if (D.cls && D.cls[(long long)(row0 + yr) * nx + x] != 0) {
                 // solid node: no fluid, no contribution to the diagnostics
@@ -369,18 +428,16 @@ __global__ void __launch_bounds__(kMomBlock) moments_kernel(DomDesc D, int parit
             s_word += __float_as_int(word_raw);
             ++s_n;
             s_um = finite ? fmaxf(s_um, umf) : s_um;
-            s_bad += finite ? 0 : 1;
+            acc.bad += finite ? 0u : 1u;
         }
-        acc[0] = double(s_n) + double(s_drho);
-        acc[1] = double(s_word) / G0<float>::kScale + double(s_tail);
-        acc[2] = double(s_jx);
-        acc[3] = double(s_jy);
-        acc[4] = double(s_um);
-        acc[5] = double(s_bad);
+        acc.s[0] = double(s_n) + double(s_drho);
+        acc.s[1] = double(s_word) / G0<float>::kScale + double(s_tail);
+        acc.s[2] = double(s_jx);
+        acc.s[3] = double(s_jy);
+        acc.u2 = __float_as_uint(s_um);  // max |u| itself
     } else {
-        for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n;
-             k += (long long)gridDim.x * blockDim.x) {
-            const int yr = int(k / nx), x = int(k - (long long)yr * nx);
+        for (unsigned k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
+            const unsigned yr = k / nx, x = k - yr * nx;
             const long long q = (long long)yr * ld + x;
             if (D.cls && D.cls[(long long)(row0 + yr) * nx + x] != 0) {
                 if (rho) rho[q] = 0.0;
@@ -391,80 +448,71 @@ __global__ void __launch_bounds__(kMomBlock) moments_kernel(DomDesc D, int parit
             }
             const long long o = (long long)(row0 + yr) * pitch + x + kXOff;
             double f[9], g[9];
-            for (int i = 0; i < 9; ++i) f[i] = double(fs[i * P + o]);
-            g[0] = G0<Real>::decode(gs[o]);
-            for (int i = 1; i < 9; ++i) g[i] = D.compact ? 0.0 : double(gs[i * P + o]);
+            for (int i = 0; i < 9; ++i) f[i] = fs[i * P + o];
+            for (int i = 0; i < 9; ++i) g[i] = gs[i * P + o];
             const double drho = (((f[0] + f[1]) + (f[2] + f[3])) + ((f[4] + f[5]) + (f[6] + f[7]))) + f[8];
             const double jx = (f[1] - f[2]) + (f[5] - f[6]) + (f[8] - f[7]);
             const double jy = (f[3] - f[4]) + (f[5] - f[6]) + (f[7] - f[8]);
             const double ph = phi_sum<double>(g);
-            const double r = 1.0 + drho;
-            const double vx = jx / r, vy = jy / r;
+            const double r = 1.0 + drho, inv = __drcp_rn(r);
+            const double vx = div_by(jx, r, inv), vy = div_by(jy, r, inv);
             if (rho) rho[q] = r;
             if (phi) phi[q] = ph;
             if (ux) ux[q] = vx;
             if (uy) uy[q] = vy;
-            const double um = sqrt(vx * vx + vy * vy);
-            const bool finite = isfinite(r) && isfinite(ph) && isfinite(um);
-            acc[0] += r;
-            acc[1] += ph;
-            acc[2] += jx;
-            acc[3] += jy;
-            acc[4] = finite ? fmax(acc[4], um) : acc[4];
-            acc[5] += finite ? 0.0 : 1.0;
+            if (partials == nullptr) continue;
+            const double u2 = vx * vx + vy * vy;
+            const bool finite = isfinite(r) && isfinite(ph) && isfinite(u2);
+            acc.s[0] += r;
+            acc.s[1] += ph;
+            acc.s[2] += jx;
+            acc.s[3] += jy;
+            if (finite) take_max(acc.u2, (unsigned long long)__double_as_longlong(u2));
+            acc.bad += finite ? 0u : 1u;
         }
     }
     if (partials == nullptr) return;
-    warp_reduce(acc);
-    __shared__ double red[kMomBlock / 32][kStatsFields];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    if (lane == 0)
-        for (int k = 0; k < kStatsFields; ++k) red[wid][k] = acc[k];
-    __syncthreads();
-    if (wid == 0) {
-        double v[kStatsFields];
-        for (int k = 0; k < kStatsFields; ++k)
-            v[k] = lane < (kMomBlock / 32) ? red[lane][k] : (k == 4 ? 0.0 : 0.0);
-        warp_reduce(v);
-        if (lane == 0)
-            for (int k = 0; k < kStatsFields; ++k) partials[blockIdx.x * kStatsFields + k] = v[k];
+    __shared__ bool last;
+    double sum;
+    unsigned long long u2 = 0ull;
+    unsigned bad = 0u;
+    block_reduce(acc, sum, u2, bad);
+    // one partial per block: the sums, then u2 and the count as bits
+    if (threadIdx.x < 4) {
+        partials[blockIdx.x * kStatsFields + threadIdx.x] = sum;
+        if (threadIdx.x == 0) {
+            partials[blockIdx.x * kStatsFields + 4] = __longlong_as_double((long long)u2);
+            partials[blockIdx.x * kStatsFields + 5] = __longlong_as_double((long long)bad);
+        }
+        __threadfence();
+        __syncwarp(0xfu);
+        if (threadIdx.x == 0) last = atomicAdd(done, 1) == int(gridDim.x) - 1;
     }
-}
-
-__global__ void finalize_stats_kernel(const double* __restrict__ partials, int nblocks,
-                                      StatsOut* out)
-{
-    double acc[kStatsFields] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-    for (int b = threadIdx.x; b < nblocks; b += blockDim.x)
-        for (int k = 0; k < kStatsFields; ++k) {
-            const double v = partials[b * kStatsFields + k];
-            acc[k] = (k == 4) ? fmax(acc[k], v) : acc[k] + v;
-        }
-    warp_reduce(acc);
-    __shared__ double red[32][kStatsFields];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    if (lane == 0)
-        for (int k = 0; k < kStatsFields; ++k) red[wid][k] = acc[k];
     __syncthreads();
-    if (wid == 0) {
-        double v[kStatsFields];
-        const int nw = blockDim.x >> 5;
-        for (int k = 0; k < kStatsFields; ++k) v[k] = lane < nw ? red[lane][k] : 0.0;
-        warp_reduce(v);
-        if (lane == 0) {
-            out->mass = v[0];
-            out->order = v[1];
-            out->mom_x = v[2];
-            out->mom_y = v[3];
-            out->max_u = v[4];
-            out->nonfinite = v[5];
-        }
+    if (!last) return;
+    // the last block: every block's partial is in memory
+    __threadfence();
+    acc = MomAcc{{0.0, 0.0, 0.0, 0.0}, 0ull, 0u};
+    for (int b = threadIdx.x; b < int(gridDim.x); b += kMomBlock) {
+        const double* p = partials + b * kStatsFields;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) acc.s[k] += __ldcg(p + k);
+        take_max(acc.u2, (unsigned long long)__double_as_longlong(__ldcg(p + 4)));
+        acc.bad += unsigned(__double_as_longlong(__ldcg(p + 5)));
+    }
+    block_reduce(acc, sum, u2, bad);
+    if (threadIdx.x < 4) (&out->mass)[threadIdx.x] = sum;  // mass, order, mom_x, mom_y
+    if (threadIdx.x == 0) {
+        out->max_u = sizeof(Real) == 4 ? double(__uint_as_float(unsigned(u2)))
+                                       : sqrt(__longlong_as_double((long long)u2));
+        out->nonfinite = double(bad);
+        *done = 0;  // for the next launch
     }
 }
 
 int launch_moments(int precision, const DomDesc& d, int parity, int row0, int nrows, double* rho,
                    double* phi, double* ux, double* uy, long long ld, double* partials,
-                   int max_partials, StatsOut* out, void* stream)
+                   int max_partials, StatsOut* out, int* done, void* stream)
 {
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const long long n = (long long)d.nx * nrows;
@@ -476,13 +524,10 @@ int launch_moments(int precision, const DomDesc& d, int parity, int row0, int nr
     double* part = out ? partials : nullptr;
     if (precision == 0)
         moments_kernel<float><<<grid, kMomBlock, 0, s>>>(d, parity, row0, nrows, rho, phi, ux, uy,
-                                                         ld, part);
+                                                         ld, part, out, done);
     else
         moments_kernel<double><<<grid, kMomBlock, 0, s>>>(d, parity, row0, nrows, rho, phi, ux,
-                                                          uy, ld, part);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess || out == nullptr) return static_cast<int>(e);
-    finalize_stats_kernel<<<1, 256, 0, s>>>(partials, grid, out);
+                                                          uy, ld, part, out, done);
     return static_cast<int>(cudaGetLastError());
 }
 
@@ -502,39 +547,64 @@ __device__ __forceinline__ double phi_at_node(const Real* g, long long P, long l
     return phi_sum<double>(v);
 }
 
+// An estimate of phi that costs no FP64 operation where the storage allows
+// one: the FP32 sum (compact: the word's value).
+template <typename Real>
+__device__ __forceinline__ Real phi_estimate(const Real* g, long long P, long long o, bool compact)
+{
+    if (sizeof(Real) == 4 && compact) return G0<Real>::value(g[o]);
+    Real v[9];
+    for (int i = 0; i < 9; ++i) v[i] = g[i * P + o];
+    return phi_sum<Real>(v);
+}
+
+// Whether a link whose ends have these estimates surely carries no crossing:
+// both of one sign, far from zero against the estimates' error (nine
+// roundings of numbers below 8: under 1e-5), and of a size phi has.  Only the
+// few links near the interface are evaluated in FP64.
+template <typename Real>
+__device__ __forceinline__ bool surely_none(Real a, Real b)
+{
+    const Real lo = Real(1e-3), hi = Real(4);
+    return (a > lo && b > lo && a < hi && b < hi) || (a < -lo && b < -lo && a > -hi && b > -hi);
+}
+
 template <typename Real>
 __global__ void crossings_kernel(DomDesc D, int parity, double* pts, int* count, int cap)
 {
     const Real* gs = static_cast<const Real*>((parity ? D.g[1] : D.g[0]));
     const long long P = D.plane;
-    const int nx = D.nx, ny = D.ny, pitch = D.pitch;
-    const long long n = (long long)nx * ny;
-    for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n;
-         k += (long long)gridDim.x * blockDim.x) {
-        const int y = int(k / nx), x = int(k - (long long)y * nx);
-        const unsigned char* cls = D.cls;
-        if (cls && cls[k] != 0) continue;  // links touching a solid node carry no interface
-        const bool cmp = D.compact != 0;
-        const double a = phi_at_node(gs, P, (long long)y * pitch + x + kXOff, cmp);
-        const int xp = x + 1 == nx ? 0 : x + 1;
-        const double b = phi_at_node(gs, P, (long long)y * pitch + xp + kXOff, cmp);
-        const bool bfluid = !cls || cls[(long long)y * nx + xp] == 0;
-        if (bfluid && ((a > 0.0 && b < 0.0) || (a < 0.0 && b > 0.0))) {
-            const int idx = atomicAdd(count, 1);
-            if (idx < cap) {
-                pts[2 * idx] = x + a / (a - b);
-                pts[2 * idx + 1] = double(y);
-            }
+    const unsigned nx = unsigned(D.nx), ny = unsigned(D.ny), pitch = unsigned(D.pitch);
+    const unsigned n = nx * ny;
+    const bool cmp = D.compact != 0;
+    const unsigned char* cls = D.cls;
+    auto append = [&](double px, double py) {
+        const int idx = atomicAdd(count, 1);
+        if (idx < cap) {
+            pts[2 * idx] = px;
+            pts[2 * idx + 1] = py;
         }
-        if (y + 1 < ny && (!cls || cls[(long long)(y + 1) * nx + x] == 0)) {
-            const double c = phi_at_node(gs, P, (long long)(y + 1) * pitch + x + kXOff, cmp);
-            if ((a > 0.0 && c < 0.0) || (a < 0.0 && c > 0.0)) {
-                const int idx = atomicAdd(count, 1);
-                if (idx < cap) {
-                    pts[2 * idx] = double(x);
-                    pts[2 * idx + 1] = y + a / (a - c);
-                }
-            }
+    };
+    for (unsigned k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
+        const unsigned y = k / nx, x = k - y * nx;
+        if (cls && cls[k] != 0) continue;  // links touching a solid node carry no interface
+        const unsigned xp = x + 1 == nx ? 0 : x + 1;
+        const long long o = (long long)y * pitch + x + kXOff;
+        const long long ob = (long long)y * pitch + xp + kXOff, oc = o + pitch;
+        const bool right = !cls || cls[y * nx + xp] == 0;
+        const bool up = y + 1 < ny && (!cls || cls[k + nx] == 0);
+        const Real ea = phi_estimate(gs, P, o, cmp);
+        const bool look_right = right && !surely_none(ea, phi_estimate(gs, P, ob, cmp));
+        const bool look_up = up && !surely_none(ea, phi_estimate(gs, P, oc, cmp));
+        if (!look_right && !look_up) continue;
+        const double a = phi_at_node(gs, P, o, cmp);
+        if (look_right) {
+            const double b = phi_at_node(gs, P, ob, cmp);
+            if ((a > 0.0 && b < 0.0) || (a < 0.0 && b > 0.0)) append(x + a / (a - b), double(y));
+        }
+        if (look_up) {
+            const double c = phi_at_node(gs, P, oc, cmp);
+            if ((a > 0.0 && c < 0.0) || (a < 0.0 && c > 0.0)) append(double(x), y + a / (a - c));
         }
     }
 }
