@@ -57,6 +57,7 @@ constexpr int kGraphBig = 64;
 // strips.
 constexpr int kMaxDeps = 15;
 constexpr int kGraphSmall = 2;
+constexpr int kMaxRemainders = 8;  // lengths of remainders with a graph of their own
 constexpr size_t kPtsHeader = 16;  // bytes before the interface points (their count)
 constexpr int kPtsFirst = 1024;    // interface points fetched together with their count
 constexpr int kChunk = 1 << 20;  // nodes per staging chunk for host field output
@@ -231,6 +232,7 @@ struct lb_handle {
     long long steps = 0;
     long long launches = 0;
     std::map<std::pair<int, int>, cudaGraphExec_t> graphs;  // (length, start parity)
+    std::vector<int> remainders;  // remainders of step counts asked for so far
     std::vector<double> host_pts;
     int n_geo = 0;  // domains with an obstacle map
     // rows of each domain's step tiles and the length of its tile list
@@ -261,6 +263,7 @@ void clear_graphs(lb_handle* h)
 {
     for (auto& kv : h->graphs) cudaGraphExecDestroy(kv.second);
     h->graphs.clear();
+    h->remainders.clear();
 }
 
 // Class of a domain under the handle's schedule.
@@ -628,9 +631,9 @@ lb_schedule default_schedule(const lb_handle* h)
 // bound by the FP64 pipe and the tiles still fit the SMs evenly (us per step,
 // staged and small: FP32 28 x 15 4.0 and 2.5, 200 x 100 4.3 and 2.9, 1000 x 500
 // 15.4 and 13.8, 2000 x 350 20.7 and 20.0, but 900^2 24.4 and 27.4; compact
-// 28 x 15 4.5 and 3.4, 200 x 100 4.8 and 3.3, 512 x 256 7.2 and 5.9, but 2000 x
-// 100 7.7 and 8.1; FP64 28 x 15 8.3 and 6.4, 200 x 100 11 and 7.4, 1000 x 500 115
-// and 110, 1200^2 313 and 300, but 2048^2 831 and 850).
+// 28 x 15 4.5 and 3.5, 200 x 100 4.8 and 3.6, 512 x 256 7.2 and 5.9, but 700 x
+// 300 7.8 and 8.8; FP64 28 x 15 8.3 and 6.5, 200 x 100 11 and 7.5, 1000 x 500
+// 115 and 111, but 1200^2 313 and 302 to 317, 2048^2 828 and 850).
 //  - FP32: 4 rows (3 to 7 are within 5 %);
 //  - compact, whose tiles expand a two-node halo: the fewest rows from 4 on
 //    with which every tile has an SM to itself, else 7;
@@ -644,7 +647,7 @@ int small_rows(const lb_handle* h)
     const DomDesc& D = h->descs[0];
     const bool fp64 = h->precision == LB_FP64;
     const long long nodes = (long long)D.nx * D.ny;
-    if (nodes > (fp64 ? 2000000 : (D.compact ? 120000 : 700000))) return 0;
+    if (nodes > (fp64 ? 800000 : (D.compact ? 140000 : 700000))) return 0;
     auto tiles = [&](int rows) { return (long long)((D.nx + 31) / 32) * ((D.ny + rows - 1) / rows); };
     if (D.compact) {
         for (int r = 4; r < 7; ++r)
@@ -922,6 +925,22 @@ int capture_steps(lb_handle* h, int len, int parity, bool fixed_parity, cudaGrap
     return LB_OK;
 }
 
+// Steps of the next launch of n remaining ones: graphs of 64, then one graph
+// for the remainder where the same one was asked for before (an interval
+// between two readings, stepped again and again: 500 steps are 8 launches
+// instead of 33, each 3.3 us of idle GPU), else graphs of two, which need no
+// capture of their own, and a single launch.
+int next_length(lb_handle* h, int n)
+{
+    if (n >= kGraphBig) return kGraphBig;
+    if (n > 2 * kGraphSmall) {
+        auto it = std::find(h->remainders.begin(), h->remainders.end(), n);
+        if (it != h->remainders.end()) return n;
+        if (int(h->remainders.size()) < kMaxRemainders) h->remainders.push_back(n);
+    }
+    return n >= kGraphSmall ? kGraphSmall : 1;
+}
+
 int get_graph(lb_handle* h, int len, int parity, cudaGraphExec_t* out)
 {
     auto key = std::make_pair(len, parity);
@@ -1166,6 +1185,7 @@ int make_handle(const lb_params* per_dom, const int* nx, const int* ny, int n_do
             D.hcls[k] = 0.0;
             D.fhcls[k] = 0.0f;
         }
+        D.self = h->d_descs() + d;
         D.c64 = nullptr;
         if (h->precision == LB_FP64) {
             D.c64 = reinterpret_cast<const double*>(h->base + L.c64 + sizeof(lbfe::Node64) * d);
@@ -1469,8 +1489,10 @@ int lb_step(lb_handle* h, int n)
     if (n < 0) return fail(LB_ERR_INVALID_ARG, "n must be >= 0");
     if (use_device(h) != LB_OK) return LB_ERR_CUDA;
     if (n > 0 && h->descs[0].compact) h->ghosts_stale = true;
+    bool pairs = false;  // the remainder goes by graphs of two
     while (n > 0) {
-        int len = n >= kGraphBig ? kGraphBig : (n >= kGraphSmall ? kGraphSmall : 1);
+        const int len = pairs ? std::min(n, kGraphSmall) : next_length(h, n);
+        pairs = pairs || len == kGraphSmall;
         if (len == 1) {
             const int rc = enqueue_step(h, h->parity, h->stream);
             if (rc != LB_OK) return rc;
@@ -1636,9 +1658,8 @@ int lb_set_wetting(lb_handle* h, int dom, double h_bottom, double h_top)
     if (!std::isfinite(h_bottom) || !std::isfinite(h_top))
         return fail(LB_ERR_INVALID_ARG, "wetting gradients must be finite");
     DomDesc& D = h->descs[dom];
-    // kernels take the descriptor by value (captured in the step graphs)
-    LB_CUDA(cudaStreamSynchronize(h->stream));
-    clear_graphs(h);
+    // the step kernels read the gradients from the device copy, so captured
+    // graphs stay as they are (rebuilding them took 170 us)
     h->params[dom].h_bottom = h_bottom;
     h->params[dom].h_top = h_top;
     D.h_bot = h_bottom;

@@ -52,6 +52,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cstddef>
 #include <vector>
 
 #include "lb_async.cuh"
@@ -143,6 +144,40 @@ __device__ __forceinline__ int wrap_any(int v, int n)
     return r < 0 ? r + n : r;
 }
 
+// Constants of a CTA in shared memory: the wall wetting gradients
+// (DomDesc::self) and, in FP64, the node constants.  A thread fetches at most
+// one early and puts it down when the CTA is about to meet, so that no warp
+// waits for the load in between.
+template <typename Real>
+struct GeoConst {
+    Real h_bot, h_top;
+    __device__ __forceinline__ Real fetch(const DomDesc& D) const
+    {
+        const int t = int(threadIdx.x);
+        return t == 0 ? D.self->fh_bot : (t == 1 ? D.self->fh_top : Real(0));
+    }
+    __device__ __forceinline__ void put(Real v)
+    {
+        if (threadIdx.x < 2) (&h_bot)[threadIdx.x] = v;
+    }
+};
+template <>
+struct GeoConst<double> {
+    double h_bot, h_top;
+    Node64 c;
+    __device__ __forceinline__ double fetch(const DomDesc& D) const
+    {
+        const int t = int(threadIdx.x);
+        return t == 0 ? D.self->h_bot
+                      : (t == 1 ? D.self->h_top : (t < kNode64 + 2 ? D.c64[t - 2] : 0.0));
+    }
+    __device__ __forceinline__ void put(double v)
+    {
+        if (threadIdx.x < kNode64 + 2) (&h_bot)[threadIdx.x] = v;
+    }
+};
+static_assert(offsetof(GeoConst<double>, c) == 2 * sizeof(double), "put() fills it in order");
+
 // Per-CTA tables of a tile: the wrapped halo coordinates and the class map
 // with its halo.  They depend only on the geometry, so the persistent form
 // builds them once per launch.
@@ -154,10 +189,12 @@ struct GeoTables {
     signed char cl[TY + 2 * kGC][kGCX];  // 0 fluid, k > 0 solid class k, -1 / -2 wall rows
 };
 
-template <int TY>
-__device__ __forceinline__ void geo_tile_setup(const DomDesc& D, int x0, int y0, GeoTables<TY>& t)
+template <typename Real, int TY>
+__device__ __forceinline__ void geo_tile_setup(const DomDesc& D, int x0, int y0, GeoTables<TY>& t,
+                                               GeoConst<Real>& K)
 {
     constexpr int CY = TY + 2 * kGC;
+    const Real kv = K.fetch(D);
     const int nx = D.nx, ny = D.ny;
     // periodic wrap of the halo coordinates
     for (int k = threadIdx.x; k < kGCX + CY; k += blockDim.x) {
@@ -183,6 +220,7 @@ __device__ __forceinline__ void geo_tile_setup(const DomDesc& D, int x0, int y0,
             c = D.cls[t.rowc[cy] + (t.colx[cx] - kXOff)];
         t.cl[cy][cx] = static_cast<signed char>(c);
     }
+    K.put(kv);
     __syncthreads();
 }
 
@@ -204,17 +242,15 @@ __device__ __forceinline__ Real geo_ld(const Real* p)
 // only, the diagonal) directions d towards fluid of phi(s + k d) - k h, k =
 // D.wet_k.
 template <typename Real, class ClsF, class PhiF>
-__device__ __forceinline__ bool geo_ghost(const DomDesc& D, int x, int y, int y_lat, ClsF cls,
-                                          PhiF phi, Real& value)
+__device__ __forceinline__ bool geo_ghost(const DomDesc& D, const GeoConst<Real>& K, int x, int y,
+                                          int y_lat, ClsF cls, PhiF phi, Real& value)
 {
-    const Real h_bot = sizeof(Real) == 4 ? Real(D.fh_bot) : Real(D.h_bot);
-    const Real h_top = sizeof(Real) == 4 ? Real(D.fh_top) : Real(D.h_top);
     const int k = cls(x, y);
     if (k == kNodeWall) {
-        value = y_lat == 0 ? phi(x, y + 1) - h_bot : phi(x, y - 1) - h_top;
+        value = y_lat == 0 ? phi(x, y + 1) - K.h_bot : phi(x, y - 1) - K.h_top;
         return true;
     }
-    const Real h = k == -1 ? h_bot : (k == -2 ? h_top : class_h<Real>(D, k));
+    const Real h = k == -1 ? K.h_bot : (k == -2 ? K.h_top : class_h<Real>(D, k));
     Real sum = Real(0);
     int n = 0;
 #pragma unroll
@@ -243,20 +279,6 @@ __device__ __forceinline__ bool geo_ghost(const DomDesc& D, int x, int y, int y_
     value = mean - Real(D.wet_k) * h;
     return true;
 }
-
-// The node constants of a CTA (FP64 only) and their load.
-template <typename Real>
-struct GeoConst {
-    __device__ __forceinline__ void load(const DomDesc&) {}
-};
-template <>
-struct GeoConst<double> {
-    Node64 c;
-    __device__ __forceinline__ void load(const DomDesc& D)
-    {
-        load_node64(c, D.c64, int(threadIdx.x));
-    }
-};
 
 // Collision of one fluid node from its pulled f, g, its phi c and the phi of
 // its eight neighbours (ghost values at solid ones), directions 1..8 in nb.
@@ -400,7 +422,7 @@ __device__ __forceinline__ void geo_tile_step(const DomDesc& D, const GeoConst<R
             const int sy = k / GX - 1, sx = k - (sy + 1) * GX - 1;
             if (cls(sx, sy) == 0) continue;
             Real v;
-            if (geo_ghost<Real>(D, sx, sy, y0 + sy, cls, phi, v)) phi(sx, sy) = v;
+            if (geo_ghost<Real>(D, K, sx, sy, y0 + sy, cls, phi, v)) phi(sx, sy) = v;
         }
         __syncthreads();
     }
@@ -458,8 +480,7 @@ __global__ void __launch_bounds__(kGTX * TY) geo_step_kernel(DomDesc D, int pari
     const int e = tiles[blockIdx.x], ntx = (D.nx + kGTX - 1) / kGTX;
     const int q = e & kGeoTileIndex;
     const int x0 = q % ntx * kGTX, y0 = q / ntx * TY;
-    K.load(D);
-    geo_tile_setup<TY>(D, x0, y0, t);
+    geo_tile_setup<Real, TY>(D, x0, y0, t, K);
     pdl_wait_prev();
     geo_tile_step<Real, MRT, TY, false>(D, K, parity, x0, y0, e < 0, t, ph);
 }
@@ -508,7 +529,7 @@ __device__ __forceinline__ void geo_node_update(const DomDesc& D, const GeoConst
         const int qx = x + gex(i), qy = y + gey(i);
         if (cls_l(qx, qy) != 0) {
             next_to_solid = true;
-            geo_ghost<Real>(D, qx, qy, qy, cls_l, phi_l, nb[i]);
+            geo_ghost<Real>(D, K, qx, qy, qy, cls_l, phi_l, nb[i]);
         } else {
             nb[i] = phi_l(qx, qy);
         }
@@ -539,7 +560,7 @@ __global__ void __launch_bounds__(kGTX * kGTY, sizeof(Real) == 4 ? 4 : 2)
     const int x0 = blockIdx.x * kGTX, y0 = blockIdx.y * kGTY;
     const int nx = D.nx, ny = D.ny;
     const int tid = int(threadIdx.x), nthr = int(blockDim.x);
-    S.K.load(D);
+    S.K.put(S.K.fetch(D));
     // 0. wrapped halo coordinates and the class map on the tile + kFC
     for (int k = tid; k < kFCX + kFCY; k += nthr) {
         if (k < kFCX)
@@ -692,8 +713,7 @@ __global__ void __launch_bounds__(kGTX * kGTY, sizeof(Real) == 4 ? 4 : 2)
     const int ntx = int(gridDim.x), nty = int(gridDim.y);
     const int tx = int(blockIdx.x), ty = int(blockIdx.y), me = ty * ntx + tx;
     const int x0 = tx * kGTX, y0 = ty * kGTY;
-    K.load(D);
-    geo_tile_setup<kGTY>(D, x0, y0, t);
+    geo_tile_setup<Real, kGTY>(D, x0, y0, t, K);
     if (threadIdx.x == 0) {
         // the tiles under the halo (the wrapped columns and rows of the
         // tables; a short last tile can bring a second tile within reach)

@@ -54,6 +54,10 @@ struct DomDesc {
     const unsigned char* cls;
     double hcls[8];
     float fhcls[8];
+    // This descriptor's copy in device memory, whose wetting gradients the step
+    // kernels read: they change between steps (lb_set_wetting) without a new
+    // capture of the step graphs, which hold the other fields by value.
+    const DomDesc* self;
     const double* c64;  // FP64: the node constants (Node64, lb_node64.cuh) in device memory
 };
 

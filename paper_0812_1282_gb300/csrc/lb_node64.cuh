@@ -101,12 +101,11 @@ __device__ __forceinline__ double rcp64(const Node64& C, double x)
     return __fma_rn(r, __fma_rn(e, e, e), r);
 }
 
-// m of a wall ghost row (lb_step64.cuh) from the m of the row it mirrors: phi
-// less wet_k h, 4 + 1 + 1 times, on the scaled phi.  (As one fused operation
-// it costs the row loop 8 %: the compiler keeps fewer constants.)
-__device__ __forceinline__ double ghost_m64(const Node64& C, double m, int wet_k, double h)
+// What m of a wall ghost row (lb_step64.cuh) is less than the m of the row it
+// mirrors: phi is wet_k h less, 4 + 1 + 1 times, on the scaled phi.
+__device__ __forceinline__ double ghost_shift64(double sig, int wet_k, double h)
 {
-    return __dsub_rn(m, __dmul_rn(6.0 * wet_k * h, C.sig));
+    return __dmul_rn(6.0 * wet_k * h, sig);
 }
 
 // phi = sum of the nine pulled g

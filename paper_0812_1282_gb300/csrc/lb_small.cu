@@ -101,7 +101,8 @@ __global__ void __launch_bounds__(kSmallMaxThreads) small_step_kernel(DomDesc D,
 {
     extern __shared__ __align__(16) unsigned char smem[];
     Real* ph = reinterpret_cast<Real*>(smem);
-    __shared__ Node64 C;  // FP64 only
+    __shared__ Node64 C;     // FP64 only
+    __shared__ Real wet[2];  // wetting gradients, bottom and top
     const int TY = int(blockDim.x) / kTX;
     const SmallTile T(D, TY);
     const int nx = D.nx, ny = D.ny, pitch = D.pitch, P = int(D.plane);
@@ -121,8 +122,10 @@ __global__ void __launch_bounds__(kSmallMaxThreads) small_step_kernel(DomDesc D,
     if (live) pull9<Real>(gs, P, pitch, ny, walls, x, y, g);
     if (halo) pull9<Real>(gs, P, pitch, ny, walls, T.x0 + hx, row(T.y0 + hy), gh);
     if (live) pull9<Real>(fs, P, pitch, ny, walls, x, y, f);
+    // the wetting gradients, in flight with the populations
+    const Real wv = tid == 0 ? wet_bottom<Real>(D) : (tid == 1 ? wet_top<Real>(D) : Real(0));
     if constexpr (sizeof(Real) == 8) {
-        if (tid < kNode64) reinterpret_cast<double*>(&C)[tid] = D.c64[tid];
+        load_node64(C, D.c64, tid);
         __syncthreads();
     }
     // the stored value: phi, in FP64 scaled for the stencils (lb_step64.cuh)
@@ -144,6 +147,7 @@ __global__ void __launch_bounds__(kSmallMaxThreads) small_step_kernel(DomDesc D,
         halo = halo_at(k, T, walls, ny, hx, hy);
         if (halo) pull9<Real>(gs, P, pitch, ny, walls, T.x0 + hx, row(T.y0 + hy), gh);
     }
+    if (tid < 2) wet[tid] = wv;
     __syncthreads();
     if (!live) return;
     const bool blo = walls && y == 0, bhi = walls && y == ny - 1;
@@ -171,12 +175,12 @@ __global__ void __launch_bounds__(kSmallMaxThreads) small_step_kernel(DomDesc D,
         if (blo) {
             const Row& v = D.wet_k == 2 ? up : cur;
             dn.k = v.k;
-            dn.m = ghost_m64(C, v.m, D.wet_k, D.h_bot);
+            dn.m = __dsub_rn(v.m, ghost_shift64(C.sig, D.wet_k, wet[0]));
         }
         if (bhi) {
             const Row& v = D.wet_k == 2 ? dn : cur;
             up.k = v.k;
-            up.m = ghost_m64(C, v.m, D.wet_k, D.h_top);
+            up.m = __dsub_rn(v.m, ghost_shift64(C.sig, D.wet_k, wet[1]));
         }
         const double X = __fma_rn(C.four, cur.k, LB64_ADD(up.k, dn.k));
         const double Y = LB64_SUB(up.m, dn.m);
@@ -198,12 +202,12 @@ __global__ void __launch_bounds__(kSmallMaxThreads) small_step_kernel(DomDesc D,
             s[j] = gm[j - 1];
         }
         if (bhi) {
-            const Real h2 = Real(D.wet_k) * prm.h_top;
+            const Real h2 = Real(D.wet_k) * wet[1];
 #pragma unroll
             for (int j = 0; j < 3; ++j) n[j] = n[j] - h2;
         }
         if (blo) {
-            const Real h2 = Real(D.wet_k) * prm.h_bot;
+            const Real h2 = Real(D.wet_k) * wet[0];
 #pragma unroll
             for (int j = 0; j < 3; ++j) s[j] = s[j] - h2;
         }
@@ -243,6 +247,8 @@ __global__ void __launch_bounds__(kSmallMaxThreads) small_compact_kernel(DomDesc
     const NodeParams<float> prm = node_params<float>(D);
     float f[9];
     if (live) pull9<float>(fs, P, pitch, ny, walls, x, y, f);
+    __shared__ float wet[2];  // wetting gradients, bottom and top
+    const float wv = tid == 0 ? wet_bottom<float>(D) : (tid == 1 ? wet_top<float>(D) : 0.f);
     // 1. expand the compact values of the tile and two nodes around it
     for (int k = tid; k < ne; k += int(blockDim.x)) {
         const int cy = k / kEW, cx = k - cy * kEW;
@@ -282,6 +288,7 @@ __global__ void __launch_bounds__(kSmallMaxThreads) small_compact_kernel(DomDesc
         // a periodic halo row is the row across the lattice's edge
         ph[(hy + 1) * kPW + hx + 1] = phi_at(hx, hy, dump).lane(0);
     }
+    if (tid < 2) wet[tid] = wv;
     __syncthreads();
     // 3. collide
     if (!live) return;
@@ -296,12 +303,12 @@ __global__ void __launch_bounds__(kSmallMaxThreads) small_compact_kernel(DomDesc
         s[j] = f2(gm[j - 1]);
     }
     if (bhi) {
-        const f2 h(float(D.wet_k) * prm.h_top);
+        const f2 h(float(D.wet_k) * wet[1]);
 #pragma unroll
         for (int j = 0; j < 3; ++j) n[j] = n[j] - h;
     }
     if (blo) {
-        const f2 h(float(D.wet_k) * prm.h_bot);
+        const f2 h(float(D.wet_k) * wet[0]);
 #pragma unroll
         for (int j = 0; j < 3; ++j) s[j] = s[j] - h;
     }

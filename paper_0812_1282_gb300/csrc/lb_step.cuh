@@ -58,6 +58,18 @@ __device__ __forceinline__ NodeParams<double> node_params<double>(const DomDesc&
                               D.lut_lo, D.lut_step, D.lut_inv, D.lut_kmax};
 }
 
+// The wall wetting gradients as they are now (DomDesc::self).
+template <typename Real>
+__device__ __forceinline__ Real wet_bottom(const DomDesc& D)
+{
+    return sizeof(Real) == 4 ? Real(D.self->fh_bot) : Real(D.self->h_bot);
+}
+template <typename Real>
+__device__ __forceinline__ Real wet_top(const DomDesc& D)
+{
+    return sizeof(Real) == 4 ? Real(D.self->fh_top) : Real(D.self->h_top);
+}
+
 // velocity y-components in the paper's order, and the opposite direction
 __device__ __forceinline__ int ey_of(int i)
 {
@@ -183,8 +195,8 @@ __device__ __forceinline__ void produce_tile(const DomDesc& D, int parity, int x
 // Compute warp cw (0-based among compute warps) processes its 32 columns of
 // one tile.  q: stage sequence number of the tile's first stage.
 // prm_shared, when set, holds the node parameters in shared memory; the
-// collision then reads them at each use instead of keeping them in
-// registers for the whole tile.
+// collision and the wall ghost rows then read them at each use instead of
+// keeping them in registers for the whole tile.
 template <typename Real, bool MRT, int S, int NWC = 0>
 __device__ __forceinline__ void consume_tile(const DomDesc& D, int parity, int x0, int y0, int rows,
                                              unsigned char* __restrict__ smem, int nw, int cw,
@@ -274,7 +286,7 @@ __device__ __forceinline__ void consume_tile(const DomDesc& D, int parity, int x
             publish(1, 1, 1);
             // each lane forms its own entries: row k - 1 less k h (k = 2:
             // mirror about row 0; k = 1: one-sided across the wall plane)
-            ghost_row(-1, D.wet_k - 1, Real(D.wet_k) * prm.h_bot);
+            ghost_row(-1, D.wet_k - 1, Real(D.wet_k) * (prm_shared ? prm_shared->h_bot : wet_bottom<Real>(D)));
         }
     }
     bool have_next = bottom_ghost;
@@ -285,7 +297,7 @@ __device__ __forceinline__ void consume_tile(const DomDesc& D, int parity, int x
                 wait_full(yn - first);
                 if (active) publish(yn - first, wrap_row(yn), yn);
             } else if (active) {
-                ghost_row(yn, ny - D.wet_k, Real(D.wet_k) * prm.h_top);
+                ghost_row(yn, ny - D.wet_k, Real(D.wet_k) * (prm_shared ? prm_shared->h_top : wet_top<Real>(D)));
             }
         }
         have_next = false;

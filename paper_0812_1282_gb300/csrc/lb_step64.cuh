@@ -18,9 +18,11 @@
 // the same sequence of barriers whatever its bounded stage waits return.
 //
 // Measured (MRT, 2048^2, best tile, per step): 1828 us with per-warp halos,
-// the phi ring read nine times a node and the plain arithmetic, 831 us so
-// (5.05 G node updates/s, 0.93 of what 112 + 4 operations allow at the
-// pipe's 628 G DFMA/s); BGK 951 us.  128 x 8 tiles are fastest there, 64 x 16
+// the phi ring read nine times a node and the plain arithmetic, 828 us so
+// (5.07 G node updates/s, 0.94 of what 112 + 4 operations allow at the
+// pipe's 628 G DFMA/s); BGK 900 us.  Wall rows take a copy of the code of
+// their own: their tests and ghost values in the common one cost it 7 %
+// (890 us).  128 x 8 tiles are fastest there, 64 x 16
 // within 1 %; wider tiles leave too few CTAs per SM to hide the barrier.
 #pragma once
 
@@ -41,11 +43,6 @@ struct Layout64 {
     __host__ __device__ explicit Layout64(int nw) : L(nw, kStages64) {}
     __host__ __device__ size_t ring_row() const { return size_t(L.W) + 2; }
     __host__ __device__ size_t total() const { return L.rings() + 2 * ring_row() * 8; }
-};
-
-// The derivative values a row contributes (see above).
-struct Row64 {
-    double k, m;
 };
 
 template <bool MRT>
@@ -91,9 +88,8 @@ __device__ __forceinline__ void consume_tile64(const DomDesc& D, const Node64& C
     struct Row {
         double phi, s, k, h, m;
     };
-    auto row_of = [&](int p, int r, Row& v) {
+    auto publish = [&](int p, Row& v, bool blo, bool bhi) {
         const double* sg = stage_ptr(p) + 9 * segw;
-        const bool blo = walls && r == 0, bhi = walls && r == ny - 1;
         double* rr = ring + size_t(p & 1) * Y.ring_row();
         double g[9];
         if (active) {
@@ -107,8 +103,15 @@ __device__ __forceinline__ void consume_tile64(const DomDesc& D, const Node64& C
             read9<double>(sg, segw, c + 4, blo, bhi, g);
             rr[c + 1] = LB64_MUL(C.sig, phi64(C, g));
         }
+    };
+    auto row_of = [&](int p, int r, Row& v) {
+        if (walls && (r == 0 || r == ny - 1))
+            publish(p, v, r == 0, r == ny - 1);
+        else
+            publish(p, v, false, false);
         __syncwarp();
         named_sync(kComputeBarrier64, 32 * NW);
+        const double* rr = ring + size_t(p & 1) * Y.ring_row();
         if (active) {
             const double w = rr[col], e = rr[col + 2];
             v.k = LB64_SUB(e, w);
@@ -117,14 +120,49 @@ __device__ __forceinline__ void consume_tile64(const DomDesc& D, const Node64& C
         }
     };
     auto wrap_row = [&](int r) { return r < 0 ? r + ny : (r >= ny ? r - ny : r); };
-
-    const int first = T.first, y1 = T.y1;
-    const bool bottom_ghost = walls && y0 == 0;
     Row cur, nxt;
     double km = 0.0, mm = 0.0;  // k and m of row y - 1
     cur.phi = cur.s = cur.k = cur.h = cur.m = 0.0;
     nxt = cur;
-    if (!bottom_ghost) {
+    // collide row y (staged at position p) from the row values around it
+    auto collide_row = [&](int y, int p, bool blo, bool bhi) {
+        double f[9];
+        read9<double>(stage_ptr(p), segw, col + 4, blo, bhi, f);
+        const double dx = __fma_rn(C.four, cur.k, LB64_ADD(nxt.k, km));
+        const double dy = LB64_SUB(nxt.m, mm);
+        const double lap = __fma_rn(C.m20, cur.s, __fma_rn(C.four, cur.h, LB64_ADD(nxt.m, mm)));
+        double fo[9], go[9];
+        collide64<MRT>(C, f, cur.phi, dx, dy, lap, D.step2 && (blo || bhi), D.step2_relax_j != 0,
+                       [&](double (&g)[9]) {
+                           read9<double>(stage_ptr(p) + 9 * segw, segw, col + 4, blo, bhi, g);
+                       },
+                       fo, go);
+        const int o = y * pitch + x + kXOff;
+#pragma unroll
+        for (int i = 0; i < 9; ++i) {
+            fd[i * P + o] = fo[i];
+            gd[i * P + o] = go[i];
+        }
+        // periodic ghost copies: logical 0, 1 also at nx, nx+1 and
+        // logical nx-2, nx-1 also at -2, -1
+        if (x < 2) {
+#pragma unroll
+            for (int i = 0; i < 9; ++i) {
+                fd[i * P + o + nx] = fo[i];
+                gd[i * P + o + nx] = go[i];
+            }
+        }
+        if (x >= nx - 2) {
+#pragma unroll
+            for (int i = 0; i < 9; ++i) {
+                fd[i * P + o - nx] = fo[i];
+                gd[i * P + o - nx] = go[i];
+            }
+        }
+    };
+
+    const int first = T.first, y1 = T.y1;
+    if (!(walls && y0 == 0)) {
         wait_full(0);
         row_of(0, wrap_row(y0 - 1), nxt);
         km = nxt.k;
@@ -136,57 +174,28 @@ __device__ __forceinline__ void consume_tile64(const DomDesc& D, const Node64& C
     for (int y = y0; y < y1; ++y) {
         const int yn = y + 1, py = y - first;
         const bool blo = walls && y == 0, bhi = walls && y == ny - 1;
-        double f[9];
         if (!bhi) {
             wait_full(yn - first);
             row_of(yn - first, wrap_row(yn), nxt);
         }
         if (active) {
-            read9<double>(stage_ptr(py), segw, col + 4, blo, bhi, f);
-            // a wall ghost row is row k - 1 (ny - k) less k h: its k is that
-            // row's and its m that row's less 6 k h (scaled)
-            if (blo) {
+            // wall rows apart, so that the others carry none of their tests
+            if (blo || bhi) {
+                // a wall ghost row is row k - 1 (ny - k) less k h: its k is
+                // that row's and its m that row's less 6 k h (scaled)
                 const bool mirror = D.wet_k == 2;
-                km = mirror ? nxt.k : cur.k;
-                mm = ghost_m64(C, mirror ? nxt.m : cur.m, D.wet_k, D.h_bot);
-            }
-            if (bhi) {
-                const bool mirror = D.wet_k == 2;
-                nxt.k = mirror ? km : cur.k;
-                nxt.m = ghost_m64(C, mirror ? mm : cur.m, D.wet_k, D.h_top);
-            }
-            const double dx = __fma_rn(C.four, cur.k, LB64_ADD(nxt.k, km));
-            const double dy = LB64_SUB(nxt.m, mm);
-            const double lap =
-                __fma_rn(C.m20, cur.s, __fma_rn(C.four, cur.h, LB64_ADD(nxt.m, mm)));
-            double fo[9], go[9];
-            collide64<MRT>(C, f, cur.phi, dx, dy, lap, D.step2 && (blo || bhi),
-                           D.step2_relax_j != 0,
-                           [&](double (&g)[9]) {
-                               read9<double>(stage_ptr(py) + 9 * segw, segw, col + 4, blo, bhi, g);
-                           },
-                           fo, go);
-            const int o = y * pitch + x + kXOff;
-#pragma unroll
-            for (int i = 0; i < 9; ++i) {
-                fd[i * P + o] = fo[i];
-                gd[i * P + o] = go[i];
-            }
-            // periodic ghost copies: logical 0, 1 also at nx, nx+1 and
-            // logical nx-2, nx-1 also at -2, -1
-            if (x < 2) {
-#pragma unroll
-                for (int i = 0; i < 9; ++i) {
-                    fd[i * P + o + nx] = fo[i];
-                    gd[i * P + o + nx] = go[i];
+                if (blo) {
+                    km = mirror ? nxt.k : cur.k;
+                    mm = __dsub_rn(mirror ? nxt.m : cur.m,
+                                   ghost_shift64(C.sig, D.wet_k, wet_bottom<double>(D)));
+                } else {
+                    nxt.k = mirror ? km : cur.k;
+                    nxt.m = __dsub_rn(mirror ? mm : cur.m,
+                                      ghost_shift64(C.sig, D.wet_k, wet_top<double>(D)));
                 }
-            }
-            if (x >= nx - 2) {
-#pragma unroll
-                for (int i = 0; i < 9; ++i) {
-                    fd[i * P + o - nx] = fo[i];
-                    gd[i * P + o - nx] = go[i];
-                }
+                collide_row(y, py, blo, bhi);
+            } else {
+                collide_row(y, py, false, false);
             }
             km = cur.k;
             mm = cur.m;

@@ -387,7 +387,7 @@ __device__ __forceinline__ void consume_tile_c(const DomDesc& D, int parity, int
             row3(rslot(y), cw_, cc, ce);
             if (bhi) {
                 row3(rslot(ny - D.wet_k), nw_, nc, ne);
-                const f2 h(float(D.wet_k) * (PRM_SMEM ? prm_shared->h_top : prm.h_top));
+                const f2 h(float(D.wet_k) * (PRM_SMEM ? prm_shared->h_top : wet_top<float>(D)));
                 nw_ = nw_ - h;
                 nc = nc - h;
                 ne = ne - h;
@@ -396,7 +396,7 @@ __device__ __forceinline__ void consume_tile_c(const DomDesc& D, int parity, int
             }
             if (blo) {
                 row3(rslot(D.wet_k - 1), sw, sc_, se);
-                const f2 h(float(D.wet_k) * (PRM_SMEM ? prm_shared->h_bot : prm.h_bot));
+                const f2 h(float(D.wet_k) * (PRM_SMEM ? prm_shared->h_bot : wet_bottom<float>(D)));
                 sw = sw - h;
                 sc_ = sc_ - h;
                 se = se - h;
