@@ -284,7 +284,9 @@ int lb_load_state(lb_handle* h, const void* host_buf, size_t bytes);
  * (lb_schedule).  Invalidates captured graphs.  A handle starts with a shape
  * chosen from its domains' sizes; a small single domain starts with a step
  * made for small lattices, for which the shape here is the one the general
- * step would take (setting a shape selects the general step). */
+ * step would take (setting a shape selects the general step).  On a large
+ * single domain with compact storage a shape of at least 48 rows keeps two
+ * steps per launch (lb_schedule), one of fewer rows takes one. */
 int lb_set_tile(lb_handle* h, int block_x, int rows);
 int lb_get_tile(const lb_handle* h, int* block_x, int* rows);
 
@@ -334,8 +336,12 @@ int lb_get_tile(const lb_handle* h, int* block_x, int* rows);
  *               2 runs two steps per launch (each CTA steps its tile and a
  *               four-node halo into shared memory, then its tile again; the
  *               halo is computed redundantly, no launch sits between the
- *               two steps); 0 or 1 one step per launch.  Ignored elsewhere
- *               and under persist.
+ *               two steps); 0 or 1 one step per launch.  A single domain
+ *               without obstacles and with compact g storage likewise (each
+ *               CTA carries its rows through both steps, so that the state
+ *               crosses the memory once per two steps; block_x[0] 64, 96 or
+ *               128, at least 8 x 8 nodes, else one step per launch); large
+ *               ones start so.  Ignored elsewhere and under persist.
  *  seal_edges[k]: compact storage: 1 makes class k's strips that cover
  *               their whole domain also zero the padding and (stale) ghost
  *               columns that share a 32-byte sector with their rows' first

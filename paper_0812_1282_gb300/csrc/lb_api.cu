@@ -228,6 +228,10 @@ struct lb_handle {
     // alone, so after steps they may be stale; they are refreshed before
     // another schedule (which may split a domain) or a checkpoint uses them
     bool ghosts_stale = false;
+    // two-step launches keep ghost columns four wide: whether the current
+    // buffer's are (wide_ok), and whether any buffer's outer ones may be other
+    // than the zeros that every other kernel leaves there (wide_used)
+    bool wide_ok = false, wide_used = false;
     int parity = 0;
     long long steps = 0;
     long long launches = 0;
@@ -408,6 +412,16 @@ void persist_grids(lb_handle* h, const std::vector<WorkItem>& items)
     }
 }
 
+// A single compact domain without obstacles may run two steps per launch and
+// pass over memory (launch_two_step).
+bool two_step(const lb_handle* h)
+{
+    const DomDesc& D = h->descs[0];
+    const int bx = h->block_x();
+    return h->n_dom == 1 && D.compact && !D.cls && h->sched.steps_per_launch == 2 &&
+           (bx == 64 || bx == 96 || bx == 128) && D.nx >= 8 && D.ny >= 8;
+}
+
 // Start order of the row bands of a single domain's launch (band_of in the
 // kernels).  About N = resident CTAs / strips bands are in flight at a time,
 // and a band reads its first rows when it starts and its last ones when it
@@ -424,9 +438,10 @@ int band_multiplier(const lb_handle* h)
     const DomDesc& D = h->descs[0];
     if (D.cls || h->n_dom != 1 || !D.compact) return 1;
     const int bx = h->block_x(), rows = h->rows();
-    const int w = D.compact ? lbfe::compact_strip(bx) : bx;
+    const int w = two_step(h) ? lbfe::two_step_strip(bx) : lbfe::compact_strip(bx);
     const long long strips = (D.nx + w - 1) / w, B = (D.ny + rows - 1) / rows;
-    const int occ = lbfe::step_single_occupancy(h->precision, h->coll, D.compact, bx);
+    const int occ = two_step(h) ? lbfe::two_step_occupancy(h->coll, bx)
+                                : lbfe::step_single_occupancy(h->precision, h->coll, D.compact, bx);
     const long long L = 3LL * occ * h->sm_count / (4 * std::max(strips, 1LL));
     if (L < 2 || B <= L + 1) return 1;
     for (long long l = L | 1; l < B; l += 2) {
@@ -516,6 +531,42 @@ int build_items(lb_handle* h)
     }
     LB_CUDA(cudaStreamSynchronize(h->stream));
     return LB_OK;
+}
+
+// Large single domains with compact storage, bound by memory, take two steps
+// per launch (lb_step_compact2.cuh).  A tile of R rows takes about R + 9
+// iterations, so among one to eight equal waves of CTAs the shape with the
+// fewest iterations over all waves is taken, up to 160 rows (more lose the
+// shared rows between bands in L2), 64-wide CTAs counted 7 % dearer (their
+// halo columns).  Measured, us per step, one step per launch and two: 700^2
+// 13.9 and 12.7, 1024^2 25.3 and 23.0, 2048^2 79.7 and 67.6, 4096^2 272 and
+// 236, 8192^2 1035 and 880; but 1000 x 500 13.8 and 14.4, and 160 x 5000, whose
+// strips are a third empty, 20.4 and 21.8.
+bool two_step_shape(const lb_handle* h, lb_schedule& s)
+{
+    const DomDesc& D = h->descs[0];
+    if (h->n_dom != 1 || !D.compact || D.cls || D.nx < 8 || D.ny < 8 ||
+        (long long)D.nx * D.ny < 600000)
+        return false;
+    double best = 1e300;
+    for (int bx : {128, 64}) {
+        const int w = lbfe::two_step_strip(bx);
+        const long long strips = (D.nx + w - 1) / w;
+        const long long wave = (long long)lbfe::two_step_occupancy(h->coll, bx) * h->sm_count;
+        if (D.nx < 0.75 * double(strips) * w) continue;
+        for (int waves = 1; waves <= 8; ++waves) {
+            const long long bands = waves * wave / strips;
+            if (bands < 1) continue;
+            const int rows = int((D.ny + bands - 1) / bands);
+            const double cost = waves * (rows + 9.0) * (bx == 64 ? 1.07 : 1.0);
+            if (rows < 6 || rows > 160 || cost >= best) continue;
+            best = cost;
+            s.steps_per_launch = 2;
+            s.block_x[0] = bx;
+            s.rows[0] = rows;
+        }
+    }
+    return best < 1e300;
 }
 
 // The schedule a handle starts with (lb_autotune times others): one class,
@@ -622,6 +673,7 @@ lb_schedule default_schedule(const lb_handle* h)
     }
     s.order = !single && (one_wave || fp64);
     s.chains = 1;
+    two_step_shape(h, s);
     return s;
 }
 
@@ -752,7 +804,46 @@ bool geo_fused(const lb_handle* h)
 }
 
 // Buffer flips of `len` steps (a two-step launch flips once).
-int buffer_flips(const lb_handle* h, int len) { return geo_fused(h) ? len / 2 + (len & 1) : len; }
+int buffer_flips(const lb_handle* h, int len)
+{
+    return geo_fused(h) || two_step(h) ? len / 2 + (len & 1) : len;
+}
+
+int launch_pair(lb_handle* h, int parity, cudaStream_t s)
+{
+    const int e = lbfe::launch_two_step(h->coll, h->descs[0], parity, h->block_x(), h->rows(),
+                                        h->band_mul, s);
+    if (e != 0)
+        return fail(LB_ERR_CUDA, "two-step launch failed: %s", cudaGetErrorString(cudaError_t(e)));
+    return LB_OK;
+}
+
+// Four-wide ghost columns of the current buffer, as two-step launches read
+// them.
+int widen_ghosts(lb_handle* h)
+{
+    if (h->wide_ok) return LB_OK;
+    int e = lbfe::launch_fill_ghosts(h->precision, h->descs[0], h->parity, h->stream);
+    if (e == 0) e = lbfe::launch_wide_ghosts(h->descs[0], h->parity, false, h->stream);
+    if (e != 0) return fail(LB_ERR_CUDA, "ghost fill failed: %s", cudaGetErrorString(cudaError_t(e)));
+    h->launches += 2;
+    h->wide_ok = h->wide_used = true;
+    return LB_OK;
+}
+
+// The outer ghost columns of both buffers back to zeros.
+int narrow_ghosts(lb_handle* h)
+{
+    h->wide_ok = false;
+    if (!h->wide_used) return LB_OK;
+    for (int b = 0; b < 2; ++b) {
+        const int e = lbfe::launch_wide_ghosts(h->descs[0], b, true, h->stream);
+        if (e != 0) return fail(LB_ERR_CUDA, "ghost reset failed: %s", cudaGetErrorString(cudaError_t(e)));
+        h->launches += 1;
+    }
+    h->wide_used = false;
+    return LB_OK;
+}
 
 // `len` steps of every domain with obstacles on `s`.
 int enqueue_geo_steps(lb_handle* h, int len, int parity, bool fixed_parity, cudaStream_t s)
@@ -839,6 +930,7 @@ long long launches_for(const lb_handle* h, int len)
     long long geo = 0;
     for (const DomDesc& D : h->descs)
         if (D.cls) geo += geo_persistent(h, D) ? 1 : (geo_fused(h) ? len / 2 + (len & 1) : len);
+    if (two_step(h)) return len / 2 + (len & 1);
     if (!persistent(h)) return len * (launches_per_step(h) - h->n_geo) + geo;
     return active_classes(h) + geo;
 }
@@ -871,6 +963,15 @@ int enqueue_steps(lb_handle* h, int len, int parity, bool fixed_parity, cudaStre
         return enqueue_geo_steps(h, len, parity, fixed_parity, s);
     }
     if (!(h->sched.chains && active_classes(h) > 1)) {
+        if (two_step(h)) {
+            // pairs of steps, then a single one for an odd count
+            const int pairs = len / 2;
+            for (int k = 0; k < pairs; ++k) {
+                const int rc = launch_pair(h, par(k), s);
+                if (rc != LB_OK) return rc;
+            }
+            return (len & 1) ? enqueue_step(h, par(pairs), s) : LB_OK;
+        }
         // a single domain with obstacles: its steps, maybe in one launch
         if (h->n_dom == 1 && h->descs[0].cls) return enqueue_geo_steps(h, len, parity, fixed_parity, s);
         for (int k = 0; k < len; ++k) {
@@ -961,6 +1062,8 @@ int get_graph(lb_handle* h, int len, int parity, cudaGraphExec_t* out)
 // the columns they copy (see lb_handle::ghosts_stale).
 int refresh_ghosts(lb_handle* h)
 {
+    const int rn = narrow_ghosts(h);
+    if (rn != LB_OK) return rn;
     if (!h->ghosts_stale) return LB_OK;
     for (const DomDesc& D : h->descs) {
         if (D.cls) continue;
@@ -1026,7 +1129,8 @@ int finish_init(lb_handle* h, int dom)
     // every domain of a handle shares one parity; the new state goes to the
     // current buffer, phi0 sat in the other one
     const DomDesc& D = h->descs[dom];
-    int e;
+    int e = narrow_ghosts(h);
+    if (e != LB_OK) return e;
     // phi0 is consumed once the equilibria are written: clear its scratch, so
     // that the idle buffer's padding columns, which no step reads and only
     // sealing whole-domain strips overwrite (with zeros), hold zeros whatever
@@ -1102,6 +1206,7 @@ int make_handle(const lb_params* per_dom, const int* nx, const int* ny, int n_do
         return rc;
     };
     if ((e = cudaError_t(lbfe::prepare_step_kernels())) != cudaSuccess ||
+        (e = cudaError_t(lbfe::prepare_two_step())) != cudaSuccess ||
         (e = cudaError_t(lbfe::prepare_geo_step2())) != cudaSuccess)
         return bail(fail(LB_ERR_CUDA, "kernel setup failed: %s", cudaGetErrorString(e)));
     if ((e = cudaDeviceGetAttribute(&h->sm_count, cudaDevAttrMultiProcessorCount, h->device)) !=
@@ -1490,6 +1595,10 @@ int lb_step(lb_handle* h, int n)
     if (use_device(h) != LB_OK) return LB_ERR_CUDA;
     if (n > 0 && h->descs[0].compact) h->ghosts_stale = true;
     bool pairs = false;  // the remainder goes by graphs of two
+    if (n >= 2 && two_step(h)) {
+        const int rc = widen_ghosts(h);
+        if (rc != LB_OK) return rc;
+    }
     while (n > 0) {
         const int len = pairs ? std::min(n, kGraphSmall) : next_length(h, n);
         pairs = pairs || len == kGraphSmall;
@@ -1503,6 +1612,7 @@ int lb_step(lb_handle* h, int n)
             LB_CUDA(cudaGraphLaunch(g, h->stream));
         }
         if (buffer_flips(h, len) & 1) h->parity ^= 1;
+        if (len & 1) h->wide_ok = false;  // a single step wrote this buffer
         h->steps += len;
         h->launches += launches_for(h, len);
         n -= len;
@@ -1947,7 +2057,7 @@ int lb_load_state(lb_handle* h, const void* host_buf, size_t bytes)
     }
     LB_CUDA(cudaStreamSynchronize(h->stream));
     h->steps = hdr[3];
-    h->ghosts_stale = false;
+    h->ghosts_stale = h->wide_ok = false;
     return LB_OK;
 }
 
@@ -1958,6 +2068,11 @@ int lb_set_tile(lb_handle* h, int block_x, int rows)
     sc.n_class = 1;
     sc.block_x[0] = block_x;
     sc.rows[0] = rows;
+    // a large compact domain keeps two steps per launch with rows enough to
+    // carry their lead-in, and takes one with fewer
+    lb_schedule two{};
+    if (h->n_dom == 1 && h->descs[0].compact)
+        sc.steps_per_launch = rows >= 48 && two_step_shape(h, two) ? 2 : 1;
     return lb_set_schedule(h, &sc);
 }
 
@@ -2158,18 +2273,31 @@ int lb_autotune(lb_handle* h, int reps, int* block_x, int* rows, double* best_ms
         // compact storage: two columns per thread, so half the threads per
         // strip, and strips up to nine compute warps wide (a domain that fits
         // one strip wraps in shared memory)
-        const std::vector<int> bxs =
+        std::vector<int> bxs =
             h->descs[0].compact ? std::vector<int>{32, 64, 96, 128, 160, 192, 224, 256, 288}
                                 : std::vector<int>{64, 128, 256};
-        const int rws[] = {4, 8, 16, 32, 64, 128};
+        std::vector<int> rws = {4, 8, 16, 32, 64, 128};
         // the shape by size, and the small-lattice step where that is the rule
         lb_schedule def = h->sched;
+        const lb_schedule ds = default_schedule(h);
         def.n_class = 1;
-        def.block_x[0] = default_schedule(h).block_x[0];
-        def.rows[0] = default_schedule(h).rows[0];
+        def.block_x[0] = ds.block_x[0];
+        def.rows[0] = ds.rows[0];
+        if (h->descs[0].compact) def.steps_per_launch = ds.steps_per_launch;
         small = small_rows(h) > 0;
         if (small) cands.push_back(def);
         cands.push_back(def);
+        if (two_step_shape(h, def)) {
+            // and about it; of one step per launch only what a lattice of this
+            // size has come out with
+            for (int r : {def.rows[0] / 2, def.rows[0] * 3 / 4, def.rows[0] * 3 / 2}) {
+                lb_schedule s = def;
+                s.rows[0] = std::max(r, 6);
+                cands.push_back(s);
+            }
+            bxs = {64, 96, 128};
+            rws = {4, 8, 16, 32};
+        }
         for (int bx : bxs)
             for (int r : rws) {
                 if (r > max_ny && r != rws[0]) continue;
@@ -2177,6 +2305,7 @@ int lb_autotune(lb_handle* h, int reps, int* block_x, int* rows, double* best_ms
                 s.n_class = 1;
                 s.block_x[0] = bx;
                 s.rows[0] = r;
+                if (h->descs[0].compact) s.steps_per_launch = 1;
                 cands.push_back(s);
             }
     }
@@ -2195,19 +2324,25 @@ int lb_autotune(lb_handle* h, int reps, int* block_x, int* rows, double* best_ms
     auto time_candidate = [&](size_t k, int len, int r) -> double {
         if ((rc = lb_set_schedule(h, &cands[k])) != LB_OK) return -1.0;
         if (small && k == 0) h->small_rows = small_rows(h);
+        // two steps per launch read four-wide ghost columns
+        if (two_step(h) && (rc = widen_ghosts(h)) != LB_OK) return -1.0;
         if (graphs) return time_graph_steps(h, len, r, e0, e1);
         // warm-up, then time `r` launches that read the current buffer and
         // write the idle one (the state itself does not advance)
-        if ((rc = enqueue_step(h, h->parity, h->stream)) != LB_OK) return -1.0;
+        auto launch = [&]() {
+            return two_step(h) ? launch_pair(h, h->parity, h->stream)
+                               : enqueue_step(h, h->parity, h->stream);
+        };
+        if ((rc = launch()) != LB_OK) return -1.0;
         cudaEventRecord(e0, h->stream);
-        for (int k = 0; k < r && rc == LB_OK; ++k) rc = enqueue_step(h, h->parity, h->stream);
+        for (int k = 0; k < r && rc == LB_OK; ++k) rc = launch();
         cudaEventRecord(e1, h->stream);
         if (rc != LB_OK) return -1.0;
         float t = 0.f;
         h->launches += (r + 1) * launches_per_step(h);
         if (cudaEventSynchronize(e1) != cudaSuccess || cudaEventElapsedTime(&t, e0, e1) != cudaSuccess)
             return -1.0;
-        return double(t) / r;
+        return double(t) / (two_step(h) ? 2 * r : r);
     };
     // a batch or a small lattice: graphs of 16 steps, so that chains and tails
     // show; then the fastest eight again over graphs of the length the steps run in (the

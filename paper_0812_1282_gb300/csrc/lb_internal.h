@@ -20,6 +20,10 @@ constexpr int kXOff = 4;
 // of 4 so that strips start on 16-byte boundaries.
 __host__ __device__ constexpr int compact_strip(int bx) { return (62 * (bx / 32) - 2) / 4 * 4; }
 
+// The same for two steps per pass over memory (lb_step_compact2.cuh), whose
+// strips need two more columns of the first step on each side; even.
+__host__ __device__ constexpr int two_step_strip(int bx) { return 62 * (bx / 32) - 6; }
+
 // One domain as the kernels see it.  Populations live in two ping-pong
 // buffers; buffer b holds f at f[b] and g at g[b], each 9 planes of
 // `plane` elements (pitch * ny, x fastest).
@@ -117,6 +121,18 @@ int launch_persist(int coll, const PersistLaunch& a, void* stream);
 int persist_occupancy(int coll, int block_x);
 int persist_footprint(int coll, int block_x, int* regs, size_t* smem);
 int prepare_persist();
+
+// Two steps of a single compact domain without obstacles in one launch: reads
+// buffer `parity`, whose periodic ghost columns must be four wide
+// (launch_wide_ghosts), and writes the other one with four-wide ghosts, which
+// then holds the state two steps on.  block_x: 64, 96 or 128.
+int launch_two_step(int coll, const DomDesc& d, int parity, int block_x, int rows, int band_mul,
+                    void* stream);
+int two_step_occupancy(int coll, int block_x);
+int prepare_two_step();
+// The outer two of four ghost columns per side: copies of the columns they
+// stand for, or (clear) the zeros they hold otherwise.
+int launch_wide_ghosts(const DomDesc& d, int parity, bool clear, void* stream);
 
 int launch_init_phi_drop(int precision, const DomDesc& d, double* phi0, double R, double cx,
                          double cy, void* stream);
