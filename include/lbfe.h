@@ -282,9 +282,9 @@ int lb_load_state(lb_handle* h, const void* host_buf, size_t bytes);
  * through (rows >= 1).  Results do not
  * depend on it.  On a batch it sets a one-class schedule with that shape
  * (lb_schedule).  Invalidates captured graphs.  A handle starts with a shape
- * chosen from its domains' sizes; a small single domain starts with a step
- * made for small lattices, for which the shape here is the one the general
- * step would take (setting a shape selects the general step).  On a large
+ * chosen from its domains' sizes; a small single domain or batch starts with a
+ * step made for small lattices, for which the shape here is the one the
+ * general step would take (setting a shape selects the general step).  On a large
  * single domain with compact storage a shape of at least 48 rows keeps two
  * steps per launch (lb_schedule), one of fewer rows takes one. */
 int lb_set_tile(lb_handle* h, int block_x, int rows);

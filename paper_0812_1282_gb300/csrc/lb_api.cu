@@ -216,8 +216,8 @@ struct lb_handle {
     cudaEvent_t fork_ev = nullptr;
     cudaEvent_t join_ev[LB_MAX_SCHED_CLASSES - 1] = {nullptr};
     int n_items = 0;
-    // single domain without obstacles: rows per tile of the small-lattice step
-    // (0: the staged one, whose shape `sched` holds either way)
+    // domains without obstacles: rows per tile of the small-lattice step (0: the
+    // staged one, whose shape `sched` holds either way)
     int small_rows = 0;
     // persistent schedules: CTAs of each class's launch
     int pgrid[LB_MAX_SCHED_CLASSES] = {0};
@@ -469,6 +469,11 @@ int build_items(lb_handle* h)
     for (int c = 0; c < LB_MAX_SCHED_CLASSES; ++c) h->cls_begin[c] = h->cls_count[c] = 0;
     if (h->n_dom == 1) {
         h->n_items = 0;
+        if (two_step(h)) {
+            const cudaError_t e = cudaError_t(lbfe::prepare_two_step());
+            if (e != cudaSuccess)
+                return fail(LB_ERR_CUDA, "kernel setup failed: %s", cudaGetErrorString(e));
+        }
         h->band_mul = band_multiplier(h);
         return LB_OK;
     }
@@ -479,6 +484,12 @@ int build_items(lb_handle* h)
         for (int d = 0; d < h->n_dom; ++d) {
             const DomDesc& D = h->descs[d];
             if (D.cls || class_of(h, D.nx) != c) continue;  // obstacles: their own kernels
+            if (h->small_rows > 0) {  // the tiles of the small-lattice step
+                for (int y0 = 0; y0 < D.ny; y0 += h->small_rows)
+                    for (int x0 = 0; x0 < D.nx; x0 += 32)
+                        mine.push_back(WorkItem{d, x0, y0, h->small_rows, 0, 0});
+                continue;
+            }
             if (D.compact) {
                 // the compact step's strips leave room for four halo columns; a
                 // domain is cut into near-equal strips (multiples of 4 columns,
@@ -498,7 +509,7 @@ int build_items(lb_handle* h)
                 for (int x0 = 0; x0 < D.nx; x0 += bx)
                     mine.push_back(WorkItem{d, x0, y0, std::min(rows, D.ny - y0), 0, 0});
         }
-        if (h->sched.order == 1) {
+        if (h->sched.order == 1 && h->small_rows == 0) {
             // largest first: nodes of the item (the full-storage strip is
             // bx wide, clipped to the domain)
             auto size = [&](const WorkItem& w) {
@@ -677,15 +688,18 @@ lb_schedule default_schedule(const lb_handle* h)
     return s;
 }
 
-// Rows per tile of the small-lattice step (lb_small.cu) where a single domain
-// should take it, 0 where the staged step is the faster one.  It is the
+// Rows per tile of the small-lattice step (lb_small.cu) where a handle should
+// take it, 0 where the staged step is the faster one.  It is the
 // faster one while the lattice is bound by latency, in FP64 also while it is
 // bound by the FP64 pipe and the tiles still fit the SMs evenly (us per step,
 // staged and small: FP32 28 x 15 4.0 and 2.5, 200 x 100 4.3 and 2.9, 1000 x 500
 // 15.4 and 13.8, 2000 x 350 20.7 and 20.0, but 900^2 24.4 and 27.4; compact
 // 28 x 15 4.5 and 3.5, 200 x 100 4.8 and 3.6, 512 x 256 7.2 and 5.9, but 700 x
 // 300 7.8 and 8.8; FP64 28 x 15 8.3 and 6.5, 200 x 100 11 and 7.5, 1000 x 500
-// 115 and 111, but 1200^2 313 and 302 to 317, 2048^2 828 and 850).
+// 115 and 111, but 1200^2 313 and 302 to 317, 2048^2 828 and 850).  In a batch
+// a tile first finds its domain, two loads in series: 6 domains of 22 k nodes
+// FP32 6.6 and 3.6, compact 7.7 and 4.3, FP64 14.3 and 11, 8 of 178 k 11.7 and
+// 8.0, 11.2 and 9.6, 60 and 47, but 40 of 623 k 28 and 27, 25 and 27, 165 and 165.
 //  - FP32: 4 rows (3 to 7 are within 5 %);
 //  - compact, whose tiles expand a two-node halo: the fewest rows from 4 on
 //    with which every tile has an SM to itself, else 7;
@@ -695,13 +709,19 @@ lb_schedule default_schedule(const lb_handle* h)
 //    5, 6, 7 rows: 8.2, 9.9, 7.4, 8.1, 9.0).
 int small_rows(const lb_handle* h)
 {
-    if (h->n_dom != 1) return 0;
-    const DomDesc& D = h->descs[0];
-    const bool fp64 = h->precision == LB_FP64;
-    const long long nodes = (long long)D.nx * D.ny;
-    if (nodes > (fp64 ? 800000 : (D.compact ? 140000 : 700000))) return 0;
-    auto tiles = [&](int rows) { return (long long)((D.nx + 31) / 32) * ((D.ny + rows - 1) / rows); };
-    if (D.compact) {
+    const bool fp64 = h->precision == LB_FP64, compact = h->descs[0].compact != 0;
+    long long nodes = 0;
+    for (const DomDesc& D : h->descs) nodes += (long long)D.nx * D.ny;
+    const long long most = h->n_dom > 1 ? (compact ? 200000 : 300000)
+                                        : (fp64 ? 800000 : (compact ? 140000 : 700000));
+    if (nodes > most) return 0;
+    auto tiles = [&](int rows) {
+        long long n = 0;
+        for (const DomDesc& D : h->descs)
+            n += (long long)((D.nx + 31) / 32) * ((D.ny + rows - 1) / rows);
+        return n;
+    };
+    if (compact) {
         for (int r = 4; r < 7; ++r)
             if (tiles(r) <= h->sm_count) return r;
         return 7;
@@ -736,10 +756,14 @@ int class_grid(const lb_handle* h, int c)
 // runs 1.7 % faster on the body built for its width, which it keeps).
 int launch_class(lb_handle* h, int c, int parity, cudaStream_t s)
 {
-    const int e = lbfe::launch_step(h->precision, h->coll, h->descs[0], h->d_descs(),
-                                    h->d_items() + h->cls_begin[c], h->cls_count[c], h->n_dom,
-                                    parity, h->sched.block_x[c], h->sched.rows[c], 1,
-                                    class_grid(h, c), h->d_sched(c), h->sched.n_class > 1, s);
+    const int e = h->small_rows > 0
+        ? lbfe::launch_small_step(h->precision, h->coll, h->descs[0], h->d_descs(),
+                                  h->d_items() + h->cls_begin[c], h->cls_count[c], parity,
+                                  h->small_rows, s)
+        : lbfe::launch_step(h->precision, h->coll, h->descs[0], h->d_descs(),
+                            h->d_items() + h->cls_begin[c], h->cls_count[c], h->n_dom, parity,
+                            h->sched.block_x[c], h->sched.rows[c], 1, class_grid(h, c),
+                            h->d_sched(c), h->sched.n_class > 1, s);
     if (e != 0)
         return fail(LB_ERR_CUDA, "step launch failed: %s", cudaGetErrorString(cudaError_t(e)));
     return LB_OK;
@@ -893,8 +917,8 @@ int enqueue_step(lb_handle* h, int parity, cudaStream_t s)
 {
     if (h->n_dom == 1) {
         if (h->descs[0].cls == nullptr && h->small_rows > 0) {
-            const int e = lbfe::launch_small_step(h->precision, h->coll, h->descs[0], parity,
-                                                  h->small_rows, s);
+            const int e = lbfe::launch_small_step(h->precision, h->coll, h->descs[0], nullptr, nullptr,
+                                                  0, parity, h->small_rows, s);
             if (e != 0)
                 return fail(LB_ERR_CUDA, "step launch failed: %s", cudaGetErrorString(cudaError_t(e)));
         } else if (h->descs[0].cls == nullptr) {
@@ -1206,7 +1230,6 @@ int make_handle(const lb_params* per_dom, const int* nx, const int* ny, int n_do
         return rc;
     };
     if ((e = cudaError_t(lbfe::prepare_step_kernels())) != cudaSuccess ||
-        (e = cudaError_t(lbfe::prepare_two_step())) != cudaSuccess ||
         (e = cudaError_t(lbfe::prepare_geo_step2())) != cudaSuccess)
         return bail(fail(LB_ERR_CUDA, "kernel setup failed: %s", cudaGetErrorString(e)));
     if ((e = cudaDeviceGetAttribute(&h->sm_count, cudaDevAttrMultiProcessorCount, h->device)) !=
@@ -2269,6 +2292,8 @@ int lb_autotune(lb_handle* h, int reps, int* block_x, int* rows, double* best_ms
         }
     } else if (h->n_dom > 1) {
         cands = batch_candidates(h);
+        small = small_rows(h) > 0;
+        if (small) cands.insert(cands.begin(), cands.front());
     } else {
         // compact storage: two columns per thread, so half the threads per
         // strip, and strips up to nine compute warps wide (a domain that fits
@@ -2314,6 +2339,10 @@ int lb_autotune(lb_handle* h, int reps, int* block_x, int* rows, double* best_ms
     LB_CUDA(cudaEventCreate(&e1));
     const lb_schedule old = h->sched;
     const int old_small = h->small_rows;
+    auto use_small = [&](int tile_rows) -> int {
+        h->small_rows = tile_rows;
+        return tile_rows > 0 && h->n_dom > 1 ? build_items(h) : LB_OK;
+    };
     double best = 1e300;
     lb_schedule chosen = old;
     int chosen_small = old_small, rc = LB_OK;
@@ -2323,7 +2352,7 @@ int lb_autotune(lb_handle* h, int reps, int* block_x, int* rows, double* best_ms
     // one timing of candidate k (ms per step); negative on failure
     auto time_candidate = [&](size_t k, int len, int r) -> double {
         if ((rc = lb_set_schedule(h, &cands[k])) != LB_OK) return -1.0;
-        if (small && k == 0) h->small_rows = small_rows(h);
+        if (small && k == 0 && (rc = use_small(small_rows(h))) != LB_OK) return -1.0;
         // two steps per launch read four-wide ghost columns
         if (two_step(h) && (rc = widen_ghosts(h)) != LB_OK) return -1.0;
         if (graphs) return time_graph_steps(h, len, r, e0, e1);
@@ -2379,9 +2408,10 @@ int lb_autotune(lb_handle* h, int reps, int* block_x, int* rows, double* best_ms
     cudaEventDestroy(e1);
     if (rc == LB_OK) rc = sync_and_check(h);
     const int rc2 = lb_set_schedule(h, rc == LB_OK ? &chosen : &old);
-    h->small_rows = rc == LB_OK ? chosen_small : old_small;
+    const int rc3 = use_small(rc == LB_OK ? chosen_small : old_small);
     if (rc != LB_OK) return rc;
     if (rc2 != LB_OK) return rc2;
+    if (rc3 != LB_OK) return rc3;
     if (block_x) *block_x = h->block_x();
     if (rows) *rows = h->rows();
     if (best_ms) *best_ms = best;

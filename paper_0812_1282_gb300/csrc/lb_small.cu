@@ -38,9 +38,8 @@ constexpr int kEW = kTX + 4;     // g' array (compact): two
 // The tile of a CTA: node columns [x0, x0 + wc), rows [y0, y0 + hc).
 struct SmallTile {
     int x0, y0, wc, hc;
-    __device__ __forceinline__ SmallTile(const DomDesc& D, int ty)
-        : x0(int(blockIdx.x) * kTX), y0(int(blockIdx.y) * ty), wc(min(kTX, D.nx - x0)),
-          hc(min(ty, D.ny - y0))
+    __device__ __forceinline__ SmallTile(const DomDesc& D, int x0_, int y0_, int ty)
+        : x0(x0_), y0(y0_), wc(min(kTX, D.nx - x0)), hc(min(ty, D.ny - y0))
     {
     }
 };
@@ -96,15 +95,19 @@ __device__ __forceinline__ bool halo_at(int k, const SmallTile& T, bool walls, i
 
 // Full storage.  blockDim.x = 32 TY (a multiple of a warp; every thread has
 // at most a node of its own); phi: (TY + 2) x 34 values of shared memory.
-template <typename Real, bool MRT>
-__global__ void __launch_bounds__(kSmallMaxThreads) small_step_kernel(DomDesc D, int parity)
+// PRM_SMEM (FP32, a batch): the node parameters are read from shared memory at
+// each use, as in the staged batch kernel, which keeps the bits of its BGK
+// collision (the compiler fuses other products there than with parameters in
+// registers).
+template <typename Real, bool MRT, bool PRM_SMEM>
+__device__ __forceinline__ void small_step(const DomDesc& D, int parity, const SmallTile& T)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     Real* ph = reinterpret_cast<Real*>(smem);
     __shared__ Node64 C;     // FP64 only
     __shared__ Real wet[2];  // wetting gradients, bottom and top
+    __shared__ NodeParams<Real> tile_prm;  // PRM_SMEM only
     const int TY = int(blockDim.x) / kTX;
-    const SmallTile T(D, TY);
     const int nx = D.nx, ny = D.ny, pitch = D.pitch, P = int(D.plane);
     const bool walls = D.walls != 0;
     const Real* __restrict__ fs = static_cast<const Real*>(parity ? D.f[1] : D.f[0]);
@@ -148,6 +151,7 @@ __global__ void __launch_bounds__(kSmallMaxThreads) small_step_kernel(DomDesc D,
         if (halo) pull9<Real>(gs, P, pitch, ny, walls, T.x0 + hx, row(T.y0 + hy), gh);
     }
     if (tid < 2) wet[tid] = wv;
+    if (PRM_SMEM && tid == 0) tile_prm = node_params<Real>(D);
     __syncthreads();
     if (!live) return;
     const bool blo = walls && y == 0, bhi = walls && y == ny - 1;
@@ -212,7 +216,12 @@ __global__ void __launch_bounds__(kSmallMaxThreads) small_step_kernel(DomDesc D,
             for (int j = 0; j < 3; ++j) s[j] = s[j] - h2;
         }
         stencils<Real>(c, r0[1], r0[-1], n[1], s[1], n[2], n[0], s[2], s[0], dx, dy, lap);
-        collide<Real, MRT>(prm, f, g, c, dx, dy, lap, s2, D.step2_relax_j != 0, fo, go);
+        if constexpr (PRM_SMEM) {
+            const volatile NodeParams<Real>& PV = tile_prm;
+            collide<Real, MRT>(PV, f, g, c, dx, dy, lap, s2, D.step2_relax_j != 0, fo, go);
+        } else {
+            collide<Real, MRT>(prm, f, g, c, dx, dy, lap, s2, D.step2_relax_j != 0, fo, go);
+        }
     }
     Real* __restrict__ fd = static_cast<Real*>(parity ? D.f[0] : D.f[1]);
     Real* __restrict__ gd = static_cast<Real*>(parity ? D.g[0] : D.g[1]);
@@ -227,14 +236,13 @@ __global__ void __launch_bounds__(kSmallMaxThreads) small_step_kernel(DomDesc D,
 // Compact g storage.  Shared memory: nine values (g'_1..g'_8 and their sum)
 // and the phi word of (TY + 4) x 36 positions, then phi of (TY + 2) x 34.
 template <bool MRT>
-__global__ void __launch_bounds__(kSmallMaxThreads) small_compact_kernel(DomDesc D, int parity)
+__device__ __forceinline__ void small_compact_step(const DomDesc& D, int parity, const SmallTile& T)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     const int TY = int(blockDim.x) / kTX;
     const int ne = (TY + 4) * kEW;
     float* E = reinterpret_cast<float*>(smem);  // E[i * ne + position], i = 0: the sum, 9: the word
     float* ph = E + 10 * ne;
-    const SmallTile T(D, TY);
     const int nx = D.nx, ny = D.ny, pitch = D.pitch, P = int(D.plane);
     const bool walls = D.walls != 0;
     const float* __restrict__ fs = static_cast<const float*>(parity ? D.f[1] : D.f[0]);
@@ -330,30 +338,81 @@ __global__ void __launch_bounds__(kSmallMaxThreads) small_compact_kernel(DomDesc
     store_ghosts(cd + 3 * P, o, x, nx, uy.lane(0));
 }
 
-template <bool MRT>
-cudaError_t launch_t(int precision, const DomDesc& d, int parity, int rows, cudaStream_t s)
+// How a tile is stored: FP64, FP32, or FP32 with compact g.
+enum class SmallKind { F64, F32, Compact };
+
+template <SmallKind K, bool MRT, bool BATCH>
+__device__ __forceinline__ void small_tile(const DomDesc& D, int parity, const SmallTile& T)
 {
-    const dim3 grid((d.nx + kTX - 1) / kTX, (d.ny + rows - 1) / rows);
-    const int threads = kTX * rows;
-    const size_t phi = size_t(rows + 2) * kPW;
-    if (precision != 0)
-        small_step_kernel<double, MRT><<<grid, threads, phi * 8, s>>>(d, parity);
-    else if (d.compact)
-        small_compact_kernel<MRT>
-            <<<grid, threads, (size_t(rows + 4) * kEW * 10 + phi) * 4, s>>>(d, parity);
+    if constexpr (K == SmallKind::F64)
+        small_step<double, MRT, false>(D, parity, T);
+    else if constexpr (K == SmallKind::F32)
+        small_step<float, MRT, BATCH>(D, parity, T);
     else
-        small_step_kernel<float, MRT><<<grid, threads, phi * 4, s>>>(d, parity);
+        small_compact_step<MRT>(D, parity, T);
+}
+
+template <SmallKind K, bool MRT>
+__global__ void __launch_bounds__(kSmallMaxThreads) small_step_kernel(DomDesc D, int parity)
+{
+    const int ty = int(blockDim.x) / kTX;
+    small_tile<K, MRT, false>(D, parity, SmallTile(D, int(blockIdx.x) * kTX, int(blockIdx.y) * ty, ty));
+}
+
+// Batch form: a CTA per work item (a tile of 32 columns x blockDim.x / 32
+// rows of one domain).
+template <SmallKind K, bool MRT>
+__global__ void __launch_bounds__(kSmallMaxThreads)
+    small_batch_kernel(const DomDesc* __restrict__ descs, const WorkItem* __restrict__ items,
+                       int parity)
+{
+    const WorkItem w = items[blockIdx.x];
+    const DomDesc& D = descs[w.dom];
+    small_tile<K, MRT, true>(D, parity, SmallTile(D, w.x0, w.y0, int(blockDim.x) / kTX));
+}
+
+size_t small_smem(SmallKind k, int rows)
+{
+    const size_t phi = size_t(rows + 2) * kPW;
+    return k == SmallKind::F64 ? phi * 8
+                               : (k == SmallKind::F32 ? phi * 4
+                                                      : (size_t(rows + 4) * kEW * 10 + phi) * 4);
+}
+
+template <SmallKind K, bool MRT>
+cudaError_t launch_t(const DomDesc& d, const DomDesc* descs, const WorkItem* items, int n_items,
+                     int parity, int rows, cudaStream_t s)
+{
+    const int threads = kTX * rows;
+    const size_t smem = small_smem(K, rows);
+    if (items)
+        small_batch_kernel<K, MRT><<<n_items, threads, smem, s>>>(descs, items, parity);
+    else
+        small_step_kernel<K, MRT>
+            <<<dim3((d.nx + kTX - 1) / kTX, (d.ny + rows - 1) / rows), threads, smem, s>>>(d, parity);
     return cudaGetLastError();
+}
+
+template <SmallKind K>
+cudaError_t launch_c(int coll, const DomDesc& d, const DomDesc* descs, const WorkItem* items,
+                     int n_items, int parity, int rows, cudaStream_t s)
+{
+    return coll ? launch_t<K, true>(d, descs, items, n_items, parity, rows, s)
+                : launch_t<K, false>(d, descs, items, n_items, parity, rows, s);
 }
 
 }  // namespace
 
-int launch_small_step(int precision, int coll, const DomDesc& d, int parity, int rows, void* stream)
+int launch_small_step(int precision, int coll, const DomDesc& d, const DomDesc* descs,
+                      const WorkItem* items, int n_items, int parity, int rows, void* stream)
 {
     if (rows < 1 || rows > kSmallMaxThreads / kTX) return int(cudaErrorInvalidValue);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    return int(coll ? launch_t<true>(precision, d, parity, rows, s)
-                    : launch_t<false>(precision, d, parity, rows, s));
+    if (precision != 0)
+        return int(launch_c<SmallKind::F64>(coll, d, descs, items, n_items, parity, rows, s));
+    if (d.compact)
+        return int(launch_c<SmallKind::Compact>(coll, d, descs, items, n_items, parity, rows, s));
+    return int(launch_c<SmallKind::F32>(coll, d, descs, items, n_items, parity, rows, s));
 }
 
 }  // namespace lbfe

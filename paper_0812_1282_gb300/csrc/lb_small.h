@@ -7,8 +7,10 @@ namespace lbfe {
 
 constexpr int kSmallMaxThreads = 256;
 
-// One step of a single domain without obstacles on tiles of 32 columns x
-// `rows` rows (1..8).
-int launch_small_step(int precision, int coll, const DomDesc& d, int parity, int rows, void* stream);
+// One step on tiles of 32 columns x `rows` rows (1..8), without obstacles: of
+// the single domain d (items NULL), or of the n_items tiles of a batch's list
+// (descs, items in device memory; d any of its domains).
+int launch_small_step(int precision, int coll, const DomDesc& d, const DomDesc* descs,
+                      const WorkItem* items, int n_items, int parity, int rows, void* stream);
 
 }  // namespace lbfe

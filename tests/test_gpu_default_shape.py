@@ -84,3 +84,39 @@ def test_small_lattice_step_is_bit_identical(lbf, storage, nx, ny, walls, rule, 
     for f, g, blob in out[1:]:
         assert np.array_equal(f, out[0][0]) and np.array_equal(g, out[0][1])
         assert blob == out[0][2]
+
+
+@pytest.mark.parametrize("storage", sorted(STORAGE))
+@pytest.mark.parametrize("collision,relax,walls,tau_phi", [("bgk", False, True, 1.0),
+                                                           ("mrt", True, True, 1.0),
+                                                           ("mrt", False, False, 1.0),
+                                                           ("bgk", False, False, 0.8),
+                                                           ("mrt", False, True, 1.3)])
+def test_small_batch_is_bit_identical(lbf, storage, collision, relax, walls, tau_phi):
+    """The step a small batch starts with against the staged one, domain by
+    domain with gradients of their own, and after a change of schedule and an
+    autotuned one."""
+    if storage == "compact" and tau_phi != 1.0:
+        pytest.skip("compact storage needs tau_phi = 1")
+    sizes = [(3, 3), (31, 6), (33, 5), (64, 4), (66, 29), (131, 8), (200, 61)]
+    plist = [lbf.params(collision=collision, tau_alpha=1.5, tau_beta=0.6 + 0.02 * k, walls=walls,
+                        tau_phi=tau_phi,
+                        h_bottom=0.02 * k, h_top=-0.01 * k, step2_relax_momentum=relax,
+                        **STORAGE[storage]) for k in range(len(sizes))]
+    out = []
+    for mode in ("staged", "small", "switch", "tuned"):
+        sim = lbf.Batch(plist, *zip(*sizes))
+        if mode == "staged":
+            sim.set_tile(64, 7)
+        for k in range(len(sizes)):
+            sim.init_random(0.4, 3 + k, dom=k)
+        if mode == "tuned":
+            sim.autotune(reps=1)
+        sim.step(9)
+        if mode == "switch":
+            sim.set_tile(96, 3)
+        sim.set_wetting(0.06, 0.03, dom=4)
+        sim.step(10)
+        out.append(sim.save_state())
+        sim.close()
+    assert out[1:] == out[:1] * 3
