@@ -695,7 +695,7 @@ lb_schedule default_schedule(const lb_handle* h)
 // staged and small: FP32 28 x 15 4.0 and 2.5, 200 x 100 4.3 and 2.9, 1000 x 500
 // 15.4 and 13.8, 2000 x 350 20.7 and 20.0, but 900^2 24.4 and 27.4; compact
 // 28 x 15 4.5 and 3.5, 200 x 100 4.8 and 3.6, 512 x 256 7.2 and 5.9, but 700 x
-// 300 7.8 and 8.8; FP64 28 x 15 8.3 and 6.5, 200 x 100 11 and 7.5, 1000 x 500
+// 300 7.8 and 8.8; FP64 28 x 15 8.3 and 5.1, 200 x 100 11 and 7.5, 1000 x 500
 // 115 and 111, but 1200^2 313 and 302 to 317, 2048^2 828 and 850).  In a batch
 // a tile first finds its domain, two loads in series: 6 domains of 22 k nodes
 // FP32 6.6 and 3.6, compact 7.7 and 4.3, FP64 14.3 and 11, 8 of 178 k 11.7 and
@@ -705,8 +705,12 @@ lb_schedule default_schedule(const lb_handle* h)
 //    with which every tile has an SM to itself, else 7;
 //  - FP64: a warp's operations take the pipe of its scheduler four times as
 //    long as the SM's, so up to four rows per SM cost the same and beyond that
-//    the SM with the most rows is the bound (200 x 100, us per step with 3, 4,
-//    5, 6, 7 rows: 8.2, 9.9, 7.4, 8.1, 9.0).
+//    the SM with the most rows is the bound (200 x 100, us per step with 4, 5,
+//    6, 7 rows: 9.9, 7.4, 8.1, 9.0).  With at most three rows per SM a node's
+//    work is split over two warps (us per step with 4 rows, one thread per
+//    node, and split with 1, 2, 3 rows: 100 x 50 6.6, 5.6, 5.2, 5.9; 128 x 96,
+//    156 tiles of 2 rows and 104 of 3, 6.7, 6.7, 6.9, 5.8; but 200 x 100 7.5
+//    and 8.9, 9.2, 9.1, 300 x 200 and larger a fifth to a third slower).
 int small_rows(const lb_handle* h)
 {
     const bool fp64 = h->precision == LB_FP64, compact = h->descs[0].compact != 0;
@@ -727,9 +731,11 @@ int small_rows(const lb_handle* h)
         return 7;
     }
     if (!fp64) return 4;
-    int best = 3;
+    for (int r = 2; r <= lbfe::kSmallSplitRows; ++r)
+        if (tiles(r) <= h->sm_count) return r;
+    int best = 4;
     double best_cost = 1e300;
-    for (int r = 3; r <= 7; ++r) {
+    for (int r = 4; r <= 7; ++r) {
         // rows on the fullest SM; a tile's halo costs about a quarter row
         const long long per_sm = (tiles(r) + h->sm_count - 1) / h->sm_count;
         const double cost = std::max(double(per_sm) * (r + 0.25), 4.25);

@@ -116,25 +116,27 @@ __device__ __forceinline__ double phi64(const Node64& C, const double (&g)[9])
                     g[8]);
 }
 
-// One node: pulled f (deviation form), phi and its scaled derivatives
-// X = s d_x phi, Y = s d_y phi, L = (s / 2) nabla^2 phi.  fo, go: the new
-// populations.  g (the pulled g) is read only for tau_phi != 1.
-// Step 2 (s2) takes u_eq = 0: its even velocity terms vanish with 1/rho set
-// to 0, and the odd coefficients alpha (axis) and beta (diagonal) become
-// those of the momentum rows' reading (MRT keeps j: 1/6; relaxing or BGK: 0).
-template <bool MRT, class G9>
-__device__ __forceinline__ void collide64(const Node64& C, const double (&f)[9], double phi,
-                                          double X, double Y, double L, bool s2, bool relax_j,
-                                          G9 g9, double (&fo)[9], double (&go)[9])
+// Step 1 (Eq. moments) at one node: from its pulled f (deviation form) the sums
+// s of opposite directions, rho - 1 and rho u; then, with phi, u and w = 1/tau.
+struct Moments64 {
+    double s1, s3, s5, s7, drho, jx, jy, w, ux, uy;
+};
+__device__ __forceinline__ void sums64(const Node64& C, const double (&f)[9], Moments64& m)
 {
-    // Step 1 (Eq. moments): sums and differences of opposite directions
-    const double s1 = LB64_ADD(f[1], f[2]), d1 = LB64_SUB(f[1], f[2]);
-    const double s3 = LB64_ADD(f[3], f[4]), d3 = LB64_SUB(f[3], f[4]);
-    const double s5 = LB64_ADD(f[5], f[6]), d5 = LB64_SUB(f[5], f[6]);
-    const double s7 = LB64_ADD(f[7], f[8]), d7 = LB64_SUB(f[7], f[8]);
-    const double drho = LB64_ADD(LB64_ADD(LB64_ADD(s1, s3), LB64_ADD(s5, s7)), f[0]);
-    const double jx = LB64_ADD(d1, LB64_SUB(d5, d7));
-    const double jy = LB64_ADD(d3, LB64_ADD(d5, d7));
+    m.s1 = LB64_ADD(f[1], f[2]);
+    m.s3 = LB64_ADD(f[3], f[4]);
+    m.s5 = LB64_ADD(f[5], f[6]);
+    m.s7 = LB64_ADD(f[7], f[8]);
+    const double d1 = LB64_SUB(f[1], f[2]), d3 = LB64_SUB(f[3], f[4]);
+    const double d5 = LB64_SUB(f[5], f[6]), d7 = LB64_SUB(f[7], f[8]);
+    m.drho = LB64_ADD(LB64_ADD(LB64_ADD(m.s1, m.s3), LB64_ADD(m.s5, m.s7)), f[0]);
+    m.jx = LB64_ADD(d1, LB64_SUB(d5, d7));
+    m.jy = LB64_ADD(d3, LB64_ADD(d5, d7));
+}
+// 1/rho and w from one reciprocal of rho tau.  Step 2 (s2) takes u_eq = 0, and
+// with it 1/rho = 0.
+__device__ __forceinline__ void velocity64(const Node64& C, double phi, bool s2, Moments64& m)
+{
     // Eq. (tau), or the nearest tabulated one (lookup table of Sec. V)
     double tau = __fma_rn(C.t1, phi, C.t0);
     if (C.lut_kmax > 0.0) {
@@ -142,33 +144,44 @@ __device__ __forceinline__ void collide64(const Node64& C, const double (&f)[9],
         tau = __fma_rn(k, C.lut_step, C.lut_lo);
     }
     // 1/rho = tau / (rho tau), w = 1/tau = rho / (rho tau)
-    const double r = rcp64(C, __fma_rn(tau, drho, tau));
-    const double w = __fma_rn(drho, r, r);
-    double irho = LB64_MUL(tau, r), alpha = C.c3, beta = C.c12;
-    if (s2) {
-        irho = 0.0;
-        alpha = beta = MRT && !relax_j ? 1.0 / 6.0 : 0.0;
-    }
-    const double ux = LB64_MUL(jx, irho), uy = LB64_MUL(jy, irho);
-    const double phi2 = LB64_MUL(phi, phi);
+    const double r = rcp64(C, __fma_rn(tau, m.drho, tau));
+    m.w = __fma_rn(m.drho, r, r);
+    const double irho = s2 ? 0.0 : LB64_MUL(tau, r);
+    m.ux = LB64_MUL(m.jx, irho);
+    m.uy = LB64_MUL(m.jy, irho);
+}
+
+// The new f of a node: phi and its scaled derivatives X = s d_x phi, Y = s d_y
+// phi, L = (s / 2) nabla^2 phi.  On Step-2 nodes the odd coefficients alpha
+// (axis) and beta (diagonal) are those of the momentum rows' reading (MRT
+// keeps j: 1/6; relaxing or BGK: 0).
+template <bool MRT>
+__device__ __forceinline__ void collide_f64(const Node64& C, const double (&f)[9],
+                                            const Moments64& m, double phi, double phi2, double X,
+                                            double Y, double L, bool s2, bool relax_j,
+                                            double (&fo)[9])
+{
+    const double alpha = s2 ? (MRT && !relax_j ? 1.0 / 6.0 : 0.0) : C.c3;
+    const double beta = s2 ? (MRT && !relax_j ? 1.0 / 6.0 : 0.0) : C.c12;
+    const double jx = m.jx, jy = m.jy, w = m.w;
     // A9: a ninth of 3 [p0 - kappa phi lap] - rho (Eq. p0 less the rest pressure)
     const double A9 =
         __fma_rn(phi, __fma_rn(phi, __fma_rn(C.qa, phi2, C.ma6), LB64_MUL(C.cl, L)),
-                 LB64_MUL(C.c9, drho));
+                 LB64_MUL(C.c9, m.drho));
     // rho u_a u_b and kappa d_a phi d_b phi: traces, and the two stress
     // moments of f^eq (rows 7, 8 of Eq. Matrix)
-    const double rxx = LB64_MUL(jx, ux), R = __fma_rn(jy, uy, rxx);
+    const double rxx = LB64_MUL(jx, m.ux), R = __fma_rn(jy, m.uy, rxx);
     const double kxx = LB64_MUL(X, X), K = __fma_rn(Y, Y, kxx);
     const double S = LB64_ADD(R, K);
     const double m7e = __fma_rn(C.two, LB64_ADD(rxx, kxx), -S);
-    const double m8e = __fma_rn(X, Y, LB64_MUL(jx, uy));
+    const double m8e = __fma_rn(X, Y, LB64_MUL(jx, m.uy));
     // even parts of the axis and the diagonal directions (Appendix A)
     const double Pe = __fma_rn(C.c12, S, A9);
     const double Qe = __fma_rn(C.q25, A9, __fma_rn(C.c12, R, LB64_MUL(C.m24, K)));
     const double jp = LB64_ADD(jx, jy), jm = LB64_SUB(jy, jx);
     if (MRT) {
         // Step 3: the stress moments relax at w, the others are at equilibrium
-        const double m7 = LB64_SUB(s1, s3), m8 = LB64_SUB(s5, s7);
+        const double m7 = LB64_SUB(m.s1, m.s3), m8 = LB64_SUB(m.s5, m.s7);
         const double n7 = __fma_rn(w, LB64_SUB(m7e, m7), m7);
         const double n8 = __fma_rn(w, LB64_SUB(m8e, m8), m8);
         const double Ex = __fma_rn(C.q25, n7, Pe), Ey = __fma_rn(-C.q25, n7, Pe);
@@ -181,7 +194,7 @@ __device__ __forceinline__ void collide64(const Node64& C, const double (&f)[9],
         fo[6] = __fma_rn(-beta, jp, Ed);
         fo[7] = __fma_rn(beta, jm, Ea);
         fo[8] = __fma_rn(-beta, jm, Ea);
-        fo[0] = __fma_rn(C.m4, LB64_ADD(Pe, Qe), drho);
+        fo[0] = __fma_rn(C.m4, LB64_ADD(Pe, Qe), m.drho);
     } else {
         // f' = (1 - w) f + w f^eq
         const double k = LB64_SUB(C.one, w), aw = LB64_MUL(alpha, w), bw = LB64_MUL(beta, w);
@@ -197,14 +210,21 @@ __device__ __forceinline__ void collide64(const Node64& C, const double (&f)[9],
         fo[6] = __fma_rn(k, f[6], __fma_rn(-bw, jp, wd));
         fo[7] = __fma_rn(k, f[7], __fma_rn(bw, jm, wa));
         fo[8] = __fma_rn(k, f[8], __fma_rn(-bw, jm, wa));
-        const double f0e = __fma_rn(C.m4, LB64_ADD(Pe, Qe), drho);
+        const double f0e = __fma_rn(C.m4, LB64_ADD(Pe, Qe), m.drho);
         fo[0] = __fma_rn(w, LB64_SUB(f0e, f[0]), f[0]);
     }
+}
+
+// The new g of a node.  g9 gives the pulled g, read only for tau_phi != 1.
+template <class G9>
+__device__ __forceinline__ void collide_g64(const Node64& C, const Moments64& m, double phi,
+                                            double phi2, double L, G9 g9, double (&go)[9])
+{
     // g^eq (Appendix A): a third of Gamma mu, then the velocity terms
     const double G3 = __fma_rn(phi, __fma_rn(C.ga, phi2, C.mga), LB64_MUL(C.gl, L));
-    const double pux = LB64_MUL(phi, ux), puy = LB64_MUL(phi, uy);
-    const double pxx = LB64_MUL(pux, ux), puu = __fma_rn(puy, uy, pxx);
-    const double pd = __fma_rn(C.two, pxx, -puu), pxy = LB64_MUL(pux, uy);
+    const double pux = LB64_MUL(phi, m.ux), puy = LB64_MUL(phi, m.uy);
+    const double pxx = LB64_MUL(pux, m.ux), puu = __fma_rn(puy, m.uy, pxx);
+    const double pd = __fma_rn(C.two, pxx, -puu), pxy = LB64_MUL(pux, m.uy);
     const double b = LB64_MUL(C.c12, puu);
     const double H = LB64_ADD(G3, b), D = __fma_rn(C.q25, G3, b);
     const double Gx = __fma_rn(C.q25, pd, H), Gy = __fma_rn(-C.q25, pd, H);
@@ -226,6 +246,20 @@ __device__ __forceinline__ void collide64(const Node64& C, const double (&f)[9],
 #pragma unroll
         for (int i = 0; i < 9; ++i) go[i] = __fma_rn(C.kg, g[i] - go[i], go[i]);
     }
+}
+
+// One node: both.
+template <bool MRT, class G9>
+__device__ __forceinline__ void collide64(const Node64& C, const double (&f)[9], double phi,
+                                          double X, double Y, double L, bool s2, bool relax_j,
+                                          G9 g9, double (&fo)[9], double (&go)[9])
+{
+    Moments64 m;
+    sums64(C, f, m);
+    velocity64(C, phi, s2, m);
+    const double phi2 = LB64_MUL(phi, phi);
+    collide_f64<MRT>(C, f, m, phi, phi2, X, Y, L, s2, relax_j, fo);
+    collide_g64(C, m, phi, phi2, L, g9, go);
 }
 
 }  // namespace lbfe

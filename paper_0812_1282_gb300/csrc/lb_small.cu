@@ -93,6 +93,41 @@ __device__ __forceinline__ bool halo_at(int k, const SmallTile& T, bool walls, i
     return hy < T.hc;
 }
 
+// FP64: the scaled derivatives (see collide64) of the node whose scaled phi is
+// *r0, from the phi array around it (ghost rows: DomDesc::wet_k).
+__device__ __forceinline__ void deriv64(const Node64& C, const DomDesc& D, const double* r0,
+                                        bool blo, bool bhi, const double* wet, double& X,
+                                        double& Y, double& L)
+{
+    struct Row {
+        double k, h, m;
+    };
+    auto row_of = [&](const double* r) {
+        Row v;
+        v.k = LB64_SUB(r[1], r[-1]);
+        v.h = LB64_ADD(r[1], r[-1]);
+        v.m = __fma_rn(C.four, r[0], v.h);
+        return v;
+    };
+    const Row cur = row_of(r0);
+    Row up = cur, dn = cur;
+    if (!bhi) up = row_of(r0 + kPW);
+    if (!blo) dn = row_of(r0 - kPW);
+    if (blo) {
+        const Row& v = D.wet_k == 2 ? up : cur;
+        dn.k = v.k;
+        dn.m = __dsub_rn(v.m, ghost_shift64(C.sig, D.wet_k, wet[0]));
+    }
+    if (bhi) {
+        const Row& v = D.wet_k == 2 ? dn : cur;
+        up.k = v.k;
+        up.m = __dsub_rn(v.m, ghost_shift64(C.sig, D.wet_k, wet[1]));
+    }
+    X = __fma_rn(C.four, cur.k, LB64_ADD(up.k, dn.k));
+    Y = LB64_SUB(up.m, dn.m);
+    L = __fma_rn(C.m20, r0[0], __fma_rn(C.four, cur.h, LB64_ADD(up.m, dn.m)));
+}
+
 // Full storage.  blockDim.x = 32 TY (a multiple of a warp; every thread has
 // at most a node of its own); phi: (TY + 2) x 34 values of shared memory.
 // PRM_SMEM (FP32, a batch): the node parameters are read from shared memory at
@@ -156,39 +191,11 @@ __device__ __forceinline__ void small_step(const DomDesc& D, int parity, const S
     if (!live) return;
     const bool blo = walls && y == 0, bhi = walls && y == ny - 1;
     const bool s2 = D.step2 && (blo || bhi);
-    // the row of a ghost row's phi: row k - 1 (ny - k), see DomDesc::wet_k
     const Real* r0 = ph + (ty + 1) * kPW + tx + 1;
-    const Real* rp = r0 + kPW;
-    const Real* rm = r0 - kPW;
     Real fo[9], go[9];
     if constexpr (sizeof(Real) == 8) {
-        struct Row {
-            double k, h, m;
-        };
-        auto row_of = [&](const double* r) {
-            Row v;
-            v.k = LB64_SUB(r[1], r[-1]);
-            v.h = LB64_ADD(r[1], r[-1]);
-            v.m = __fma_rn(C.four, r[0], v.h);
-            return v;
-        };
-        const Row cur = row_of(r0);
-        Row up = cur, dn = cur;
-        if (!bhi) up = row_of(rp);
-        if (!blo) dn = row_of(rm);
-        if (blo) {
-            const Row& v = D.wet_k == 2 ? up : cur;
-            dn.k = v.k;
-            dn.m = __dsub_rn(v.m, ghost_shift64(C.sig, D.wet_k, wet[0]));
-        }
-        if (bhi) {
-            const Row& v = D.wet_k == 2 ? dn : cur;
-            up.k = v.k;
-            up.m = __dsub_rn(v.m, ghost_shift64(C.sig, D.wet_k, wet[1]));
-        }
-        const double X = __fma_rn(C.four, cur.k, LB64_ADD(up.k, dn.k));
-        const double Y = LB64_SUB(up.m, dn.m);
-        const double L = __fma_rn(C.m20, r0[0], __fma_rn(C.four, cur.h, LB64_ADD(up.m, dn.m)));
+        double X, Y, L;
+        deriv64(C, D, r0, blo, bhi, wet, X, Y, L);
         collide64<MRT>(C, f, c, X, Y, L, s2, D.step2_relax_j != 0,
                        [&](double (&v)[9]) {
 #pragma unroll
@@ -198,8 +205,9 @@ __device__ __forceinline__ void small_step(const DomDesc& D, int parity, const S
     } else {
         const NodeParams<Real> prm = node_params<Real>(D);
         Real dx, dy, lap, n[3], s[3];
-        const Real* gp = bhi ? r0 - (D.wet_k - 1) * kPW : rp;
-        const Real* gm = blo ? r0 + (D.wet_k - 1) * kPW : rm;
+        // the row of a ghost row's phi: row k - 1 (ny - k), see DomDesc::wet_k
+        const Real* gp = bhi ? r0 - (D.wet_k - 1) * kPW : r0 + kPW;
+        const Real* gm = blo ? r0 + (D.wet_k - 1) * kPW : r0 - kPW;
 #pragma unroll
         for (int j = 0; j < 3; ++j) {
             n[j] = gp[j - 1];
@@ -231,6 +239,100 @@ __device__ __forceinline__ void small_step(const DomDesc& D, int parity, const S
         store_ghosts(fd + i * P, o, x, nx, fo[i]);
         store_ghosts(gd + i * P, o, x, nx, go[i]);
     }
+}
+
+// FP64, two threads per node.  A warp's FP64 operation keeps the pipe of its
+// scheduler for 64 cycles, so a lattice with fewer warps of nodes than the GPU
+// has schedulers waits for one warp's 140 operations in series.  Here a warp
+// pulls f of 32 nodes and forms the new f, another pulls g and forms the new g;
+// phi, rho - 1 and rho u pass through shared memory.  The two do u and the
+// derivatives each for itself, so with warps enough for every scheduler one
+// thread per node is faster (lb_api.cu, small_rows).  100 x 50 6.60 -> 5.16 us a
+// step, BGK 6.86 -> 5.42; 128 x 96 6.66 -> 5.84.
+// blockDim.x = 64 TY: the f warps first.  Shared memory: phi as above, then the
+// exchanged values.
+template <bool MRT>
+__device__ __forceinline__ void small_split64(const DomDesc& D, int parity, const SmallTile& T)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    double* ph = reinterpret_cast<double*>(smem);
+    __shared__ Node64 C;
+    __shared__ double wet[2];  // wetting gradients, bottom and top
+    const int half = int(blockDim.x) / 2, TY = half / kTX;
+    double* ex = ph + (TY + 2) * kPW;  // drho, jx, jy, phi: ex[i * half + node]
+    const int nx = D.nx, ny = D.ny, pitch = D.pitch, P = int(D.plane);
+    const bool walls = D.walls != 0;
+    const double* __restrict__ fs = static_cast<const double*>(parity ? D.f[1] : D.f[0]);
+    const double* __restrict__ gs = static_cast<const double*>(parity ? D.g[1] : D.g[0]);
+    const int tid = int(threadIdx.x);
+    const bool is_g = tid >= half;
+    const int node = is_g ? tid - half : tid, tx = node % kTX, ty = node / kTX;
+    const int x = T.x0 + tx, y = T.y0 + ty;
+    const bool live = tx < T.wc && ty < T.hc;
+    // all loads of the thread's half node and of its halo position
+    double v[9], gh[9];
+    int hx = 0, hy = 0;
+    const int nh = 2 * kPW + 2 * TY;
+    int k = int(blockDim.x) - 1 - tid;
+    auto row = [&](int r) { return r < 0 ? r + ny : (r >= ny ? r - ny : r); };
+    bool halo = k < nh && halo_at(k, T, walls, ny, hx, hy);
+    if (live) pull9<double>(is_g ? gs : fs, P, pitch, ny, walls, x, y, v);
+    if (halo) pull9<double>(gs, P, pitch, ny, walls, T.x0 + hx, row(T.y0 + hy), gh);
+    const double wv =
+        tid == 0 ? wet_bottom<double>(D) : (tid == 1 ? wet_top<double>(D) : 0.0);
+    load_node64(C, D.c64, tid);
+    __syncthreads();
+    double c = 0.0;
+    Moments64 m;
+    if (live) {
+        if (is_g) {
+            c = phi64(C, v);
+            ph[(ty + 1) * kPW + tx + 1] = LB64_MUL(C.sig, c);
+            ex[3 * half + node] = c;
+        } else {
+            sums64(C, v, m);
+            ex[node] = m.drho;
+            ex[half + node] = m.jx;
+            ex[2 * half + node] = m.jy;
+        }
+    }
+    for (;;) {
+        if (halo) ph[(hy + 1) * kPW + hx + 1] = LB64_MUL(C.sig, phi64(C, gh));
+        k += int(blockDim.x);
+        if (k >= nh) break;
+        halo = halo_at(k, T, walls, ny, hx, hy);
+        if (halo) pull9<double>(gs, P, pitch, ny, walls, T.x0 + hx, row(T.y0 + hy), gh);
+    }
+    if (tid < 2) wet[tid] = wv;
+    __syncthreads();
+    if (!live) return;
+    const bool blo = walls && y == 0, bhi = walls && y == ny - 1;
+    const bool s2 = D.step2 && (blo || bhi);
+    const double* r0 = ph + (ty + 1) * kPW + tx + 1;
+    const int o = y * pitch + x + kXOff;
+    double X, Y, L, out[9];
+    if (is_g) {
+        m.drho = ex[node];
+        m.jx = ex[half + node];
+        m.jy = ex[2 * half + node];
+        velocity64(C, c, s2, m);
+        deriv64(C, D, r0, blo, bhi, wet, X, Y, L);
+        collide_g64(C, m, c, LB64_MUL(c, c), L,
+                    [&](double (&g)[9]) {
+#pragma unroll
+                        for (int i = 0; i < 9; ++i) g[i] = v[i];
+                    },
+                    out);
+    } else {
+        c = ex[3 * half + node];
+        velocity64(C, c, s2, m);
+        deriv64(C, D, r0, blo, bhi, wet, X, Y, L);
+        collide_f64<MRT>(C, v, m, c, LB64_MUL(c, c), X, Y, L, s2, D.step2_relax_j != 0, out);
+    }
+    double* __restrict__ dst = static_cast<double*>(is_g ? (parity ? D.g[0] : D.g[1])
+                                                         : (parity ? D.f[0] : D.f[1]));
+#pragma unroll
+    for (int i = 0; i < 9; ++i) store_ghosts(dst + i * P, o, x, nx, out[i]);
 }
 
 // Compact g storage.  Shared memory: nine values (g'_1..g'_8 and their sum)
@@ -338,14 +440,23 @@ __device__ __forceinline__ void small_compact_step(const DomDesc& D, int parity,
     store_ghosts(cd + 3 * P, o, x, nx, uy.lane(0));
 }
 
-// How a tile is stored: FP64, FP32, or FP32 with compact g.
-enum class SmallKind { F64, F32, Compact };
+// How a tile is stored: FP64, FP32, or FP32 with compact g; FP64 on two threads
+// per node.
+enum class SmallKind { F64, F32, Compact, Split64 };
+
+// threads per row of a tile
+__host__ __device__ constexpr int lane_threads(SmallKind k)
+{
+    return k == SmallKind::Split64 ? 2 * kTX : kTX;
+}
 
 template <SmallKind K, bool MRT, bool BATCH>
 __device__ __forceinline__ void small_tile(const DomDesc& D, int parity, const SmallTile& T)
 {
     if constexpr (K == SmallKind::F64)
         small_step<double, MRT, false>(D, parity, T);
+    else if constexpr (K == SmallKind::Split64)
+        small_split64<MRT>(D, parity, T);
     else if constexpr (K == SmallKind::F32)
         small_step<float, MRT, BATCH>(D, parity, T);
     else
@@ -355,7 +466,7 @@ __device__ __forceinline__ void small_tile(const DomDesc& D, int parity, const S
 template <SmallKind K, bool MRT>
 __global__ void __launch_bounds__(kSmallMaxThreads) small_step_kernel(DomDesc D, int parity)
 {
-    const int ty = int(blockDim.x) / kTX;
+    const int ty = int(blockDim.x) / lane_threads(K);
     small_tile<K, MRT, false>(D, parity, SmallTile(D, int(blockIdx.x) * kTX, int(blockIdx.y) * ty, ty));
 }
 
@@ -368,12 +479,13 @@ __global__ void __launch_bounds__(kSmallMaxThreads)
 {
     const WorkItem w = items[blockIdx.x];
     const DomDesc& D = descs[w.dom];
-    small_tile<K, MRT, true>(D, parity, SmallTile(D, w.x0, w.y0, int(blockDim.x) / kTX));
+    small_tile<K, MRT, true>(D, parity, SmallTile(D, w.x0, w.y0, int(blockDim.x) / lane_threads(K)));
 }
 
 size_t small_smem(SmallKind k, int rows)
 {
     const size_t phi = size_t(rows + 2) * kPW;
+    if (k == SmallKind::Split64) return (phi + size_t(rows) * kTX * 4) * 8;
     return k == SmallKind::F64 ? phi * 8
                                : (k == SmallKind::F32 ? phi * 4
                                                       : (size_t(rows + 4) * kEW * 10 + phi) * 4);
@@ -383,7 +495,7 @@ template <SmallKind K, bool MRT>
 cudaError_t launch_t(const DomDesc& d, const DomDesc* descs, const WorkItem* items, int n_items,
                      int parity, int rows, cudaStream_t s)
 {
-    const int threads = kTX * rows;
+    const int threads = lane_threads(K) * rows;
     const size_t smem = small_smem(K, rows);
     if (items)
         small_batch_kernel<K, MRT><<<n_items, threads, smem, s>>>(descs, items, parity);
@@ -408,6 +520,8 @@ int launch_small_step(int precision, int coll, const DomDesc& d, const DomDesc* 
 {
     if (rows < 1 || rows > kSmallMaxThreads / kTX) return int(cudaErrorInvalidValue);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
+    if (precision != 0 && rows <= kSmallSplitRows)
+        return int(launch_c<SmallKind::Split64>(coll, d, descs, items, n_items, parity, rows, s));
     if (precision != 0)
         return int(launch_c<SmallKind::F64>(coll, d, descs, items, n_items, parity, rows, s));
     if (d.compact)

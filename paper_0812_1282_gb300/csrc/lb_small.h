@@ -6,6 +6,8 @@
 namespace lbfe {
 
 constexpr int kSmallMaxThreads = 256;
+// FP64 tiles of at most this many rows run on two threads per node.
+constexpr int kSmallSplitRows = 3;
 
 // One step on tiles of 32 columns x `rows` rows (1..8), without obstacles: of
 // the single domain d (items NULL), or of the n_items tiles of a batch's list

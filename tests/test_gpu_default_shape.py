@@ -52,7 +52,8 @@ def test_default_shape_is_bit_identical(lbf, storage, sizes, walls):
 
 
 @pytest.mark.parametrize("storage", sorted(STORAGE))
-@pytest.mark.parametrize("nx,ny", [(3, 3), (4, 33), (31, 6), (33, 5), (66, 8), (131, 29)])
+@pytest.mark.parametrize("nx,ny", [(3, 3), (4, 33), (31, 6), (33, 5), (66, 8), (131, 29),
+                                   (131, 76), (203, 97)])
 @pytest.mark.parametrize("walls,rule", [(True, 0), (True, 1), (False, 0)])
 @pytest.mark.parametrize("collision,relax,lut,tau_phi", [("bgk", False, 0, 1.0), ("bgk", False, 0, 0.8),
                                                          ("mrt", False, 0, 1.0), ("mrt", True, 9, 1.0),
