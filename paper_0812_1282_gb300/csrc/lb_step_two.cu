@@ -17,20 +17,21 @@ cudaError_t launch_t(const DomDesc& d, int parity, int rows, int band_mul, cudaS
 }
 
 template <bool MRT, int NWC>
-int occupancy_t()
-{
-    int n = 0;
-    const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-        &n, step_two_compact_kernel<MRT, NWC>, 64 * NWC + 32, TwoStepLayout(NWC, kStagesTwo).total());
-    return e == cudaSuccess ? n : 0;
-}
-
-template <bool MRT, int NWC>
 cudaError_t prepare_t()
 {
     return cudaFuncSetAttribute(step_two_compact_kernel<MRT, NWC>,
                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 int(TwoStepLayout(NWC, kStagesTwo).total()));
+}
+
+template <bool MRT, int NWC>
+int occupancy_t()
+{
+    int n = 0;
+    if (prepare_t<MRT, NWC>() != cudaSuccess) return 0;  // else none fits
+    const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+        &n, step_two_compact_kernel<MRT, NWC>, 64 * NWC + 32, TwoStepLayout(NWC, kStagesTwo).total());
+    return e == cudaSuccess ? n : 0;
 }
 
 template <bool MRT>

@@ -3,6 +3,10 @@ steps_per_launch = 2) against one step per launch, bit for bit and byte for
 byte of the checkpoint: strips that end inside and at the domain's edge, tiles
 of a few rows and of the whole domain, walls and periodic rows, odd step
 counts, a new initial state and a loaded one in between."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 
@@ -106,3 +110,13 @@ def test_large_domain_starts_with_it(lbf):
     assert a.save_state() == b.save_state()
     a.close()
     b.close()
+
+
+def test_large_domain_starts_with_it_in_a_new_process(lbf):
+    """The rule asks for the kernel's occupancy before any two-step schedule was
+    set in the process."""
+    code = ("import paper_0812_1282_gb300 as lbf\n"
+            "p = lbf.params(precision='fp32', compact_g=True)\n"
+            "assert lbf.Lattice(p, 1210, 701).schedule()['steps_per_launch'] == 2\n")
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    subprocess.run([sys.executable, "-c", code], check=True, cwd=root, timeout=300)
