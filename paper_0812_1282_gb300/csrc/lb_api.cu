@@ -422,6 +422,42 @@ bool two_step(const lb_handle* h)
            (bx == 64 || bx == 96 || bx == 128) && D.nx >= 8 && D.ny >= 8;
 }
 
+// A small FP32 lattice takes several steps per launch (launch_small_steps):
+// their number (1: it does not) and the rows of a tile.  More steps save more
+// launches, and their tiles' borders cost more: four while tiles of at most
+// eight rows fit one per SM, then three, then two; two also with two such tiles
+// per SM.  Measured, us per step with 1, 2, 3, 4 steps at the best rows for
+// each: FP32 28 x 15 2.3, 1.6, 1.5, 1.4, 200 x 100 2.7, 2.0, 1.9, 1.8, 300 x
+// 100 2.7, 2.1, 2.5, 3.2, 320 x 200 3.6, 2.7, 4.1, 4.8, 500 x 200 4.2, 4.2, 5.4,
+// 7.4; compact 28 x 15 3.4, 2.0, 1.9, 1.9, 200 x 100 3.5, 2.5, 2.4, 2.3, 300 x
+// 100 3.4, 2.7, 3.7, 4.3, 320 x 200 4.2, 3.7, 6.2, 6.5.
+std::pair<int, int> small_steps(const lb_handle* h)
+{
+    const DomDesc& D = h->descs[0];
+    if (h->n_dom != 1 || h->small_rows == 0 || h->precision != LB_FP32 || D.cls || D.nx < 8 ||
+        D.ny < 8)
+        return {1, 0};
+    auto tiles = [&](int steps, int rows) {
+        const int w = lbfe::small_steps_cols(steps);
+        return (long long)((D.nx + w - 1) / w) * ((D.ny + rows - 1) / rows);
+    };
+    for (int steps = 4; steps >= 2; --steps)
+        for (int rows = 2; rows <= 8; ++rows)
+            if (tiles(steps, rows) <= h->sm_count) return {steps, rows};
+    if (tiles(2, 8) <= 2LL * h->sm_count) return {2, 8};
+    return {1, 0};
+}
+
+// Steps per launch of a single domain without obstacles.
+int single_steps(const lb_handle* h) { return two_step(h) ? 2 : small_steps(h).first; }
+
+// Launches, each with a flip of the buffer, of `len` steps of such a domain.
+int single_launches(const lb_handle* h, int len)
+{
+    const int k = single_steps(h);
+    return (len + k - 1) / k;
+}
+
 // Start order of the row bands of a single domain's launch (band_of in the
 // kernels).  About N = resident CTAs / strips bands are in flight at a time,
 // and a band reads its first rows when it starts and its last ones when it
@@ -836,15 +872,19 @@ bool geo_fused(const lb_handle* h)
 // Buffer flips of `len` steps (a two-step launch flips once).
 int buffer_flips(const lb_handle* h, int len)
 {
-    return geo_fused(h) || two_step(h) ? len / 2 + (len & 1) : len;
+    if (single_steps(h) > 1) return single_launches(h, len);
+    return geo_fused(h) ? len / 2 + (len & 1) : len;
 }
 
-int launch_pair(lb_handle* h, int parity, cudaStream_t s)
+// A launch of `steps` (2 .. single_steps) steps.
+int launch_several(lb_handle* h, int steps, int parity, cudaStream_t s)
 {
-    const int e = lbfe::launch_two_step(h->coll, h->descs[0], parity, h->block_x(), h->rows(),
-                                        h->band_mul, s);
+    const int e = two_step(h) ? lbfe::launch_two_step(h->coll, h->descs[0], parity, h->block_x(),
+                                                      h->rows(), h->band_mul, s)
+                              : lbfe::launch_small_steps(h->coll, h->descs[0], parity, steps,
+                                                         small_steps(h).second, s);
     if (e != 0)
-        return fail(LB_ERR_CUDA, "two-step launch failed: %s", cudaGetErrorString(cudaError_t(e)));
+        return fail(LB_ERR_CUDA, "step launch failed: %s", cudaGetErrorString(cudaError_t(e)));
     return LB_OK;
 }
 
@@ -960,7 +1000,7 @@ long long launches_for(const lb_handle* h, int len)
     long long geo = 0;
     for (const DomDesc& D : h->descs)
         if (D.cls) geo += geo_persistent(h, D) ? 1 : (geo_fused(h) ? len / 2 + (len & 1) : len);
-    if (two_step(h)) return len / 2 + (len & 1);
+    if (single_steps(h) > 1) return single_launches(h, len);
     if (!persistent(h)) return len * (launches_per_step(h) - h->n_geo) + geo;
     return active_classes(h) + geo;
 }
@@ -993,14 +1033,13 @@ int enqueue_steps(lb_handle* h, int len, int parity, bool fixed_parity, cudaStre
         return enqueue_geo_steps(h, len, parity, fixed_parity, s);
     }
     if (!(h->sched.chains && active_classes(h) > 1)) {
-        if (two_step(h)) {
-            // pairs of steps, then a single one for an odd count
-            const int pairs = len / 2;
-            for (int k = 0; k < pairs; ++k) {
-                const int rc = launch_pair(h, par(k), s);
+        if (const int m = single_steps(h); m > 1) {
+            for (int k = 0; len > 0; ++k, len -= m) {
+                const int rc = len > 1 ? launch_several(h, std::min(len, m), par(k), s)
+                                       : enqueue_step(h, par(k), s);
                 if (rc != LB_OK) return rc;
             }
-            return (len & 1) ? enqueue_step(h, par(pairs), s) : LB_OK;
+            return LB_OK;
         }
         // a single domain with obstacles: its steps, maybe in one launch
         if (h->n_dom == 1 && h->descs[0].cls) return enqueue_geo_steps(h, len, parity, fixed_parity, s);
@@ -2365,7 +2404,7 @@ int lb_autotune(lb_handle* h, int reps, int* block_x, int* rows, double* best_ms
         // warm-up, then time `r` launches that read the current buffer and
         // write the idle one (the state itself does not advance)
         auto launch = [&]() {
-            return two_step(h) ? launch_pair(h, h->parity, h->stream)
+            return two_step(h) ? launch_several(h, 2, h->parity, h->stream)
                                : enqueue_step(h, h->parity, h->stream);
         };
         if ((rc = launch()) != LB_OK) return -1.0;

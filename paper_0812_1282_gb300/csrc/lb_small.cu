@@ -1,5 +1,5 @@
-// Fused step of small lattices without obstacles: one launch per step, one
-// node per thread, plain loads.
+// Fused step of small lattices without obstacles: one node per thread, plain
+// loads; one step per launch, or several.
 //
 // A lattice whose CTAs all fit the GPU at once is bound by latency: a
 // dependent launch costs 0.6 us, a global load and a store 0.5 us more, and
@@ -16,6 +16,13 @@
 //    on the tile and a two-node halo, expands them to g' in shared memory;
 //    then phi(t+1) of the tile and a one-node halo is formed from the g' that
 //    arrive there; then the nodes collide.
+//  - the smallest: FP32 (both storages) takes up to four steps per launch,
+//    with a border of two nodes more per step around the tile (small_steps);
+//    FP64, bound by its pipe instead, splits a node over two threads
+//    (small_split64).
+// us a step, staged, one step per launch, and as here: FP32 28 x 15 4.0, 2.3, 1.4,
+// 200 x 100 4.4, 2.7, 1.8; compact 28 x 15 4.5, 3.4, 1.9, 200 x 100 4.9, 3.5, 2.3;
+// FP64 28 x 15 8.3, 6.6, 5.1, 200 x 100 11, 7.5.
 // The arithmetic is that of the staged kernels, operation for operation, and
 // so are the stored populations and ghost columns, bit for bit.
 #include <cuda_runtime.h>
@@ -66,6 +73,23 @@ __device__ __forceinline__ void pull9(const Real* __restrict__ src, int P, int p
     v[8] = src[bhi ? 7 * P + o : 8 * P + op - 1];
 }
 
+// The same from a step's result in shared memory: planes of SP values, rows of 32
+// columns, the node at o; its neighbours are in the array.
+__device__ __forceinline__ void pull_shared(const float* s, int SP, int o, bool blo, bool bhi,
+                                            float (&v)[9])
+{
+    const int om = o - kTX, op = o + kTX;
+    v[0] = s[o];
+    v[1] = s[SP + o - 1];
+    v[2] = s[2 * SP + o + 1];
+    v[3] = s[blo ? 4 * SP + o : 3 * SP + om];
+    v[4] = s[bhi ? 3 * SP + o : 4 * SP + op];
+    v[5] = s[blo ? 6 * SP + o : 5 * SP + om - 1];
+    v[6] = s[bhi ? 5 * SP + o : 6 * SP + op + 1];
+    v[7] = s[blo ? 8 * SP + o : 7 * SP + om + 1];
+    v[8] = s[bhi ? 7 * SP + o : 8 * SP + op - 1];
+}
+
 // Store one value of a plane at offset o and its periodic ghost copies:
 // logical columns 0, 1 also at nx, nx + 1 and nx - 2, nx - 1 also at -2, -1.
 template <typename Real>
@@ -76,21 +100,20 @@ __device__ __forceinline__ void store_ghosts(Real* __restrict__ p, int o, int x,
     if (x >= nx - 2) p[o - nx] = v;
 }
 
-// Position k of the one-node halo of a tile, relative to its first node;
-// false if the tile or the lattice has none there.
-__device__ __forceinline__ bool halo_at(int k, const SmallTile& T, bool walls, int ny, int& hx,
-                                        int& hy)
+// Position k of the one-node halo of w x h nodes (w at most 32), relative to the
+// first one: the two rows, then the two columns; false if there is none.
+__device__ __forceinline__ bool halo_at(int k, int w, int h, int& hx, int& hy)
 {
     if (k < 2 * kPW) {
         const bool low = k < kPW;
         hx = (low ? k : k - kPW) - 1;
-        hy = low ? -1 : T.hc;
-        return hx <= T.wc && !(walls && (low ? T.y0 == 0 : T.y0 + T.hc == ny));
+        hy = low ? -1 : h;
+        return hx <= w;
     }
     k -= 2 * kPW;
-    hx = (k & 1) ? T.wc : -1;
+    hx = (k & 1) ? w : -1;
     hy = k >> 1;
-    return hy < T.hc;
+    return hy < h;
 }
 
 // FP64: the scaled derivatives (see collide64) of the node whose scaled phi is
@@ -128,111 +151,95 @@ __device__ __forceinline__ void deriv64(const Node64& C, const DomDesc& D, const
     L = __fma_rn(C.m20, r0[0], __fma_rn(C.four, cur.h, LB64_ADD(up.m, dn.m)));
 }
 
-// Full storage.  blockDim.x = 32 TY (a multiple of a warp; every thread has
-// at most a node of its own); phi: (TY + 2) x 34 values of shared memory.
-// PRM_SMEM (FP32, a batch): the node parameters are read from shared memory at
-// each use, as in the staged batch kernel, which keeps the bits of its BGK
-// collision (the compiler fuses other products there than with parameters in
-// registers).
-template <typename Real, bool MRT, bool PRM_SMEM>
-__device__ __forceinline__ void small_step(const DomDesc& D, int parity, const SmallTile& T)
+// FP32: the derivatives of the node whose phi is c = *r0.
+__device__ __forceinline__ void deriv32(const DomDesc& D, const float* r0, float c, bool blo,
+                                        bool bhi, const float* wet, float& dx, float& dy,
+                                        float& lap)
+{
+    float n[3], s[3];
+    // the row of a ghost row's phi: row k - 1 (ny - k), see DomDesc::wet_k
+    const float* gp = bhi ? r0 - (D.wet_k - 1) * kPW : r0 + kPW;
+    const float* gm = blo ? r0 + (D.wet_k - 1) * kPW : r0 - kPW;
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+        n[j] = gp[j - 1];
+        s[j] = gm[j - 1];
+    }
+    if (bhi) {
+        const float h2 = float(D.wet_k) * wet[1];
+#pragma unroll
+        for (int j = 0; j < 3; ++j) n[j] = n[j] - h2;
+    }
+    if (blo) {
+        const float h2 = float(D.wet_k) * wet[0];
+#pragma unroll
+        for (int j = 0; j < 3; ++j) s[j] = s[j] - h2;
+    }
+    stencils<float>(c, r0[1], r0[-1], n[1], s[1], n[2], n[0], s[2], s[0], dx, dy, lap);
+}
+
+// FP64.  blockDim.x = 32 TY (every thread has at most a node of its own); phi,
+// scaled for the stencils (lb_step64.cuh): (TY + 2) x 34 values of shared memory.
+template <bool MRT>
+__device__ __forceinline__ void small_step64(const DomDesc& D, int parity, const SmallTile& T)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    Real* ph = reinterpret_cast<Real*>(smem);
-    __shared__ Node64 C;     // FP64 only
-    __shared__ Real wet[2];  // wetting gradients, bottom and top
-    __shared__ NodeParams<Real> tile_prm;  // PRM_SMEM only
+    double* ph = reinterpret_cast<double*>(smem);
+    __shared__ Node64 C;
+    __shared__ double wet[2];  // wetting gradients, bottom and top
     const int TY = int(blockDim.x) / kTX;
     const int nx = D.nx, ny = D.ny, pitch = D.pitch, P = int(D.plane);
     const bool walls = D.walls != 0;
-    const Real* __restrict__ fs = static_cast<const Real*>(parity ? D.f[1] : D.f[0]);
-    const Real* __restrict__ gs = static_cast<const Real*>(parity ? D.g[1] : D.g[0]);
+    const double* __restrict__ fs = static_cast<const double*>(parity ? D.f[1] : D.f[0]);
+    const double* __restrict__ gs = static_cast<const double*>(parity ? D.g[1] : D.g[0]);
     const int tid = int(threadIdx.x), tx = tid % kTX, ty = tid / kTX;
     const int x = T.x0 + tx, y = T.y0 + ty;
     const bool live = tx < T.wc && ty < T.hc;
     // all loads of the thread's node and of its halo position
-    Real f[9], g[9], gh[9];
+    double f[9], g[9], gh[9];
     int hx = 0, hy = 0;
     const int nh = 2 * kPW + 2 * TY;
     int k = int(blockDim.x) - 1 - tid;
     auto row = [&](int r) { return r < 0 ? r + ny : (r >= ny ? r - ny : r); };
-    bool halo = k < nh && halo_at(k, T, walls, ny, hx, hy);
-    if (live) pull9<Real>(gs, P, pitch, ny, walls, x, y, g);
-    if (halo) pull9<Real>(gs, P, pitch, ny, walls, T.x0 + hx, row(T.y0 + hy), gh);
-    if (live) pull9<Real>(fs, P, pitch, ny, walls, x, y, f);
+    auto inside = [&](int r) { return !walls || (r >= 0 && r < ny); };
+    bool halo = k < nh && halo_at(k, T.wc, T.hc, hx, hy) && inside(T.y0 + hy);
+    if (live) pull9<double>(gs, P, pitch, ny, walls, x, y, g);
+    if (halo) pull9<double>(gs, P, pitch, ny, walls, T.x0 + hx, row(T.y0 + hy), gh);
+    if (live) pull9<double>(fs, P, pitch, ny, walls, x, y, f);
     // the wetting gradients, in flight with the populations
-    const Real wv = tid == 0 ? wet_bottom<Real>(D) : (tid == 1 ? wet_top<Real>(D) : Real(0));
-    if constexpr (sizeof(Real) == 8) {
-        load_node64(C, D.c64, tid);
-        __syncthreads();
-    }
-    // the stored value: phi, in FP64 scaled for the stencils (lb_step64.cuh)
-    auto put = [&](int cx, int cy, const Real (&v)[9], Real& phi) {
-        if constexpr (sizeof(Real) == 8) {
-            phi = phi64(C, v);
-            ph[(cy + 1) * kPW + cx + 1] = LB64_MUL(C.sig, phi);
-        } else {
-            phi = phi_sum<Real>(v);
-            ph[(cy + 1) * kPW + cx + 1] = phi;
-        }
+    const double wv = tid == 0 ? wet_bottom<double>(D) : (tid == 1 ? wet_top<double>(D) : 0.0);
+    load_node64(C, D.c64, tid);
+    __syncthreads();
+    auto put = [&](int cx, int cy, const double (&v)[9], double& phi) {
+        phi = phi64(C, v);
+        ph[(cy + 1) * kPW + cx + 1] = LB64_MUL(C.sig, phi);
     };
-    Real c = Real(0), dump;
+    double c = 0.0, dump;
     if (live) put(tx, ty, g, c);
     for (;;) {
         if (halo) put(hx, hy, gh, dump);
         k += int(blockDim.x);
         if (k >= nh) break;
-        halo = halo_at(k, T, walls, ny, hx, hy);
-        if (halo) pull9<Real>(gs, P, pitch, ny, walls, T.x0 + hx, row(T.y0 + hy), gh);
+        halo = halo_at(k, T.wc, T.hc, hx, hy) && inside(T.y0 + hy);
+        if (halo) pull9<double>(gs, P, pitch, ny, walls, T.x0 + hx, row(T.y0 + hy), gh);
     }
     if (tid < 2) wet[tid] = wv;
-    if (PRM_SMEM && tid == 0) tile_prm = node_params<Real>(D);
     __syncthreads();
     if (!live) return;
     const bool blo = walls && y == 0, bhi = walls && y == ny - 1;
     const bool s2 = D.step2 && (blo || bhi);
-    const Real* r0 = ph + (ty + 1) * kPW + tx + 1;
-    Real fo[9], go[9];
-    if constexpr (sizeof(Real) == 8) {
-        double X, Y, L;
-        deriv64(C, D, r0, blo, bhi, wet, X, Y, L);
-        collide64<MRT>(C, f, c, X, Y, L, s2, D.step2_relax_j != 0,
-                       [&](double (&v)[9]) {
+    const double* r0 = ph + (ty + 1) * kPW + tx + 1;
+    double fo[9], go[9];
+    double X, Y, L;
+    deriv64(C, D, r0, blo, bhi, wet, X, Y, L);
+    collide64<MRT>(C, f, c, X, Y, L, s2, D.step2_relax_j != 0,
+                   [&](double (&v)[9]) {
 #pragma unroll
-                           for (int i = 0; i < 9; ++i) v[i] = g[i];
-                       },
-                       fo, go);
-    } else {
-        const NodeParams<Real> prm = node_params<Real>(D);
-        Real dx, dy, lap, n[3], s[3];
-        // the row of a ghost row's phi: row k - 1 (ny - k), see DomDesc::wet_k
-        const Real* gp = bhi ? r0 - (D.wet_k - 1) * kPW : r0 + kPW;
-        const Real* gm = blo ? r0 + (D.wet_k - 1) * kPW : r0 - kPW;
-#pragma unroll
-        for (int j = 0; j < 3; ++j) {
-            n[j] = gp[j - 1];
-            s[j] = gm[j - 1];
-        }
-        if (bhi) {
-            const Real h2 = Real(D.wet_k) * wet[1];
-#pragma unroll
-            for (int j = 0; j < 3; ++j) n[j] = n[j] - h2;
-        }
-        if (blo) {
-            const Real h2 = Real(D.wet_k) * wet[0];
-#pragma unroll
-            for (int j = 0; j < 3; ++j) s[j] = s[j] - h2;
-        }
-        stencils<Real>(c, r0[1], r0[-1], n[1], s[1], n[2], n[0], s[2], s[0], dx, dy, lap);
-        if constexpr (PRM_SMEM) {
-            const volatile NodeParams<Real>& PV = tile_prm;
-            collide<Real, MRT>(PV, f, g, c, dx, dy, lap, s2, D.step2_relax_j != 0, fo, go);
-        } else {
-            collide<Real, MRT>(prm, f, g, c, dx, dy, lap, s2, D.step2_relax_j != 0, fo, go);
-        }
-    }
-    Real* __restrict__ fd = static_cast<Real*>(parity ? D.f[0] : D.f[1]);
-    Real* __restrict__ gd = static_cast<Real*>(parity ? D.g[0] : D.g[1]);
+                       for (int i = 0; i < 9; ++i) v[i] = g[i];
+                   },
+                   fo, go);
+    double* __restrict__ fd = static_cast<double*>(parity ? D.f[0] : D.f[1]);
+    double* __restrict__ gd = static_cast<double*>(parity ? D.g[0] : D.g[1]);
     const int o = y * pitch + x + kXOff;
 #pragma unroll
     for (int i = 0; i < 9; ++i) {
@@ -275,7 +282,8 @@ __device__ __forceinline__ void small_split64(const DomDesc& D, int parity, cons
     const int nh = 2 * kPW + 2 * TY;
     int k = int(blockDim.x) - 1 - tid;
     auto row = [&](int r) { return r < 0 ? r + ny : (r >= ny ? r - ny : r); };
-    bool halo = k < nh && halo_at(k, T, walls, ny, hx, hy);
+    auto inside = [&](int r) { return !walls || (r >= 0 && r < ny); };
+    bool halo = k < nh && halo_at(k, T.wc, T.hc, hx, hy) && inside(T.y0 + hy);
     if (live) pull9<double>(is_g ? gs : fs, P, pitch, ny, walls, x, y, v);
     if (halo) pull9<double>(gs, P, pitch, ny, walls, T.x0 + hx, row(T.y0 + hy), gh);
     const double wv =
@@ -300,7 +308,7 @@ __device__ __forceinline__ void small_split64(const DomDesc& D, int parity, cons
         if (halo) ph[(hy + 1) * kPW + hx + 1] = LB64_MUL(C.sig, phi64(C, gh));
         k += int(blockDim.x);
         if (k >= nh) break;
-        halo = halo_at(k, T, walls, ny, hx, hy);
+        halo = halo_at(k, T.wc, T.hc, hx, hy) && inside(T.y0 + hy);
         if (halo) pull9<double>(gs, P, pitch, ny, walls, T.x0 + hx, row(T.y0 + hy), gh);
     }
     if (tid < 2) wet[tid] = wv;
@@ -335,50 +343,157 @@ __device__ __forceinline__ void small_split64(const DomDesc& D, int parity, cons
     for (int i = 0; i < 9; ++i) store_ghosts(dst + i * P, o, x, nx, out[i]);
 }
 
-// Compact g storage.  Shared memory: nine values (g'_1..g'_8 and their sum)
-// and the phi word of (TY + 4) x 36 positions, then phi of (TY + 2) x 34.
-template <bool MRT>
-__device__ __forceinline__ void small_compact_step(const DomDesc& D, int parity, const SmallTile& T)
+// FP32 full storage, K steps.  A launch and the loads and stores at its
+// ends are 1.5 us of the 2.4 us a step of a small lattice takes, and are paid
+// once for K steps here.  The region of a CTA is its tile and E = 2 (K - 1)
+// nodes around it, a thread per node: 32 columns x TY + 2 E rows.  The first
+// step is done on the region, from phi of the region and one node around it;
+// its f and g go to shared memory, from which phi of the region less one node
+// and the next step on the region less two nodes follow, and so on down to the
+// tile.  blockDim.x = 32 (TY + 2 E), 96 at least.  Shared memory: phi,
+// (TY + 2 E + 2) x 34; for K > 1 f and g, 18 x blockDim.x.
+// PRM_SMEM (a batch): the node parameters are read from shared memory at each
+// use, as in the staged batch kernel, which keeps the bits of its BGK collision
+// (the compiler fuses other products there than with parameters in registers).
+template <bool MRT, bool PRM_SMEM>
+__device__ __forceinline__ void small_steps(const DomDesc& D, int parity, int K, const SmallTile& T)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    const int TY = int(blockDim.x) / kTX;
-    const int ne = (TY + 4) * kEW;
+    __shared__ float wet[2];  // wetting gradients, bottom and top
+    __shared__ NodeParams<float> tile_prm;  // PRM_SMEM only
+    float* ph = reinterpret_cast<float*>(smem);
+    const int RH = int(blockDim.x) / kTX;  // rows of a full region
+    float* F = ph + (RH + 2) * kPW;
+    const int SP = int(blockDim.x);  // plane stride of F and G
+    float* G = F + 9 * SP;
+    const int nx = D.nx, ny = D.ny, pitch = D.pitch, P = int(D.plane);
+    const bool walls = D.walls != 0;
+    const float* __restrict__ fs = static_cast<const float*>(parity ? D.f[1] : D.f[0]);
+    const float* __restrict__ gs = static_cast<const float*>(parity ? D.g[1] : D.g[0]);
+    const int tid = int(threadIdx.x), i = tid % kTX, j = tid / kTX;
+    const int E = 2 * (K - 1), xr = T.x0 - E, yr = T.y0 - E;
+    const int rw = T.wc + 2 * E, rh = T.hc + 2 * E;  // the region
+    auto row = [&](int r) { return r < 0 ? r + ny : (r >= ny ? r - ny : r); };
+    // K = 1 stays within the ghost columns
+    auto col = [&](int c) { return K == 1 ? c : (c < 0 ? c + nx : (c >= nx ? c - nx : c)); };
+    auto inside = [&](int r) { return !walls || (r >= 0 && r < ny); };
+    const int x = xr + i, yl = yr + j, y = row(yl);
+    const bool live = i < rw && j < rh && inside(yl);
+    int hx, hy;
+    const bool halo = halo_at(SP - 1 - tid, rw, rh, hx, hy) && inside(yr + hy);
+    float f[9], g[9], gh[9];
+    if (live) pull9<float>(gs, P, pitch, ny, walls, col(x), y, g);
+    if (halo) pull9<float>(gs, P, pitch, ny, walls, col(xr + hx), row(yr + hy), gh);
+    if (live) pull9<float>(fs, P, pitch, ny, walls, col(x), y, f);
+    const float wv = tid == 0 ? wet_bottom<float>(D) : (tid == 1 ? wet_top<float>(D) : 0.f);
+    float* r0 = ph + (j + 1) * kPW + i + 1;
+    float c = 0.f;
+    if (live) *r0 = c = phi_sum<float>(g);
+    if (halo) ph[(hy + 1) * kPW + hx + 1] = phi_sum<float>(gh);
+    if (tid < 2) wet[tid] = wv;
+    if (PRM_SMEM && tid == 0) tile_prm = node_params<float>(D);
+    __syncthreads();
+    const bool blo = walls && y == 0, bhi = walls && y == ny - 1;
+    const bool s2 = D.step2 && (blo || bhi);
+    const NodeParams<float> prm = node_params<float>(D);
+    float fo[9], go[9];
+    bool on = live;
+#pragma unroll 1
+    for (int m = 1;; m += 2) {
+        if (on) {
+            float dx, dy, lap;
+            deriv32(D, r0, c, blo, bhi, wet, dx, dy, lap);
+            if constexpr (PRM_SMEM) {
+                const volatile NodeParams<float>& PV = tile_prm;
+                collide<float, MRT>(PV, f, g, c, dx, dy, lap, s2, D.step2_relax_j != 0, fo, go);
+            } else {
+                collide<float, MRT>(prm, f, g, c, dx, dy, lap, s2, D.step2_relax_j != 0, fo, go);
+            }
+        }
+        if (m > E) break;
+        if (on) {
+#pragma unroll
+            for (int q = 0; q < 9; ++q) {
+                F[q * SP + tid] = fo[q];
+                G[q * SP + tid] = go[q];
+            }
+        }
+        __syncthreads();
+        on = live && i >= m && i < rw - m && j >= m && j < rh - m;
+        if (on) {
+            pull_shared(G, SP, tid, blo, bhi, g);
+            *r0 = c = phi_sum<float>(g);
+        }
+        on = on && i > m && i < rw - m - 1 && j > m && j < rh - m - 1;
+        if (on) pull_shared(F, SP, tid, blo, bhi, f);
+        __syncthreads();
+    }
+    if (!on) return;
+    float* __restrict__ fd = static_cast<float*>(parity ? D.f[0] : D.f[1]);
+    float* __restrict__ gd = static_cast<float*>(parity ? D.g[0] : D.g[1]);
+    const int o = y * pitch + x + kXOff;
+#pragma unroll
+    for (int q = 0; q < 9; ++q) {
+        store_ghosts(fd + q * P, o, x, nx, fo[q]);
+        store_ghosts(gd + q * P, o, x, nx, go[q]);
+    }
+}
+
+// Compact g storage.  Shared memory: nine values (g'_1..g'_8 and their sum)
+// and the phi word of (TY + 4) x 36 positions, then phi of (TY + 2) x 34.
+// K steps as in small_steps: the first one from the compact values of the region
+// and two nodes around it, the others from the values of the step before, which
+// each thread expands for its own node.  blockDim.x = 32 (TY + 2 E); for K > 1
+// f of a step follows in shared memory, 9 x blockDim.x.
+template <bool MRT>
+__device__ __forceinline__ void small_compact_steps(const DomDesc& D, int parity, int K,
+                                                    const SmallTile& T)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    const int SP = int(blockDim.x), RH = SP / kTX;
+    const int ne = (RH + 4) * kEW;
     float* E = reinterpret_cast<float*>(smem);  // E[i * ne + position], i = 0: the sum, 9: the word
     float* ph = E + 10 * ne;
+    float* F = ph + (RH + 2) * kPW;
     const int nx = D.nx, ny = D.ny, pitch = D.pitch, P = int(D.plane);
     const bool walls = D.walls != 0;
     const float* __restrict__ fs = static_cast<const float*>(parity ? D.f[1] : D.f[0]);
     const float* __restrict__ cs = static_cast<const float*>(parity ? D.g[1] : D.g[0]);
-    const int tid = int(threadIdx.x), tx = tid % kTX, ty = tid / kTX;
-    const int x = T.x0 + tx, y = T.y0 + ty;
-    const bool live = tx < T.wc && ty < T.hc;
+    const int tid = int(threadIdx.x), i = tid % kTX, j = tid / kTX;
+    const int rim = 2 * (K - 1), xr = T.x0 - rim, yr = T.y0 - rim;
+    const int rw = T.wc + 2 * rim, rh = T.hc + 2 * rim;  // the region
     auto row = [&](int r) { return r < 0 ? r + ny : (r >= ny ? r - ny : r); };
+    auto col = [&](int c) { return K == 1 ? c : (c < 0 ? c + nx : (c >= nx ? c - nx : c)); };
     auto inside = [&](int r) { return !walls || (r >= 0 && r < ny); };
+    const int x = xr + i, yl = yr + j, y = row(yl);
+    const bool live = i < rw && j < rh && inside(yl);
     const NodeParams<float> prm = node_params<float>(D);
     float f[9];
-    if (live) pull9<float>(fs, P, pitch, ny, walls, x, y, f);
+    if (live) pull9<float>(fs, P, pitch, ny, walls, col(x), y, f);
     __shared__ float wet[2];  // wetting gradients, bottom and top
     const float wv = tid == 0 ? wet_bottom<float>(D) : (tid == 1 ? wet_top<float>(D) : 0.f);
-    // 1. expand the compact values of the tile and two nodes around it
-    for (int k = tid; k < ne; k += int(blockDim.x)) {
-        const int cy = k / kEW, cx = k - cy * kEW;
-        const int r = T.y0 + cy - 2;
-        if (cx - 2 > T.wc + 1 || cy - 2 > T.hc + 1 || !inside(r)) continue;
-        const float* s = cs + row(r) * pitch + T.x0 + cx - 2 + kXOff;
-        const f2 word(s[0]), G(s[P]), ux(s[2 * P]), uy(s[3 * P]);
+    auto expand = [&](int k, f2 word, f2 G, f2 ux, f2 uy) {
         f2 ge[9];
         g_equilibria2(g0_value2(word), G, ux, uy, ge);
         E[k] = g_tail_sum2(ge).lane(0);
 #pragma unroll
-        for (int i = 1; i < 9; ++i) E[i * ne + k] = ge[i].lane(0);
+        for (int q = 1; q < 9; ++q) E[q * ne + k] = ge[q].lane(0);
         E[9 * ne + k] = word.lane(0);
+    };
+    // 1. expand the compact values of the region and two nodes around it
+    for (int k = tid; k < ne; k += SP) {
+        const int cy = k / kEW, cx = k - cy * kEW;
+        const int r = yr + cy - 2;
+        if (cx - 2 > rw + 1 || cy - 2 > rh + 1 || !inside(r)) continue;
+        const float* s = cs + row(r) * pitch + col(xr + cx - 2) + kXOff;
+        expand(k, f2(s[0]), f2(s[P]), f2(s[2 * P]), f2(s[3 * P]));
     }
     __syncthreads();
-    // 2. phi(t+1) = word + [(U + H) + D - sum] of the tile and one node around
+    // 2. phi(t+1) = word + [(U + H) + D - sum] of the region and one node around
     //    it (lb_step_compact.cuh); the node's own word for its store
     auto phi_at = [&](int cx, int cy, f2& word) -> f2 {
-        const int q = (cy + 2) * kEW + cx + 2, r = T.y0 + cy;
-        auto e = [&](int i, int dx, int dy) { return f2(E[i * ne + q + dy * kEW + dx]); };
+        const int q = (cy + 2) * kEW + cx + 2, r = yr + cy;
+        auto e = [&](int n, int dx, int dy) { return f2(E[n * ne + q + dy * kEW + dx]); };
         const f2 u = walls && r == 0 ? (e(4, 0, 0) + e(6, 0, 0)) + e(8, 0, 0)
                                      : (e(3, 0, -1) + e(5, -1, -1)) + e(7, 1, -1);
         const f2 h = e(1, -1, 0) + e(2, 1, 0);
@@ -388,52 +503,75 @@ __device__ __forceinline__ void small_compact_step(const DomDesc& D, int parity,
         return g0_value2(word);
     };
     f2 word(0.f), c(0.f), dump(0.f);
+    float* r0 = ph + (j + 1) * kPW + i + 1;
     if (live) {
-        c = phi_at(tx, ty, word);
-        ph[(ty + 1) * kPW + tx + 1] = c.lane(0);
+        c = phi_at(i, j, word);
+        *r0 = c.lane(0);
     }
-    for (int k = int(blockDim.x) - 1 - tid; k < 2 * kPW + 2 * TY; k += int(blockDim.x)) {
+    for (int k = SP - 1 - tid; k < 2 * kPW + 2 * RH; k += SP) {
         int hx, hy;
-        if (!halo_at(k, T, walls, ny, hx, hy)) continue;
+        if (!halo_at(k, rw, rh, hx, hy) || !inside(yr + hy)) continue;
         // a periodic halo row is the row across the lattice's edge
         ph[(hy + 1) * kPW + hx + 1] = phi_at(hx, hy, dump).lane(0);
     }
     if (tid < 2) wet[tid] = wv;
     __syncthreads();
-    // 3. collide
-    if (!live) return;
     const bool blo = walls && y == 0, bhi = walls && y == ny - 1;
-    const float* r0 = ph + (ty + 1) * kPW + tx + 1;
-    const float* gp = bhi ? r0 - (D.wet_k - 1) * kPW : r0 + kPW;
-    const float* gm = blo ? r0 + (D.wet_k - 1) * kPW : r0 - kPW;
-    f2 n[3], s[3];
+    f2 fo[9], gmu, ux, uy;
+    bool on = live;
+#pragma unroll 1
+    for (int m = 1;; m += 2) {
+        // 3. collide
+        if (on) {
+            const float* gp = bhi ? r0 - (D.wet_k - 1) * kPW : r0 + kPW;
+            const float* gm = blo ? r0 + (D.wet_k - 1) * kPW : r0 - kPW;
+            f2 n[3], s[3];
 #pragma unroll
-    for (int j = 0; j < 3; ++j) {
-        n[j] = f2(gp[j - 1]);
-        s[j] = f2(gm[j - 1]);
+            for (int q = 0; q < 3; ++q) {
+                n[q] = f2(gp[q - 1]);
+                s[q] = f2(gm[q - 1]);
+            }
+            if (bhi) {
+                const f2 h(float(D.wet_k) * wet[1]);
+#pragma unroll
+                for (int q = 0; q < 3; ++q) n[q] = n[q] - h;
+            }
+            if (blo) {
+                const f2 h(float(D.wet_k) * wet[0]);
+#pragma unroll
+                for (int q = 0; q < 3; ++q) s[q] = s[q] - h;
+            }
+            f2 dx, dy, lap, fi[9];
+#pragma unroll
+            for (int q = 0; q < 9; ++q) fi[q] = f2(f[q]);
+            stencils2(c, f2(r0[1]), f2(r0[-1]), n[1], s[1], n[2], n[0], s[2], s[0], dx, dy, lap);
+            collide_f2<MRT>(prm, fi, c, dx, dy, lap, D.step2 && (blo || bhi),
+                            D.step2_relax_j != 0, fo, ux, uy);
+            gmu = gamma_mu2(prm, c, lap);
+        }
+        if (m > rim) break;
+        // 4. the next step's g' and f
+        if (on) {
+            expand((j + 2) * kEW + i + 2, word, gmu, ux, uy);
+#pragma unroll
+            for (int q = 0; q < 9; ++q) F[q * SP + tid] = fo[q].lane(0);
+        }
+        __syncthreads();
+        on = live && i >= m && i < rw - m && j >= m && j < rh - m;
+        if (on) {
+            c = phi_at(i, j, word);
+            *r0 = c.lane(0);
+        }
+        on = on && i > m && i < rw - m - 1 && j > m && j < rh - m - 1;
+        if (on) pull_shared(F, SP, tid, blo, bhi, f);
+        __syncthreads();
     }
-    if (bhi) {
-        const f2 h(float(D.wet_k) * wet[1]);
-#pragma unroll
-        for (int j = 0; j < 3; ++j) n[j] = n[j] - h;
-    }
-    if (blo) {
-        const f2 h(float(D.wet_k) * wet[0]);
-#pragma unroll
-        for (int j = 0; j < 3; ++j) s[j] = s[j] - h;
-    }
-    f2 dx, dy, lap, fi[9], fo[9], ux, uy;
-#pragma unroll
-    for (int i = 0; i < 9; ++i) fi[i] = f2(f[i]);
-    stencils2(c, f2(r0[1]), f2(r0[-1]), n[1], s[1], n[2], n[0], s[2], s[0], dx, dy, lap);
-    collide_f2<MRT>(prm, fi, c, dx, dy, lap, D.step2 && (blo || bhi), D.step2_relax_j != 0, fo, ux,
-                    uy);
-    const f2 gmu = gamma_mu2(prm, c, lap);
+    if (!on) return;
     float* __restrict__ fd = static_cast<float*>(parity ? D.f[0] : D.f[1]);
     float* __restrict__ cd = static_cast<float*>(parity ? D.g[0] : D.g[1]);
     const int o = y * pitch + x + kXOff;
 #pragma unroll
-    for (int i = 0; i < 9; ++i) store_ghosts(fd + i * P, o, x, nx, fo[i].lane(0));
+    for (int q = 0; q < 9; ++q) store_ghosts(fd + q * P, o, x, nx, fo[q].lane(0));
     store_ghosts(cd, o, x, nx, word.lane(0));
     store_ghosts(cd + P, o, x, nx, gmu.lane(0));
     store_ghosts(cd + 2 * P, o, x, nx, ux.lane(0));
@@ -454,13 +592,13 @@ template <SmallKind K, bool MRT, bool BATCH>
 __device__ __forceinline__ void small_tile(const DomDesc& D, int parity, const SmallTile& T)
 {
     if constexpr (K == SmallKind::F64)
-        small_step<double, MRT, false>(D, parity, T);
+        small_step64<MRT>(D, parity, T);
     else if constexpr (K == SmallKind::Split64)
         small_split64<MRT>(D, parity, T);
     else if constexpr (K == SmallKind::F32)
-        small_step<float, MRT, BATCH>(D, parity, T);
+        small_steps<MRT, BATCH>(D, parity, 1, T);
     else
-        small_compact_step<MRT>(D, parity, T);
+        small_compact_steps<MRT>(D, parity, 1, T);
 }
 
 template <SmallKind K, bool MRT>
@@ -468,6 +606,19 @@ __global__ void __launch_bounds__(kSmallMaxThreads) small_step_kernel(DomDesc D,
 {
     const int ty = int(blockDim.x) / lane_threads(K);
     small_tile<K, MRT, false>(D, parity, SmallTile(D, int(blockIdx.x) * kTX, int(blockIdx.y) * ty, ty));
+}
+
+template <bool MRT, bool COMPACT>
+__global__ void __launch_bounds__(kStepsMaxThreads)
+    small_steps_kernel(DomDesc D, int parity, int K, int rows)
+{
+    const int w = kTX - 4 * (K - 1);
+    SmallTile T(D, int(blockIdx.x) * w, int(blockIdx.y) * rows, rows);
+    T.wc = min(T.wc, w);
+    if constexpr (COMPACT)
+        small_compact_steps<MRT>(D, parity, K, T);
+    else
+        small_steps<MRT, false>(D, parity, K, T);
 }
 
 // Batch form: a CTA per work item (a tile of 32 columns x blockDim.x / 32
@@ -527,6 +678,28 @@ int launch_small_step(int precision, int coll, const DomDesc& d, const DomDesc* 
     if (d.compact)
         return int(launch_c<SmallKind::Compact>(coll, d, descs, items, n_items, parity, rows, s));
     return int(launch_c<SmallKind::F32>(coll, d, descs, items, n_items, parity, rows, s));
+}
+
+int launch_small_steps(int coll, const DomDesc& d, int parity, int steps, int rows, void* stream)
+{
+    if (steps < 2 || small_steps_cols(steps) < 1 || rows < 1 ||
+        small_steps_threads(steps, rows) > kStepsMaxThreads)
+        return int(cudaErrorInvalidValue);
+    const int threads = small_steps_threads(steps, rows), w = small_steps_cols(steps);
+    const dim3 grid((d.nx + w - 1) / w, (d.ny + rows - 1) / rows);
+    const size_t smem = small_smem(d.compact ? SmallKind::Compact : SmallKind::F32, threads / kTX) +
+                        size_t(d.compact ? 9 : 18) * threads * 4;
+    using Kernel = void (*)(DomDesc, int, int, int);
+    const Kernel kernel = d.compact
+        ? (coll ? Kernel(small_steps_kernel<true, true>) : Kernel(small_steps_kernel<false, true>))
+        : (coll ? Kernel(small_steps_kernel<true, false>) : Kernel(small_steps_kernel<false, false>));
+    if (smem > 48 * 1024) {
+        const cudaError_t e =
+            cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+        if (e != cudaSuccess) return int(e);
+    }
+    kernel<<<grid, threads, smem, static_cast<cudaStream_t>(stream)>>>(d, parity, steps, rows);
+    return int(cudaGetLastError());
 }
 
 }  // namespace lbfe

@@ -87,6 +87,38 @@ def test_small_lattice_step_is_bit_identical(lbf, storage, nx, ny, walls, rule, 
         assert blob == out[0][2]
 
 
+@pytest.mark.parametrize("storage", ["compact", "fp32"])
+@pytest.mark.parametrize("nx,ny", [(7, 30), (30, 7), (8, 8), (9, 31), (20, 9), (41, 8), (131, 76), (203, 97),
+                                   (215, 105), (245, 110), (320, 200)])
+@pytest.mark.parametrize("collision,walls,rule,lut,tau_phi", [("bgk", True, 0, 0, 1.0),
+                                                              ("mrt", True, 1, 9, 1.0),
+                                                              ("mrt", False, 0, 0, 1.0),
+                                                              ("bgk", False, 0, 0, 0.8)])
+def test_several_steps_per_launch_are_bit_identical(lbf, storage, nx, ny, collision, walls, rule, lut,
+                                                    tau_phi):
+    """Small FP32 lattices, stepped by whole graphs, remainders and single steps
+    with a change of the wetting in between, against the staged step: lattices
+    narrower than a tile's border, of one tile, and of four, three and two steps
+    per launch and two tiles per SM."""
+    if storage == "compact" and tau_phi != 1.0:
+        pytest.skip("compact storage needs tau_phi = 1")
+    p = lbf.params(collision=collision, tau_alpha=1.5, tau_beta=0.6, tau_phi=tau_phi, walls=walls,
+                   wetting_rule=rule, h_bottom=0.1, h_top=-0.07, mrt_lut=lut, **STORAGE[storage])
+    out = []
+    for staged in (True, False):
+        sim = lbf.Lattice(p, nx, ny)
+        if staged:
+            sim.set_tile(64, 2)
+        sim.init_random(0.3, nx + ny)
+        for n in (64, 7, 1, 7, 2, 7, 66):
+            sim.step(n)
+            sim.set_wetting(0.1 - 0.001 * n, 0.05)
+        out.append((*sim.populations(), sim.save_state()))
+        sim.close()
+    assert np.array_equal(out[0][0], out[1][0]) and np.array_equal(out[0][1], out[1][1])
+    assert out[0][2] == out[1][2]
+
+
 @pytest.mark.parametrize("storage", sorted(STORAGE))
 @pytest.mark.parametrize("collision,relax,walls,tau_phi", [("bgk", False, True, 1.0),
                                                            ("mrt", True, True, 1.0),
