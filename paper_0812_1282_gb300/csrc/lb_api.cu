@@ -734,8 +734,10 @@ lb_schedule default_schedule(const lb_handle* h)
 // 300 7.8 and 8.8; FP64 28 x 15 8.3 and 5.1, 200 x 100 11 and 7.5, 1000 x 500
 // 115 and 111, but 1200^2 313 and 302 to 317, 2048^2 828 and 850).  In a batch
 // a tile first finds its domain, two loads in series: 6 domains of 22 k nodes
-// FP32 6.6 and 3.6, compact 7.7 and 4.3, FP64 14.3 and 11, 8 of 178 k 11.7 and
-// 8.0, 11.2 and 9.6, 60 and 47, but 40 of 623 k 28 and 27, 25 and 27, 165 and 165.
+// FP32 6.6 and 3.3, compact 7.6 and 3.9, FP64 14.3 and 8.7, 8 of 178 k 11.7 and
+// 8.0, 11.2 and 9.6, 60 and 47, 40 of 623 k FP32 27.9 and 25.0, 24 of 692 k 28.8
+// and 27.6, but 100 of 4.1 M 137 and 152; compact 40 of 623 k 25 and 28, FP64
+// 165 and 165.
 //  - FP32: 4 rows (3 to 7 are within 5 %);
 //  - compact, whose tiles expand a two-node halo: the fewest rows from 4 on
 //    with which every tile has an SM to itself, else 7;
@@ -752,7 +754,7 @@ int small_rows(const lb_handle* h)
     const bool fp64 = h->precision == LB_FP64, compact = h->descs[0].compact != 0;
     long long nodes = 0;
     for (const DomDesc& D : h->descs) nodes += (long long)D.nx * D.ny;
-    const long long most = h->n_dom > 1 ? (compact ? 200000 : 300000)
+    const long long most = h->n_dom > 1 ? (compact ? 200000 : (fp64 ? 300000 : 700000))
                                         : (fp64 ? 800000 : (compact ? 140000 : 700000));
     if (nodes > most) return 0;
     auto tiles = [&](int rows) {

