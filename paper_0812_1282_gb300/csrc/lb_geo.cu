@@ -60,29 +60,13 @@
 #include "lb_geo_persist.h"
 #include "lb_node.cuh"
 #include "lb_node64.cuh"
+#include "lb_step.cuh"
 
 namespace lbfe {
 
 namespace {
 
 constexpr int kGeoBlock = 128;
-
-template <typename Real>
-__device__ __forceinline__ NodeParams<Real> geo_params(const DomDesc& D);
-template <>
-__device__ __forceinline__ NodeParams<float> geo_params<float>(const DomDesc& D)
-{
-    return NodeParams<float>{D.fa,      D.fkappa,  D.fgamma,   D.fomega_phi,
-                             D.ftau_c0, D.ftau_c1, D.fh_bot,   D.fh_top,
-                             D.flut_lo, D.flut_step, D.flut_inv, D.flut_kmax};
-}
-template <>
-__device__ __forceinline__ NodeParams<double> geo_params<double>(const DomDesc& D)
-{
-    return NodeParams<double>{D.a,      D.kappa,  D.gamma,   D.omega_phi,
-                              D.tau_c0, D.tau_c1, D.h_bot,   D.h_top,
-                              D.lut_lo, D.lut_step, D.lut_inv, D.lut_kmax};
-}
 
 template <typename Real>
 __device__ __forceinline__ Real class_h(const DomDesc& D, int k);
@@ -308,7 +292,7 @@ __device__ __forceinline__ void geo_collide(const DomDesc& D, const GeoConst<Rea
         Real dx, dy, lap;
         // order: centre, E, W, N, S, NE, NW, SE, SW
         stencils<Real>(c, nb[1], nb[2], nb[3], nb[4], nb[5], nb[7], nb[8], nb[6], dx, dy, lap);
-        const NodeParams<Real> prm = geo_params<Real>(D);
+        const NodeParams<Real> prm = node_params<Real>(D);
         collide<Real, MRT>(prm, f, g, c, dx, dy, lap, step2, D.step2_relax_j != 0, fo, go);
     }
 }

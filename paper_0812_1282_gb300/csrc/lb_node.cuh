@@ -31,8 +31,6 @@ template <typename Real>
 __device__ __forceinline__ Real rcp_rn(Real x);
 template <>
 __device__ __forceinline__ float rcp_rn<float>(float x) { return __frcp_rn(x); }
-template <>
-__device__ __forceinline__ double rcp_rn<double>(double x) { return __drcp_rn(x); }
 
 // x / K for a small integer constant K, unbiased.  In FP32 the product with
 // the rounded reciprocal fl(1/K) carries a systematic relative bias (e.g.

@@ -50,14 +50,6 @@ __device__ __forceinline__ NodeParams<float> node_params<float>(const DomDesc& D
                              D.ftau_c0, D.ftau_c1, D.fh_bot,   D.fh_top,
                              D.flut_lo, D.flut_step, D.flut_inv, D.flut_kmax};
 }
-template <>
-__device__ __forceinline__ NodeParams<double> node_params<double>(const DomDesc& D)
-{
-    return NodeParams<double>{D.a,      D.kappa,  D.gamma,   D.omega_phi,
-                              D.tau_c0, D.tau_c1, D.h_bot,   D.h_top,
-                              D.lut_lo, D.lut_step, D.lut_inv, D.lut_kmax};
-}
-
 // The wall wetting gradients as they are now (DomDesc::self).
 template <typename Real>
 __device__ __forceinline__ Real wet_bottom(const DomDesc& D)

@@ -18,7 +18,7 @@ namespace lbfe {
 
 // Stage-ring depth: rows of bulk copies in flight per CTA.
 template <typename Real>
-constexpr int kStages = sizeof(Real) == 4 ? 4 : 3;
+constexpr int kStages = 4;
 // Named barrier of the compute warps of the batched full-storage form.
 constexpr int kComputeBarrierFull = 1;
 
