@@ -940,12 +940,12 @@ int enqueue_geo_steps(lb_handle* h, int len, int parity, bool fixed_parity, cuda
             if (e == 0 && (len & 1))
                 e = lbfe::launch_geo_step(h->precision, h->coll, D,
                                           fixed_parity ? parity : parity ^ (pairs & 1),
-                                          tile_rows, tiles, n_tiles, s);
+                                          tile_rows, tiles, n_tiles, h->sm_count, s);
         } else {
             for (int k = 0; k < len && e == 0; ++k)
                 e = lbfe::launch_geo_step(h->precision, h->coll, D,
                                           fixed_parity ? parity : parity ^ (k & 1), tile_rows,
-                                          tiles, n_tiles, s);
+                                          tiles, n_tiles, h->sm_count, s);
         }
         if (e != 0)
             return fail(LB_ERR_CUDA, "obstacle step launch failed: %s", cudaGetErrorString(cudaError_t(e)));

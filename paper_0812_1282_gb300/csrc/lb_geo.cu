@@ -26,7 +26,7 @@
 // A step is one launch over the tiles that hold a fluid or wall node (a list
 // the host makes with the map).  A CTA owns a tile of 32 x TY nodes (one per
 // thread) and, in shared memory, the class map of the tile and a four-node
-// halo.  Then
+// halo; further warps help with halo positions and ghost values.  Then
 //   1. each thread pulls f and g of its node and g of one halo position, and
 //      stores the phi of both (Eq. moments).  A tile needs phi on a one-node
 //      halo, and a tile with a solid neighbour somewhere on a three-node one:
@@ -44,10 +44,10 @@
 // latency rather than by HBM bandwidth, so it uses plain loads instead of
 // the staged pipeline of the plain step, and one launch with one shared
 // phi field instead of a phi pass through memory.  Measured, us per step:
-// 1000 x 120 channel FP32 7.6 -> 5.3 (a three-node phi halo in every tile,
+// 1000 x 120 channel FP32 7.6 -> 4.3 (a three-node phi halo in every tile,
 // ghost values formed anew for each fluid neighbour, g pulled twice, tiles of
-// solid nodes launched; then as above), 2000 x 200 FP32 18 -> 10.9, 401 x 77
-// FP64 22 -> 10.2 (with the arithmetic of lb_node64.cuh); a single tile 4.2 ->
+// solid nodes launched; then as above), 2000 x 200 FP32 18 -> 10.6, 401 x 77
+// FP64 22 -> 9.5 (with the arithmetic of lb_node64.cuh); a single tile 4.2 ->
 // 3.2, of which the launch is about half.
 #include <cuda_runtime.h>
 
@@ -341,14 +341,14 @@ struct GeoHalo {
 };
 
 // One time step of the tile at (x0, y0).  near: the tile holds a fluid node
-// with a solid neighbour.  Every thread of the CTA calls it (it holds CTA
-// barriers).
-template <typename Real, bool MRT, int TY, bool L2ONLY>
+// with a solid neighbour.  Every one of the CTA's N threads calls it (it holds
+// CTA barriers); those beyond the tile's nodes help with halo positions and
+// ghost values.
+template <typename Real, bool MRT, int TY, int N, bool L2ONLY>
 __device__ __forceinline__ void geo_tile_step(const DomDesc& D, const GeoConst<Real>& K, int parity,
                                               int x0, int y0, bool near, const GeoTables<TY>& t,
                                               Real (&ph)[TY + 2 * kGH][kGPX])
 {
-    constexpr int N = kGTX * TY;
     const int nx = D.nx, ny = D.ny;
     const long long P = D.plane;
     const Real* fs = static_cast<const Real*>(parity ? D.f[1] : D.f[0]);
@@ -370,7 +370,8 @@ __device__ __forceinline__ void geo_tile_step(const DomDesc& D, const GeoConst<R
         }
     };
     const int tid = int(threadIdx.x), x = tid % kGTX, y = tid / kGTX;
-    const int cme = (x0 + x < nx && y0 + y < ny) ? cls(x, y) : 1;
+    const bool has_node = N == kGTX * TY || tid < kGTX * TY;
+    const int cme = (has_node && x0 + x < nx && y0 + y < ny) ? cls(x, y) : 1;
     const bool live = cme == 0 || cme == kNodeWall;
     // 1. own f and g, and g of halo positions
     Real f[9], g[9];
@@ -379,7 +380,7 @@ __device__ __forceinline__ void geo_tile_step(const DomDesc& D, const GeoConst<R
         pull(fs, x, y, f);
     }
     const int nh = GeoHalo<TY>::kRing1 + (near ? GeoHalo<TY>::kRing3 : 0);
-    for (int k = tid; k < nh; k += N) {
+    for (int k = N - 1 - tid; k < nh; k += N) {
         int hx, hy;
         GeoHalo<TY>::at(k, hx, hy);
         if (cls(hx, hy) == 0) {
@@ -394,7 +395,7 @@ __device__ __forceinline__ void geo_tile_step(const DomDesc& D, const GeoConst<R
     if (live) {
         c = geo_phi<Real>(K, g);
         phi(x, y) = c;
-    } else if (cls(x, y) == 0) {
+    } else if (has_node && cls(x, y) == 0) {
         pull(gs, x, y, g);
         phi(x, y) = geo_phi<Real>(K, g);
     }
@@ -452,10 +453,11 @@ __device__ __forceinline__ void pdl_allow_next()
 }
 __device__ __forceinline__ void pdl_wait_prev() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
-// tiles: the domain's list (make_geo_tiles).
-template <typename Real, bool MRT, int TY>
-__global__ void __launch_bounds__(kGTX * TY) geo_step_kernel(DomDesc D, int parity,
-                                                             const int* __restrict__ tiles)
+// tiles: the domain's list (make_geo_tiles).  XW warps beyond those of the nodes
+// (see geo_extra_warps).
+template <typename Real, bool MRT, int TY, int XW>
+__global__ void __launch_bounds__(kGTX * (TY + XW))
+    geo_step_kernel(DomDesc D, int parity, const int* __restrict__ tiles)
 {
     __shared__ GeoTables<TY> t;
     __shared__ Real ph[TY + 2 * kGH][kGPX];
@@ -466,7 +468,7 @@ __global__ void __launch_bounds__(kGTX * TY) geo_step_kernel(DomDesc D, int pari
     const int x0 = q % ntx * kGTX, y0 = q / ntx * TY;
     geo_tile_setup<Real, TY>(D, x0, y0, t, K);
     pdl_wait_prev();
-    geo_tile_step<Real, MRT, TY, false>(D, K, parity, x0, y0, e < 0, t, ph);
+    geo_tile_step<Real, MRT, TY, kGTX * (TY + XW), false>(D, K, parity, x0, y0, e < 0, t, ph);
 }
 
 // Two steps per launch (temporal blocking; the state stays in L2, so a step
@@ -732,7 +734,7 @@ __global__ void __launch_bounds__(kGTX * kGTY, sizeof(Real) == 4 ? 4 : 2)
             __syncthreads();
             if (stop) break;
         }
-        geo_tile_step<Real, MRT, kGTY, true>(D, K, parity0 ^ (s & flip), x0, y0, true, t, ph);
+        geo_tile_step<Real, MRT, kGTY, kGTX * kGTY, true>(D, K, parity0 ^ (s & flip), x0, y0, true, t, ph);
         __syncthreads();
         if (threadIdx.x == 0) {
             __threadfence();
@@ -852,17 +854,33 @@ dim3 geo_grid(const DomDesc& d) { return dim3((d.nx + kGeoBlock - 1) / kGeoBlock
 // A dependent launch, except for FP64 domains of few tiles: the next grid's
 // CTAs are placed while this one's still run, some of them two to an SM, and
 // there the FP64 pipe of the fullest SM is the bound (401 x 77 channel, about
-// one tile per SM: 10.2 us a step without, 20.9 with; 2000 x 200, twelve
+// one tile per SM: 9.5 us a step without, 20.9 with; 2000 x 200, twelve
 // tiles per SM: 58.0 without, 56.2 with; FP32 1000 x 120: 6.4 without, 5.3
-// with).
+// with, before the extra warps).
 constexpr int kFewTiles = 1024;
 
-template <typename Real, bool MRT, int TY>
+// Warps of a CTA beyond those of its nodes.  A near tile has more halo positions
+// (276 with 8 rows, 252 with 4) and possible ghost values (340, 204) than nodes,
+// and the second round of a few of them holds up the whole CTA.  Three more warps
+// take both in one round, while two such CTAs fit each SM; with more tiles than
+// that one more, which saves the second round of the halo.  us a step with none,
+// one and three more: 1000 x 120 channel (230 tiles) 5.3, 5.1, 4.3; 401 x 77 4.0,
+// 3.7, 3.5; 1500 x 100 (356) 5.6, 5.2, 6.8; with 4 rows, whose tiles fill the GPU
+// (2000 x 200), none 10.6, two 12.7, three 14.4.  FP64, bound by the pipe: four more while
+// each tile has an SM to itself (401 x 77 10.4 -> 9.5), else none (1000 x 120 20.6
+// and 22.2).
+int geo_extra_warps(bool fp64, int rows, int n_tiles, int sm_count)
+{
+    if (fp64) return n_tiles <= sm_count ? 4 : 0;
+    return rows == 8 ? (n_tiles <= 2 * sm_count ? 3 : 1) : 0;
+}
+
+template <typename Real, bool MRT, int TY, int XW>
 cudaError_t geo_step_t(const DomDesc& d, int parity, const int* tiles, int n_tiles, cudaStream_t s)
 {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(n_tiles);
-    cfg.blockDim = dim3(kGTX * TY);
+    cfg.blockDim = dim3(kGTX * (TY + XW));
     cfg.dynamicSmemBytes = 0;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
@@ -870,7 +888,7 @@ cudaError_t geo_step_t(const DomDesc& d, int parity, const int* tiles, int n_til
     attr[0].val.programmaticStreamSerializationAllowed = sizeof(Real) == 4 || n_tiles >= kFewTiles;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, geo_step_kernel<Real, MRT, TY>, d, parity, tiles);
+    return cudaLaunchKernelEx(&cfg, geo_step_kernel<Real, MRT, TY, XW>, d, parity, tiles);
 }
 
 template <typename Real, bool MRT>
@@ -958,17 +976,21 @@ int prepare_geo_step2()
 }
 
 int launch_geo_step(int precision, int coll, const DomDesc& d, int parity, int tile_rows,
-                    const int* tiles, int n_tiles, void* stream)
+                    const int* tiles, int n_tiles, int sm_count, void* stream)
 {
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    if (precision != 0)
-        return int(coll ? geo_step_t<double, true, 4>(d, parity, tiles, n_tiles, s)
-                        : geo_step_t<double, false, 4>(d, parity, tiles, n_tiles, s));
-    if (tile_rows == 8)
-        return int(coll ? geo_step_t<float, true, 8>(d, parity, tiles, n_tiles, s)
-                        : geo_step_t<float, false, 8>(d, parity, tiles, n_tiles, s));
-    return int(coll ? geo_step_t<float, true, 4>(d, parity, tiles, n_tiles, s)
-                    : geo_step_t<float, false, 4>(d, parity, tiles, n_tiles, s));
+    using Launch = cudaError_t (*)(const DomDesc&, int, const int*, int, cudaStream_t);
+    Launch f;
+    switch (geo_extra_warps(precision != 0, tile_rows, n_tiles, sm_count)) {
+        case 4: f = coll ? geo_step_t<double, true, 4, 4> : geo_step_t<double, false, 4, 4>; break;
+        case 3: f = coll ? geo_step_t<float, true, 8, 3> : geo_step_t<float, false, 8, 3>; break;
+        case 1: f = coll ? geo_step_t<float, true, 8, 1> : geo_step_t<float, false, 8, 1>; break;
+        default:
+            f = precision != 0
+                ? (coll ? geo_step_t<double, true, 4, 0> : geo_step_t<double, false, 4, 0>)
+                : (coll ? geo_step_t<float, true, 4, 0> : geo_step_t<float, false, 4, 0>);
+    }
+    return int(f(d, parity, tiles, n_tiles, s));
 }
 
 size_t geo_tile_capacity(int nx, int ny)

@@ -156,7 +156,7 @@ int launch_fill_ghosts(int precision, const DomDesc& d, int parity, void* stream
 // tiles: device list of n_tiles entries of tile_rows rows (GeoTiles,
 // lb_geo_persist.h).
 int launch_geo_step(int precision, int coll, const DomDesc& d, int parity, int tile_rows,
-                    const int* tiles, int n_tiles, void* stream);
+                    const int* tiles, int n_tiles, int sm_count, void* stream);
 int launch_geo_init_eq(int precision, const DomDesc& d, const double* phi0, int parity,
                        void* stream);
 int launch_geo_solid_rest(int precision, const DomDesc& d, int b, void* stream);

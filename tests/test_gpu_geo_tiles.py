@@ -32,7 +32,7 @@ def block_map(nx, ny, walls):
     return cls
 
 
-@pytest.mark.parametrize("nx,ny", [(1301, 131), (333, 30), (227, 37)])
+@pytest.mark.parametrize("nx,ny", [(1301, 131), (1101, 85), (333, 30), (227, 37)])
 @pytest.mark.parametrize("walls", [True, False])
 @pytest.mark.parametrize("precision,tol", [("fp64", 1e-13), ("fp32", 2e-6)])
 def test_tile_list(lbf, oracle_mod, nx, ny, walls, precision, tol):
