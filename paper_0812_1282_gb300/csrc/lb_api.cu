@@ -429,8 +429,8 @@ bool two_step(const lb_handle* h)
 // per SM.  Measured, us per step with 1, 2, 3, 4 steps at the best rows for
 // each: FP32 28 x 15 2.3, 1.6, 1.5, 1.4, 200 x 100 2.7, 2.0, 1.9, 1.8, 300 x
 // 100 2.7, 2.1, 2.5, 3.2, 320 x 200 3.6, 2.7, 4.1, 4.8, 500 x 200 4.2, 4.2, 5.4,
-// 7.4; compact 28 x 15 3.4, 2.0, 1.9, 1.9, 200 x 100 3.5, 2.5, 2.4, 2.3, 300 x
-// 100 3.4, 2.7, 3.7, 4.3, 320 x 200 4.2, 3.7, 6.2, 6.5.
+// 7.4; compact (before its loads ahead) 28 x 15 3.4, 2.0, 1.9, 1.9, 200 x 100
+// 3.5, 2.5, 2.4, 2.3, 300 x 100 3.4, 2.7, 3.7, 4.3, 320 x 200 4.2, 3.7, 6.2, 6.5.
 std::pair<int, int> small_steps(const lb_handle* h)
 {
     const DomDesc& D = h->descs[0];
@@ -730,11 +730,11 @@ lb_schedule default_schedule(const lb_handle* h)
 // bound by the FP64 pipe and the tiles still fit the SMs evenly (us per step,
 // staged and small: FP32 28 x 15 4.0 and 1.4, 200 x 100 4.3 and 1.8, 1000 x 500
 // 15.4 and 13.3, 2000 x 350 20.7 and 20.0, but 900^2 24.4 and 27.4; compact
-// 28 x 15 4.5 and 1.9, 200 x 100 4.8 and 2.3, 512 x 256 7.2 and 5.9, but 700 x
+// 28 x 15 4.5 and 1.8, 200 x 100 4.8 and 2.2, 512 x 256 7.2 and 5.9, but 700 x
 // 300 7.8 and 8.8; FP64 28 x 15 8.3 and 5.1, 200 x 100 11 and 7.5, 1000 x 500
 // 115 and 111, but 1200^2 313 and 302 to 317, 2048^2 828 and 850).  In a batch
 // a tile first finds its domain, two loads in series: 6 domains of 22 k nodes
-// FP32 6.6 and 3.3, compact 7.6 and 3.9, FP64 14.3 and 8.7, 8 of 178 k 11.7 and
+// FP32 6.6 and 3.3, compact 7.6 and 3.8, FP64 14.3 and 8.7, 8 of 178 k 11.7 and
 // 8.0, 11.2 and 9.6, 60 and 47, 40 of 623 k FP32 27.9 and 25.0, 24 of 692 k 28.8
 // and 27.6, but 100 of 4.1 M 137 and 152; compact 40 of 623 k 25 and 28, FP64
 // 165 and 165.

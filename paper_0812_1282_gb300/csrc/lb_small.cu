@@ -21,7 +21,7 @@
 //    FP64, bound by its pipe instead, splits a node over two threads
 //    (small_split64).
 // us a step, staged, one step per launch, and as here: FP32 28 x 15 4.0, 2.3, 1.4,
-// 200 x 100 4.4, 2.7, 1.8; compact 28 x 15 4.5, 3.4, 1.9, 200 x 100 4.9, 3.5, 2.3;
+// 200 x 100 4.4, 2.7, 1.8; compact 28 x 15 4.5, 3.4, 1.8, 200 x 100 4.9, 3.5, 2.2;
 // FP64 28 x 15 8.3, 6.6, 5.1, 200 x 100 11, 7.5.
 // The arithmetic is that of the staged kernels, operation for operation, and
 // so are the stored populations and ghost columns, bit for bit.
@@ -445,7 +445,11 @@ __device__ __forceinline__ void small_steps(const DomDesc& D, int parity, int K,
 // and two nodes around it, the others from the values of the step before, which
 // each thread expands for its own node.  blockDim.x = 32 (TY + 2 E); for K > 1
 // f of a step follows in shared memory, 9 x blockDim.x.
-template <bool MRT>
+// AHEAD: a thread's first two positions are loaded before either is expanded (us a
+// step: 28 x 15 1.87 -> 1.78, 200 x 100 2.32 -> 2.22, 300 x 100 2.66 -> 2.51, 6 domains
+// of 22 k nodes 3.9 -> 3.8; but single steps of larger lattices, which are not bound by
+// latency alone, 512 x 256 5.84 -> 5.92, without).
+template <bool MRT, bool AHEAD>
 __device__ __forceinline__ void small_compact_steps(const DomDesc& D, int parity, int K,
                                                     const SmallTile& T)
 {
@@ -481,13 +485,28 @@ __device__ __forceinline__ void small_compact_steps(const DomDesc& D, int parity
         E[9 * ne + k] = word.lane(0);
     };
     // 1. expand the compact values of the region and two nodes around it
-    for (int k = tid; k < ne; k += SP) {
+    auto source = [&](int k) -> const float* {
         const int cy = k / kEW, cx = k - cy * kEW;
         const int r = yr + cy - 2;
-        if (cx - 2 > rw + 1 || cy - 2 > rh + 1 || !inside(r)) continue;
-        const float* s = cs + row(r) * pitch + col(xr + cx - 2) + kXOff;
-        expand(k, f2(s[0]), f2(s[P]), f2(s[2 * P]), f2(s[3 * P]));
+        if (k >= ne || cx - 2 > rw + 1 || cy - 2 > rh + 1 || !inside(r)) return nullptr;
+        return cs + row(r) * pitch + col(xr + cx - 2) + kXOff;
+    };
+    int k0 = tid;
+    if constexpr (AHEAD) {
+        const float* s0 = source(tid);
+        const float* s1 = source(tid + SP);
+        float v0[4], v1[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            if (s0) v0[q] = s0[q * P];
+            if (s1) v1[q] = s1[q * P];
+        }
+        if (s0) expand(tid, f2(v0[0]), f2(v0[1]), f2(v0[2]), f2(v0[3]));
+        if (s1) expand(tid + SP, f2(v1[0]), f2(v1[1]), f2(v1[2]), f2(v1[3]));
+        k0 += 2 * SP;
     }
+    for (int k = k0; k < ne; k += SP)
+        if (const float* s = source(k)) expand(k, f2(s[0]), f2(s[P]), f2(s[2 * P]), f2(s[3 * P]));
     __syncthreads();
     // 2. phi(t+1) = word + [(U + H) + D - sum] of the region and one node around
     //    it (lb_step_compact.cuh); the node's own word for its store
@@ -598,7 +617,7 @@ __device__ __forceinline__ void small_tile(const DomDesc& D, int parity, const S
     else if constexpr (K == SmallKind::F32)
         small_steps<MRT, BATCH>(D, parity, 1, T);
     else
-        small_compact_steps<MRT>(D, parity, 1, T);
+        small_compact_steps<MRT, BATCH>(D, parity, 1, T);
 }
 
 template <SmallKind K, bool MRT>
@@ -616,7 +635,7 @@ __global__ void __launch_bounds__(kStepsMaxThreads)
     SmallTile T(D, int(blockIdx.x) * w, int(blockIdx.y) * rows, rows);
     T.wc = min(T.wc, w);
     if constexpr (COMPACT)
-        small_compact_steps<MRT>(D, parity, K, T);
+        small_compact_steps<MRT, true>(D, parity, K, T);
     else
         small_steps<MRT, false>(D, parity, K, T);
 }
