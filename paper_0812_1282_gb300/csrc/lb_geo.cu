@@ -44,11 +44,11 @@
 // latency rather than by HBM bandwidth, so it uses plain loads instead of
 // the staged pipeline of the plain step, and one launch with one shared
 // phi field instead of a phi pass through memory.  Measured, us per step:
-// 1000 x 120 channel FP32 7.6 -> 4.3 (a three-node phi halo in every tile,
+// 1000 x 120 channel FP32 7.6 -> 3.7 (a three-node phi halo in every tile,
 // ghost values formed anew for each fluid neighbour, g pulled twice, tiles of
-// solid nodes launched; then as above), 2000 x 200 FP32 18 -> 10.6, 401 x 77
-// FP64 22 -> 9.5 (with the arithmetic of lb_node64.cuh); a single tile 4.2 ->
-// 3.2, of which the launch is about half.
+// solid nodes launched; then as above), 2000 x 200 FP32 18 -> 9.8, 401 x 77
+// FP64 22 -> 8.9 (with the arithmetic of lb_node64.cuh); a single tile 4.2 ->
+// 2.5.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -340,53 +340,205 @@ struct GeoHalo {
     }
 };
 
-// One time step of the tile at (x0, y0).  near: the tile holds a fluid node
-// with a solid neighbour.  Every one of the CTA's N threads calls it (it holds
+// What a thread does in a tile, from the class map alone: a launch prepares it,
+// its loads' addresses too, while the step before it finishes.  us a step, with the
+// class map looked at on the way and as here: 1000 x 120 channel FP32 4.3 -> 3.7,
+// 401 x 77 3.5 -> 2.7, 1500 x 100 5.2 -> 4.4, 2000 x 200 10.6 -> 9.8, a single tile
+// 3.1 -> 2.5; FP64 401 x 77 9.5 -> 8.9, 1000 x 120 20.7 and 20.8.
+struct GeoNode {      // a node whose populations are pulled
+    int col[3], row[3];  // offsets of its columns x - 1, x, x + 1 and rows
+    unsigned bounce;     // bit i: the source of direction i is solid
+};
+template <typename Real>
+struct GeoGhost {  // a solid node's ghost value (see geo_ghost)
+    int at;         // its place in the phi array
+    int d[2];       // offsets of the mirror nodes: d[0], -d[0], d[1], -d[1]
+    unsigned mask;  // which of the four count; 0: no ghost value
+    Real shift;     // k h
+    bool wall;      // a node wall: phi(at + d[0]) - shift
+};
+template <typename Real>
+struct GeoPlan {
+    int cme;             // class of the thread's own node (1: none)
+    bool phi_only;       // a node beyond the lattice whose phi is needed
+    bool next_to_solid;  // a neighbour of it is not fluid
+    GeoNode own, halo;
+    int halo_at;         // place of the halo position in the phi array, -1: none
+    GeoGhost<Real> ghost;
+};
+
+template <typename Real, int TY, int N>
+struct GeoTile {
+    static constexpr int S = kGPX;  // row stride of the phi array
+    const DomDesc& D;
+    const GeoConst<Real>& K;
+    const GeoTables<TY>& t;
+    int x0, y0;
+    bool near;  // the tile holds a fluid node with a solid neighbour
+    __device__ __forceinline__ GeoTile(const DomDesc& D_, const GeoConst<Real>& K_,
+                                       const GeoTables<TY>& t_, int x0_, int y0_, bool near_)
+        : D(D_), K(K_), t(t_), x0(x0_), y0(y0_), near(near_)
+    {
+    }
+    // positions relative to the tile's first node
+    __device__ __forceinline__ int cls(int x, int y) const { return t.cl[y + kGC][x + kGC]; }
+    __device__ __forceinline__ static int at(int x, int y) { return (y + kGH) * S + x + kGH; }
+    __device__ __forceinline__ GeoNode node(int x, int y) const
+    {
+        GeoNode n;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            n.col[k] = t.colx[x + kGC + k - 1];
+            n.row[k] = t.rowo[y + kGC + k - 1];
+        }
+        n.bounce = 0;
+#pragma unroll
+        for (int i = 1; i < 9; ++i) {
+            const int c = cls(x - gex(i), y - gey(i));
+            if (c != 0 && c != kNodeWall) n.bounce |= 1u << i;
+        }
+        return n;
+    }
+    // ghost position k of the tile and its one-node halo
+    __device__ __forceinline__ GeoGhost<Real> ghost(int k) const
+    {
+        constexpr int GX = kGTX + 2;
+        const int y = k / GX - 1, x = k - (y + 1) * GX - 1;
+        GeoGhost<Real> g;
+        g.mask = 0;
+        if (k >= GX * (TY + 2)) return g;
+        const int c = cls(x, y);
+        if (c == 0) return g;
+        g.at = at(x, y);
+        g.wall = c == kNodeWall;
+        if (g.wall) {
+            const bool bottom = y0 + y == 0;
+            g.mask = 1;
+            g.d[0] = bottom ? S : -S;
+            g.d[1] = 0;
+            g.shift = bottom ? K.h_bot : K.h_top;
+            return g;
+        }
+        unsigned axis = 0, diag = 0;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int ax = j == 0 ? 1 : (j == 1 ? -1 : 0), ay = j == 2 ? 1 : (j == 3 ? -1 : 0);
+            const int bx = (j == 0 || j == 3) ? 1 : -1, by = (j == 0 || j == 2) ? 1 : -1;
+            if (cls(x + ax, y + ay) == 0) axis |= 1u << j;
+            if (cls(x + bx, y + by) == 0) diag |= 1u << j;
+        }
+        const int w = D.wet_k;
+        g.mask = axis ? axis : diag;
+        g.d[0] = axis ? w : w * (S + 1);
+        g.d[1] = axis ? w * S : w * (S - 1);
+        const Real h = c == -1 ? K.h_bot : (c == -2 ? K.h_top : class_h<Real>(D, c));
+        g.shift = Real(w) * h;
+        return g;
+    }
+    __device__ __forceinline__ GeoPlan<Real> plan() const
+    {
+        GeoPlan<Real> p;
+        const int tid = int(threadIdx.x), x = tid % kGTX, y = tid / kGTX;
+        const bool has_node = N == kGTX * TY || tid < kGTX * TY;
+        p.cme = 1;
+        p.phi_only = p.next_to_solid = false;
+        if (has_node) {
+            if (x0 + x < D.nx && y0 + y < D.ny)
+                p.cme = cls(x, y);
+            else
+                p.phi_only = cls(x, y) == 0;
+            p.own = node(x, y);
+#pragma unroll
+            for (int i = 1; i < 9; ++i)
+                p.next_to_solid = p.next_to_solid || (near && cls(x + gex(i), y + gey(i)) != 0);
+        }
+        p.halo_at = -1;
+        if (N - 1 - tid < halo_count()) halo(N - 1 - tid, p.halo, p.halo_at);
+        p.ghost.mask = 0;
+        if (near) p.ghost = ghost(tid);
+        return p;
+    }
+    __device__ __forceinline__ int halo_count() const
+    {
+        return GeoHalo<TY>::kRing1 + (near ? GeoHalo<TY>::kRing3 : 0);
+    }
+    __device__ __forceinline__ void halo(int k, GeoNode& n, int& place) const
+    {
+        int hx, hy;
+        GeoHalo<TY>::at(k, hx, hy);
+        place = -1;
+        if (cls(hx, hy) != 0) return;
+        n = node(hx, hy);
+        place = at(hx, hy);
+    }
+};
+
+// Store a solid node's ghost value from phi around it.
+template <typename Real>
+__device__ __forceinline__ void geo_put_ghost(const GeoGhost<Real>& g, Real* __restrict__ ph)
+{
+    if (g.mask == 0) return;
+    const Real* c = ph + g.at;
+    if (g.wall) {
+        ph[g.at] = c[g.d[0]] - g.shift;
+        return;
+    }
+    const Real p[4] = {c[g.d[0]], c[-g.d[0]], c[g.d[1]], c[-g.d[1]]};
+    Real sum = Real(0);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) sum = (g.mask >> j) & 1u ? sum + p[j] : sum;
+    const int n = __popc(g.mask);
+    const Real mean =
+        n == 1 ? sum : (n == 2 ? sum * Real(0.5) : (n == 3 ? div_const<3>(sum) : sum * Real(0.25)));
+    ph[g.at] = mean - g.shift;
+}
+
+// One time step of a tile.  Every one of the CTA's N threads calls it (it holds
 // CTA barriers); those beyond the tile's nodes help with halo positions and
 // ghost values.
 template <typename Real, bool MRT, int TY, int N, bool L2ONLY>
-__device__ __forceinline__ void geo_tile_step(const DomDesc& D, const GeoConst<Real>& K, int parity,
-                                              int x0, int y0, bool near, const GeoTables<TY>& t,
-                                              Real (&ph)[TY + 2 * kGH][kGPX])
+__device__ __forceinline__ void geo_tile_step(const GeoTile<Real, TY, N>& T,
+                                              const GeoPlan<Real>& p, int parity,
+                                              Real (&phi)[TY + 2 * kGH][kGPX])
 {
-    const int nx = D.nx, ny = D.ny;
+    const DomDesc& D = T.D;
+    const GeoConst<Real>& K = T.K;
     const long long P = D.plane;
     const Real* fs = static_cast<const Real*>(parity ? D.f[1] : D.f[0]);
     const Real* gs = static_cast<const Real*>(parity ? D.g[1] : D.g[0]);
-    // positions relative to the tile's first node
-    auto cls = [&](int x, int y) -> int { return t.cl[y + kGC][x + kGC]; };
-    auto phi = [&](int x, int y) -> Real& { return ph[y + kGH][x + kGH]; };
-    auto off = [&](int x, int y) -> int { return t.rowo[y + kGC] + t.colx[x + kGC]; };
+    Real* ph = &phi[0][0];
     // the nine pulled values of a fluid or wall node; a solid source bounces
     // back (the node's own reversed population), a wall node streams
-    auto pull = [&](const Real* src, int x, int y, Real (&v)[9]) {
-        const int own = off(x, y);
+    auto pull = [&](const Real* src, const GeoNode& n, Real (&v)[9]) {
+        const int own = n.row[1] + n.col[1];
+        v[0] = geo_ld<L2ONLY>(src + own);
 #pragma unroll
-        for (int i = 0; i < 9; ++i) {
-            const int sx = x - gex(i), sy = y - gey(i);
-            const int c = i == 0 ? 0 : cls(sx, sy);
-            v[i] = c != 0 && c != kNodeWall ? geo_ld<L2ONLY>(src + gopp(i) * P + own)
-                                            : geo_ld<L2ONLY>(src + i * P + off(sx, sy));
-        }
+        for (int i = 1; i < 9; ++i)
+            v[i] = (n.bounce >> i) & 1u
+                ? geo_ld<L2ONLY>(src + gopp(i) * P + own)
+                : geo_ld<L2ONLY>(src + i * P + (n.row[1 - gey(i)] + n.col[1 - gex(i)]));
     };
     const int tid = int(threadIdx.x), x = tid % kGTX, y = tid / kGTX;
-    const bool has_node = N == kGTX * TY || tid < kGTX * TY;
-    const int cme = (has_node && x0 + x < nx && y0 + y < ny) ? cls(x, y) : 1;
-    const bool live = cme == 0 || cme == kNodeWall;
+    const bool live = p.cme == 0 || p.cme == kNodeWall;
     // 1. own f and g, and g of halo positions
     Real f[9], g[9];
     if (live) {
-        pull(gs, x, y, g);
-        pull(fs, x, y, f);
+        pull(gs, p.own, g);
+        pull(fs, p.own, f);
     }
-    const int nh = GeoHalo<TY>::kRing1 + (near ? GeoHalo<TY>::kRing3 : 0);
-    for (int k = N - 1 - tid; k < nh; k += N) {
-        int hx, hy;
-        GeoHalo<TY>::at(k, hx, hy);
-        if (cls(hx, hy) == 0) {
+    if (p.halo_at >= 0) {
+        Real gh[9];
+        pull(gs, p.halo, gh);
+        ph[p.halo_at] = geo_phi<Real>(K, gh);
+    }
+    for (int k = 2 * N - 1 - tid; k < T.halo_count(); k += N) {
+        GeoNode n;
+        int place;
+        T.halo(k, n, place);
+        if (place >= 0) {
             Real gh[9];
-            pull(gs, hx, hy, gh);
-            phi(hx, hy) = geo_phi<Real>(K, gh);
+            pull(gs, n, gh);
+            ph[place] = geo_phi<Real>(K, gh);
         }
     }
     // a short last tile's threads beyond the lattice take part in the phi array
@@ -394,27 +546,22 @@ __device__ __forceinline__ void geo_tile_step(const DomDesc& D, const GeoConst<R
     Real c = Real(0);
     if (live) {
         c = geo_phi<Real>(K, g);
-        phi(x, y) = c;
-    } else if (has_node && cls(x, y) == 0) {
-        pull(gs, x, y, g);
-        phi(x, y) = geo_phi<Real>(K, g);
+        ph[T.at(x, y)] = c;
+    } else if (p.phi_only) {
+        pull(gs, p.own, g);
+        ph[T.at(x, y)] = geo_phi<Real>(K, g);
     }
     __syncthreads();
     // 2. ghost values of the solid nodes on the tile and its one-node halo
-    if (near) {
-        constexpr int GX = kGTX + 2, GY = TY + 2;
-        for (int k = tid; k < GX * GY; k += N) {
-            const int sy = k / GX - 1, sx = k - (sy + 1) * GX - 1;
-            if (cls(sx, sy) == 0) continue;
-            Real v;
-            if (geo_ghost<Real>(D, K, sx, sy, y0 + sy, cls, phi, v)) phi(sx, sy) = v;
-        }
+    if (T.near) {
+        geo_put_ghost<Real>(p.ghost, ph);
+        for (int k = tid + N; k < (kGTX + 2) * (TY + 2); k += N) geo_put_ghost<Real>(T.ghost(k), ph);
         __syncthreads();
     }
     // 3. the tile's fluid and wall nodes
     if (!live) return;
     Real fo[9], go[9];
-    if (cme == kNodeWall) {
+    if (p.cme == kNodeWall) {
         // node bounce-back: every population reversed, no collision
 #pragma unroll
         for (int i = 0; i < 9; ++i) {
@@ -423,17 +570,13 @@ __device__ __forceinline__ void geo_tile_step(const DomDesc& D, const GeoConst<R
         }
     } else {
         Real nb[9];
-        bool next_to_solid = false;
 #pragma unroll
-        for (int i = 1; i < 9; ++i) {
-            nb[i] = phi(x + gex(i), y + gey(i));
-            next_to_solid = next_to_solid || (near && cls(x + gex(i), y + gey(i)) != 0);
-        }
-        geo_collide<Real, MRT>(D, K, f, g, c, nb, D.step2 != 0 && next_to_solid, fo, go);
+        for (int i = 1; i < 9; ++i) nb[i] = ph[T.at(x + gex(i), y + gey(i))];
+        geo_collide<Real, MRT>(D, K, f, g, c, nb, D.step2 != 0 && p.next_to_solid, fo, go);
     }
     Real* fd = static_cast<Real*>(parity ? D.f[0] : D.f[1]);
     Real* gd = static_cast<Real*>(parity ? D.g[0] : D.g[1]);
-    const int o = off(x, y);
+    const int o = p.own.row[1] + p.own.col[1];
 #pragma unroll
     for (int i = 0; i < 9; ++i) {
         fd[i * P + o] = fo[i];
@@ -453,10 +596,19 @@ __device__ __forceinline__ void pdl_allow_next()
 }
 __device__ __forceinline__ void pdl_wait_prev() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
+// CTAs per SM the registers of a form leave room for: two and three where the
+// tiles come to that (geo_extra_warps), eight where they fill the GPU (2000 x 200
+// FP32 9.8 us a step, with seven 10.2, without a limit 11.7); FP64 has all the
+// registers it wants.
+constexpr int geo_min_ctas(bool fp64, int xw)
+{
+    return fp64 ? 1 : (xw == 3 ? 2 : (xw == 1 ? 3 : 8));
+}
+
 // tiles: the domain's list (make_geo_tiles).  XW warps beyond those of the nodes
 // (see geo_extra_warps).
 template <typename Real, bool MRT, int TY, int XW>
-__global__ void __launch_bounds__(kGTX * (TY + XW))
+__global__ void __launch_bounds__(kGTX * (TY + XW), geo_min_ctas(sizeof(Real) == 8, XW))
     geo_step_kernel(DomDesc D, int parity, const int* __restrict__ tiles)
 {
     __shared__ GeoTables<TY> t;
@@ -467,8 +619,10 @@ __global__ void __launch_bounds__(kGTX * (TY + XW))
     const int q = e & kGeoTileIndex;
     const int x0 = q % ntx * kGTX, y0 = q / ntx * TY;
     geo_tile_setup<Real, TY>(D, x0, y0, t, K);
+    const GeoTile<Real, TY, kGTX * (TY + XW)> T(D, K, t, x0, y0, e < 0);
+    const GeoPlan<Real> plan = T.plan();
     pdl_wait_prev();
-    geo_tile_step<Real, MRT, TY, kGTX * (TY + XW), false>(D, K, parity, x0, y0, e < 0, t, ph);
+    geo_tile_step<Real, MRT, TY, kGTX * (TY + XW), false>(T, plan, parity, ph);
 }
 
 // Two steps per launch (temporal blocking; the state stays in L2, so a step
@@ -728,13 +882,14 @@ __global__ void __launch_bounds__(kGTX * kGTY, sizeof(Real) == 4 ? 4 : 2)
         stop = 0;
     }
     __syncthreads();
+    const GeoTile<Real, kGTY, kGTX * kGTY> T(D, K, t, x0, y0, true);
     for (int s = 0; s < n_steps; ++s) {
         if (s > 0) {
             if (int(threadIdx.x) < n_nbr && !flag_wait(flags + nbr[threadIdx.x], s, D.err)) stop = 1;
             __syncthreads();
             if (stop) break;
         }
-        geo_tile_step<Real, MRT, kGTY, kGTX * kGTY, true>(D, K, parity0 ^ (s & flip), x0, y0, true, t, ph);
+        geo_tile_step<Real, MRT, kGTY, kGTX * kGTY, true>(T, T.plan(), parity0 ^ (s & flip), ph);
         __syncthreads();
         if (threadIdx.x == 0) {
             __threadfence();
@@ -864,7 +1019,7 @@ constexpr int kFewTiles = 1024;
 // and the second round of a few of them holds up the whole CTA.  Three more warps
 // take both in one round, while two such CTAs fit each SM; with more tiles than
 // that one more, which saves the second round of the halo.  us a step with none,
-// one and three more: 1000 x 120 channel (230 tiles) 5.3, 5.1, 4.3; 401 x 77 4.0,
+// one and three more (before GeoPlan): 1000 x 120 channel (230 tiles) 5.3, 5.1, 4.3; 401 x 77 4.0,
 // 3.7, 3.5; 1500 x 100 (356) 5.6, 5.2, 6.8; with 4 rows, whose tiles fill the GPU
 // (2000 x 200), none 10.6, two 12.7, three 14.4.  FP64, bound by the pipe: four more while
 // each tile has an SM to itself (401 x 77 10.4 -> 9.5), else none (1000 x 120 20.6
