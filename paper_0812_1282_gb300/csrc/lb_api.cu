@@ -1195,13 +1195,16 @@ double* phi0_scratch(lb_handle* h, int dom)
     return static_cast<double*>(h->descs[dom].f[h->parity ^ 1]);
 }
 
+// Before phi0 goes to that scratch: zeros where two-step launches left wide
+// ghost columns (written later, they would be read as part of phi0).
+int begin_init(lb_handle* h) { return narrow_ghosts(h); }
+
 int finish_init(lb_handle* h, int dom)
 {
     // every domain of a handle shares one parity; the new state goes to the
     // current buffer, phi0 sat in the other one
     const DomDesc& D = h->descs[dom];
-    int e = narrow_ghosts(h);
-    if (e != LB_OK) return e;
+    int e;
     // phi0 is consumed once the equilibria are written: clear its scratch, so
     // that the idle buffer's padding columns, which no step reads and only
     // sealing whole-domain strips overwrite (with zeros), hold zeros whatever
@@ -1614,6 +1617,7 @@ int lb_init_drop(lb_handle* h, int dom, double R, double cx, double cy)
     if (rc != LB_OK) return rc;
     if (!std::isfinite(R) || !std::isfinite(cx) || !std::isfinite(cy))
         return fail(LB_ERR_INVALID_ARG, "drop geometry must be finite");
+    if ((rc = begin_init(h)) != LB_OK) return rc;
     const int e = lbfe::launch_init_phi_drop(h->precision, h->descs[dom], phi0_scratch(h, dom), R,
                                              cx, cy, h->stream);
     if (e != 0) return fail(LB_ERR_CUDA, "init launch failed: %s", cudaGetErrorString(cudaError_t(e)));
@@ -1626,6 +1630,7 @@ int lb_init_random(lb_handle* h, int dom, double amp, unsigned long long seed)
     int rc = check_dom(h, dom);
     if (rc != LB_OK) return rc;
     if (!std::isfinite(amp)) return fail(LB_ERR_INVALID_ARG, "amp must be finite");
+    if ((rc = begin_init(h)) != LB_OK) return rc;
     const int e = lbfe::launch_init_phi_random(h->precision, h->descs[dom], phi0_scratch(h, dom),
                                                amp, seed, h->stream);
     if (e != 0) return fail(LB_ERR_CUDA, "init launch failed: %s", cudaGetErrorString(cudaError_t(e)));
@@ -1638,6 +1643,7 @@ int lb_init_phi(lb_handle* h, int dom, const double* phi0, int on_device)
     int rc = check_dom(h, dom);
     if (rc != LB_OK) return rc;
     if (!phi0) return fail(LB_ERR_INVALID_ARG, "phi0 is NULL");
+    if ((rc = begin_init(h)) != LB_OK) return rc;
     const DomDesc& D = h->descs[dom];
     // page-locked host memory is read by a kernel through its device address
     // (one pass over the host link); other host memory goes by copy
