@@ -285,8 +285,9 @@ int lb_load_state(lb_handle* h, const void* host_buf, size_t bytes);
  * chosen from its domains' sizes; a small single domain or batch starts with a
  * step made for small lattices, for which the shape here is the one the
  * general step would take (setting a shape selects the general step).  On a large
- * single domain with compact storage a shape of at least 48 rows keeps two
- * steps per launch (lb_schedule), one of fewer rows takes one. */
+ * single domain with compact storage a shape of block_x 64, 96 or 128 and at
+ * least 48 rows keeps two steps per launch (lb_schedule), any other takes
+ * one. */
 int lb_set_tile(lb_handle* h, int block_x, int rows);
 int lb_get_tile(const lb_handle* h, int* block_x, int* rows);
 

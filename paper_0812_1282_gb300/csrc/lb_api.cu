@@ -413,13 +413,14 @@ void persist_grids(lb_handle* h, const std::vector<WorkItem>& items)
 }
 
 // A single compact domain without obstacles may run two steps per launch and
-// pass over memory (launch_two_step).
+// pass over memory (launch_two_step), with CTAs of these widths.
+bool two_step_width(int bx) { return bx == 64 || bx == 96 || bx == 128; }
+
 bool two_step(const lb_handle* h)
 {
     const DomDesc& D = h->descs[0];
-    const int bx = h->block_x();
     return h->n_dom == 1 && D.compact && !D.cls && h->sched.steps_per_launch == 2 &&
-           (bx == 64 || bx == 96 || bx == 128) && D.nx >= 8 && D.ny >= 8;
+           two_step_width(h->block_x()) && D.nx >= 8 && D.ny >= 8;
 }
 
 // A small FP32 lattice takes several steps per launch (launch_small_steps):
@@ -2144,11 +2145,12 @@ int lb_set_tile(lb_handle* h, int block_x, int rows)
     sc.n_class = 1;
     sc.block_x[0] = block_x;
     sc.rows[0] = rows;
-    // a large compact domain keeps two steps per launch with rows enough to
-    // carry their lead-in, and takes one with fewer
+    // a large compact domain keeps two steps per launch at a width they have
+    // and with rows enough to carry their lead-in, and takes one else
     lb_schedule two{};
     if (h->n_dom == 1 && h->descs[0].compact)
-        sc.steps_per_launch = rows >= 48 && two_step_shape(h, two) ? 2 : 1;
+        sc.steps_per_launch =
+            rows >= 48 && two_step_width(block_x) && two_step_shape(h, two) ? 2 : 1;
     return lb_set_schedule(h, &sc);
 }
 
