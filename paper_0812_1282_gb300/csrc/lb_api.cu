@@ -223,6 +223,11 @@ struct lb_handle {
     int pgrid[LB_MAX_SCHED_CLASSES] = {0};
     // single domain: the start order of its row bands (see band_multiplier)
     int band_mul = 1;
+    // a domain with two steps per launch takes single ones too (an odd count):
+    // the shape by size and the band order of their launch (us for one step, so
+    // and with the shape of two: 1500^2 48 and 60, 2048^2 82 and 101, 4096^2 274
+    // and 331, 8192^2 1037 and 1221)
+    int one_bx = 0, one_rows = 0, one_mul = 1;
     // compact g storage: a strip that covers its whole domain takes the
     // periodic wrap from its own stage copy and leaves the ghost columns
     // alone, so after steps they may be stale; they are refreshed before
@@ -469,16 +474,15 @@ int single_launches(const lb_handle* h, int len)
 // 63.4 GLUPS in order, 65.0 at L = 13, 64.5 at 17, 62.7 at 21 and beyond);
 // 1 (in order) when all bands are in flight at once.  Compact storage only:
 // the full-storage step measured no gain at any L (43.9 GLUPS in order,
-// 42.8-44.1 strided).
-int band_multiplier(const lb_handle* h)
+// 42.8-44.1 strided).  two: of launches of two steps.
+int band_multiplier(const lb_handle* h, bool two, int bx, int rows)
 {
     const DomDesc& D = h->descs[0];
     if (D.cls || h->n_dom != 1 || !D.compact) return 1;
-    const int bx = h->block_x(), rows = h->rows();
-    const int w = two_step(h) ? lbfe::two_step_strip(bx) : lbfe::compact_strip(bx);
+    const int w = two ? lbfe::two_step_strip(bx) : lbfe::compact_strip(bx);
     const long long strips = (D.nx + w - 1) / w, B = (D.ny + rows - 1) / rows;
-    const int occ = two_step(h) ? lbfe::two_step_occupancy(h->coll, bx)
-                                : lbfe::step_single_occupancy(h->precision, h->coll, D.compact, bx);
+    const int occ = two ? lbfe::two_step_occupancy(h->coll, bx)
+                        : lbfe::step_single_occupancy(h->precision, h->coll, D.compact, bx);
     const long long L = 3LL * occ * h->sm_count / (4 * std::max(strips, 1LL));
     if (L < 2 || B <= L + 1) return 1;
     for (long long l = L | 1; l < B; l += 2) {
@@ -499,6 +503,8 @@ int band_multiplier(const lb_handle* h)
     return 1;
 }
 
+lb_schedule one_step_schedule(const lb_handle* h);
+
 // Work list for the batched kernel: every (domain, x strip, row block),
 // grouped by schedule class (class c's items are one contiguous slice).
 int build_items(lb_handle* h)
@@ -510,8 +516,12 @@ int build_items(lb_handle* h)
             const cudaError_t e = cudaError_t(lbfe::prepare_two_step());
             if (e != cudaSuccess)
                 return fail(LB_ERR_CUDA, "kernel setup failed: %s", cudaGetErrorString(e));
+            const lb_schedule one = one_step_schedule(h);
+            h->one_bx = one.block_x[0];
+            h->one_rows = one.rows[0];
+            h->one_mul = band_multiplier(h, false, h->one_bx, h->one_rows);
         }
-        h->band_mul = band_multiplier(h);
+        h->band_mul = band_multiplier(h, two_step(h), h->block_x(), h->rows());
         return LB_OK;
     }
     std::vector<WorkItem> items;
@@ -617,8 +627,9 @@ bool two_step_shape(const lb_handle* h, lb_schedule& s)
     return best < 1e300;
 }
 
-// The schedule a handle starts with (lb_autotune times others): one class,
-// a persistent grid of up to 8 CTAs per SM, and a launch shape from the
+// The schedule by size of steps launched one by one, which a handle starts with
+// (lb_autotune times others) where two_step_shape has no other: one class, a
+// persistent grid of up to 8 CTAs per SM, and a launch shape from the
 // domains' sizes.  A CTA marches through its rows in series, about 1.05 us a
 // row in FP32 and 4.7 us in FP64 whatever its width, so small lattices want
 // their rows spread over the whole GPU, and large ones rows enough per CTA to
@@ -645,7 +656,7 @@ bool two_step_shape(const lb_handle* h, lb_schedule& s)
 // -> 29; compact 200 x 100 40 -> 4.9, 1000 x 500 40 -> 13.7; FP64 200 x 100 158
 // -> 11, 512 x 256 158 -> 35, 1024^2 247 -> 214; 40 drops FP32 43 -> 27, compact
 // 55 -> 25, FP64 248 -> 165.
-lb_schedule default_schedule(const lb_handle* h)
+lb_schedule one_step_schedule(const lb_handle* h)
 {
     const bool compact = h->descs[0].compact != 0, fp64 = h->precision == LB_FP64;
     const bool single = h->n_dom == 1;
@@ -721,6 +732,13 @@ lb_schedule default_schedule(const lb_handle* h)
     }
     s.order = !single && (one_wave || fp64);
     s.chains = 1;
+    return s;
+}
+
+// The schedule a handle starts with.
+lb_schedule default_schedule(const lb_handle* h)
+{
+    lb_schedule s = one_step_schedule(h);
     two_step_shape(h, s);
     return s;
 }
@@ -971,9 +989,11 @@ int enqueue_step(lb_handle* h, int parity, cudaStream_t s)
             if (e != 0)
                 return fail(LB_ERR_CUDA, "step launch failed: %s", cudaGetErrorString(cudaError_t(e)));
         } else if (h->descs[0].cls == nullptr) {
-            const int e = lbfe::launch_step(h->precision, h->coll, h->descs[0], h->d_descs(),
-                                            nullptr, 0, 1, parity, h->block_x(), h->rows(),
-                                            h->band_mul, 0, h->d_sched(0), false, s);
+            const bool two = two_step(h);
+            const int e = lbfe::launch_step(
+                h->precision, h->coll, h->descs[0], h->d_descs(), nullptr, 0, 1, parity,
+                two ? h->one_bx : h->block_x(), two ? h->one_rows : h->rows(),
+                two ? h->one_mul : h->band_mul, 0, h->d_sched(0), false, s);
             if (e != 0)
                 return fail(LB_ERR_CUDA, "step launch failed: %s", cudaGetErrorString(cudaError_t(e)));
         }
