@@ -352,6 +352,9 @@ int lb_get_tile(const lb_handle* h, int* block_x, int* rows);
  *               short, a few instructions more per row elsewhere.
  * Results do not depend on the schedule (bit for bit).  A single-domain
  * handle uses block_x[0] and rows[0] only.  Invalidates captured graphs.
+ * A schedule is that of the general step; the schedule that a handle has, set
+ * again, leaves it on the step it has, and the one it started with puts it back on
+ * the one it started with (that of small lattices, see lb_set_tile).
  * Errors: LB_ERR_INVALID_ARG for a value out of range, max_nx not
  * increasing, persist on a batch without compact FP32 storage, fill_pct outside
  * [0, 400], steps_per_launch outside [0, 2], or a seal_edges value not 0

@@ -1572,6 +1572,65 @@ int interface_points(lb_handle* h, const DomDesc& D, std::vector<double>& raw)
     return LB_OK;
 }
 
+// Checks and sets a schedule.  general: of the general step; else a handle keeps
+// the step it has where the schedule is the one it has, and the one it started with
+// where it is that (get and set leave a small lattice on its step).
+int set_schedule(lb_handle* h, const lb_schedule* sc, bool general)
+{
+    if (use_device(h) != LB_OK) return h ? LB_ERR_CUDA : LB_ERR_INVALID_ARG;
+    if (!sc) return fail(LB_ERR_INVALID_ARG, "schedule is NULL");
+    if (sc->n_class < 1 || sc->n_class > LB_MAX_SCHED_CLASSES)
+        return fail(LB_ERR_INVALID_ARG, "n_class must be in [1, %d]", LB_MAX_SCHED_CLASSES);
+    for (int c = 0; c < sc->n_class; ++c) {
+        const int bx = sc->block_x[c];
+        // compact storage takes strips of up to nine compute warps (556 columns)
+        const int max_bx = h->descs[0].compact ? kMaxBlockXCompact : kMaxBlockX;
+        if (bx < kMinBlockX || bx > max_bx || bx % 32 != 0 || sc->rows[c] < 1 ||
+            (!h->descs[0].compact && lbfe::step_smem_bytes(h->precision, bx) == 0))
+            return fail(LB_ERR_INVALID_ARG,
+                        "block_x must be a multiple of 32 in [32, %d], rows >= 1 (class %d)", max_bx,
+                        c);
+        if (sc->ctas_per_sm[c] < 0 || sc->ctas_per_sm[c] > 32)
+            return fail(LB_ERR_INVALID_ARG, "ctas_per_sm must be in [0, 32] (class %d)", c);
+        if (sc->seal_edges[c] != 0 && sc->seal_edges[c] != 1)
+            return fail(LB_ERR_INVALID_ARG, "seal_edges must be 0 or 1 (class %d)", c);
+        if (c + 1 < sc->n_class &&
+            (sc->max_nx[c] < 1 || (c > 0 && sc->max_nx[c] <= sc->max_nx[c - 1])))
+            return fail(LB_ERR_INVALID_ARG, "max_nx must be positive and increasing");
+    }
+    if ((sc->order != 0 && sc->order != 1) || (sc->chains != 0 && sc->chains != 1) ||
+        (sc->persist != 0 && sc->persist != 1))
+        return fail(LB_ERR_INVALID_ARG, "order, chains and persist must be 0 or 1");
+    if (sc->fill_pct < 0 || sc->fill_pct > 400)
+        return fail(LB_ERR_INVALID_ARG, "fill_pct must be in [0, 400]");
+    if (sc->steps_per_launch < 0 || sc->steps_per_launch > 2)
+        return fail(LB_ERR_INVALID_ARG, "steps_per_launch must be 0, 1 or 2");
+    if (sc->persist && h->n_dom > 1 && !(h->precision == LB_FP32 && h->descs[0].compact))
+        return fail(LB_ERR_INVALID_ARG, "persistent schedules need compact FP32 storage");
+    const int rg = refresh_ghosts(h);  // the new schedule may split a domain into strips
+    if (rg != LB_OK) return rg;
+    LB_CUDA(cudaStreamSynchronize(h->stream));
+    clear_graphs(h);
+    lb_schedule v = *sc;
+    for (int c = v.n_class; c < LB_MAX_SCHED_CLASSES; ++c) {  // unused classes: class 0's values
+        v.max_nx[c] = 0;
+        v.block_x[c] = v.block_x[0];
+        v.rows[c] = v.rows[0];
+        v.ctas_per_sm[c] = v.ctas_per_sm[0];
+        v.seal_edges[c] = v.seal_edges[0];
+    }
+    v.max_nx[v.n_class - 1] = 0;
+    auto same = [](const lb_schedule& a, const lb_schedule& b) {  // integers alone
+        return memcmp(&a, &b, sizeof(a)) == 0;
+    };
+    if (general)
+        h->small_rows = 0;
+    else if (!same(v, h->sched))
+        h->small_rows = same(v, default_schedule(h)) ? small_rows(h) : 0;
+    h->sched = v;
+    return build_items(h);
+}
+
 // The device address of a page-locked host buffer (nullptr if the buffer is
 // pageable or not known to CUDA).
 double* device_alias(double* p)
@@ -2171,7 +2230,7 @@ int lb_set_tile(lb_handle* h, int block_x, int rows)
     if (h->n_dom == 1 && h->descs[0].compact)
         sc.steps_per_launch =
             rows >= 48 && two_step_width(block_x) && two_step_shape(h, two) ? 2 : 1;
-    return lb_set_schedule(h, &sc);
+    return set_schedule(h, &sc, true);
 }
 
 int lb_get_tile(const lb_handle* h, int* block_x, int* rows)
@@ -2182,56 +2241,7 @@ int lb_get_tile(const lb_handle* h, int* block_x, int* rows)
     return LB_OK;
 }
 
-int lb_set_schedule(lb_handle* h, const lb_schedule* sc)
-{
-    if (use_device(h) != LB_OK) return h ? LB_ERR_CUDA : LB_ERR_INVALID_ARG;
-    if (!sc) return fail(LB_ERR_INVALID_ARG, "schedule is NULL");
-    if (sc->n_class < 1 || sc->n_class > LB_MAX_SCHED_CLASSES)
-        return fail(LB_ERR_INVALID_ARG, "n_class must be in [1, %d]", LB_MAX_SCHED_CLASSES);
-    for (int c = 0; c < sc->n_class; ++c) {
-        const int bx = sc->block_x[c];
-        // compact storage takes strips of up to nine compute warps (556 columns)
-        const int max_bx = h->descs[0].compact ? kMaxBlockXCompact : kMaxBlockX;
-        if (bx < kMinBlockX || bx > max_bx || bx % 32 != 0 || sc->rows[c] < 1 ||
-            (!h->descs[0].compact && lbfe::step_smem_bytes(h->precision, bx) == 0))
-            return fail(LB_ERR_INVALID_ARG,
-                        "block_x must be a multiple of 32 in [32, %d], rows >= 1 (class %d)", max_bx,
-                        c);
-        if (sc->ctas_per_sm[c] < 0 || sc->ctas_per_sm[c] > 32)
-            return fail(LB_ERR_INVALID_ARG, "ctas_per_sm must be in [0, 32] (class %d)", c);
-        if (sc->seal_edges[c] != 0 && sc->seal_edges[c] != 1)
-            return fail(LB_ERR_INVALID_ARG, "seal_edges must be 0 or 1 (class %d)", c);
-        if (c + 1 < sc->n_class &&
-            (sc->max_nx[c] < 1 || (c > 0 && sc->max_nx[c] <= sc->max_nx[c - 1])))
-            return fail(LB_ERR_INVALID_ARG, "max_nx must be positive and increasing");
-    }
-    if ((sc->order != 0 && sc->order != 1) || (sc->chains != 0 && sc->chains != 1) ||
-        (sc->persist != 0 && sc->persist != 1))
-        return fail(LB_ERR_INVALID_ARG, "order, chains and persist must be 0 or 1");
-    if (sc->fill_pct < 0 || sc->fill_pct > 400)
-        return fail(LB_ERR_INVALID_ARG, "fill_pct must be in [0, 400]");
-    if (sc->steps_per_launch < 0 || sc->steps_per_launch > 2)
-        return fail(LB_ERR_INVALID_ARG, "steps_per_launch must be 0, 1 or 2");
-
-    if (sc->persist && h->n_dom > 1 && !(h->precision == LB_FP32 && h->descs[0].compact))
-        return fail(LB_ERR_INVALID_ARG, "persistent schedules need compact FP32 storage");
-    const int rg = refresh_ghosts(h);  // the new schedule may split a domain into strips
-    if (rg != LB_OK) return rg;
-    LB_CUDA(cudaStreamSynchronize(h->stream));
-    clear_graphs(h);
-    lb_schedule v = *sc;
-    for (int c = v.n_class; c < LB_MAX_SCHED_CLASSES; ++c) {  // unused classes: class 0's values
-        v.max_nx[c] = 0;
-        v.block_x[c] = v.block_x[0];
-        v.rows[c] = v.rows[0];
-        v.ctas_per_sm[c] = v.ctas_per_sm[0];
-        v.seal_edges[c] = v.seal_edges[0];
-    }
-    v.max_nx[v.n_class - 1] = 0;
-    h->sched = v;
-    h->small_rows = 0;  // an explicit shape is the staged step's
-    return build_items(h);
-}
+int lb_set_schedule(lb_handle* h, const lb_schedule* sc) { return set_schedule(h, sc, false); }
 
 int lb_get_schedule(const lb_handle* h, lb_schedule* sc)
 {
@@ -2426,7 +2436,7 @@ int lb_autotune(lb_handle* h, int reps, int* block_x, int* rows, double* best_ms
         h->n_dom > 1 || !plain || (long long)h->descs[0].nx * h->descs[0].ny <= 200000;
     // one timing of candidate k (ms per step); negative on failure
     auto time_candidate = [&](size_t k, int len, int r) -> double {
-        if ((rc = lb_set_schedule(h, &cands[k])) != LB_OK) return -1.0;
+        if ((rc = set_schedule(h, &cands[k], true)) != LB_OK) return -1.0;
         if (small && k == 0 && (rc = use_small(small_rows(h))) != LB_OK) return -1.0;
         // two steps per launch read four-wide ghost columns
         if (two_step(h) && (rc = widen_ghosts(h)) != LB_OK) return -1.0;
@@ -2482,7 +2492,7 @@ int lb_autotune(lb_handle* h, int reps, int* block_x, int* rows, double* best_ms
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     if (rc == LB_OK) rc = sync_and_check(h);
-    const int rc2 = lb_set_schedule(h, rc == LB_OK ? &chosen : &old);
+    const int rc2 = set_schedule(h, rc == LB_OK ? &chosen : &old, true);
     const int rc3 = use_small(rc == LB_OK ? chosen_small : old_small);
     if (rc != LB_OK) return rc;
     if (rc2 != LB_OK) return rc2;
