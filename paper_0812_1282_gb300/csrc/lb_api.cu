@@ -2487,7 +2487,8 @@ int lb_autotune(lb_handle* h, int reps, int* block_x, int* rows, double* best_ms
         if (sc.first < best) {
             best = sc.first;
             chosen = cands[sc.second];
-            chosen_small = small && sc.second == 0 ? small_rows(h) : 0;
+            // domains with obstacles: the step they would take without is not timed
+            if (plain) chosen_small = small && sc.second == 0 ? small_rows(h) : 0;
         }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);

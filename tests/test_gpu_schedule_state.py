@@ -1,5 +1,7 @@
 """What a handle reports as its schedule is what it runs, and a schedule read
-and set again leaves it on the step it had: counted in launches per step."""
+and set again or an autotuned obstacle map that is taken off leaves it on the
+step it had: counted in launches per step."""
+import numpy as np
 import pytest
 
 pytestmark = pytest.mark.gpu
@@ -96,3 +98,19 @@ def test_batch_schedule_read_and_set_again(lbf):
         out.append((sim.save_state(), sim.schedule()))
         sim.close()
     assert out[0] == out[1]
+
+
+def test_autotuned_with_obstacles_then_without(lbf):
+    nx, ny = 120, 50
+    sim = lbf.Lattice(params(lbf, "fp32"), nx, ny)
+    sim.init_random(0.1, 3)
+    before = launches(sim, 64)
+    cls = np.zeros((ny, nx), np.uint8)
+    cls[20:24, 30:36] = 1
+    sim.set_geometry(cls, [0.0, 0.1])
+    sim.init_random(0.1, 3)
+    sim.autotune(reps=1)
+    sim.set_geometry(None, None)
+    sim.init_random(0.1, 3)
+    assert launches(sim, 64) == before
+    sim.close()
