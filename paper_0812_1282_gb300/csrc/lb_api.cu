@@ -1301,6 +1301,7 @@ int make_handle(const lb_params* per_dom, const int* nx, const int* ny, int n_do
         return rc;
     };
     if ((e = cudaError_t(lbfe::prepare_step_kernels())) != cudaSuccess ||
+        (e = cudaError_t(lbfe::prepare_small_steps())) != cudaSuccess ||
         (e = cudaError_t(lbfe::prepare_geo_step2())) != cudaSuccess)
         return bail(fail(LB_ERR_CUDA, "kernel setup failed: %s", cudaGetErrorString(e)));
     if ((e = cudaDeviceGetAttribute(&h->sm_count, cudaDevAttrMultiProcessorCount, h->device)) !=

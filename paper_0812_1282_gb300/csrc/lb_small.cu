@@ -706,6 +706,40 @@ int launch_small_step(int precision, int coll, const DomDesc& d, const DomDesc* 
     return int(launch_c<SmallKind::F32>(coll, d, descs, items, n_items, parity, rows, s));
 }
 
+namespace {
+
+// The several-step kernel of a storage, and the shared memory of its CTAs.
+using StepsKernel = void (*)(DomDesc, int, int, int);
+StepsKernel steps_kernel(bool compact, int coll)
+{
+    return compact ? (coll ? StepsKernel(small_steps_kernel<true, true>)
+                           : StepsKernel(small_steps_kernel<false, true>))
+                   : (coll ? StepsKernel(small_steps_kernel<true, false>)
+                           : StepsKernel(small_steps_kernel<false, false>));
+}
+size_t steps_smem(bool compact, int threads)
+{
+    return small_smem(compact ? SmallKind::Compact : SmallKind::F32, threads / kTX) +
+           size_t(compact ? 9 : 18) * threads * 4;
+}
+
+}  // namespace
+
+// The limit is the process's, not a launch's: the most any launch asks for, the
+// same value whoever sets it.
+int prepare_small_steps()
+{
+    for (int k = 0; k < 4; ++k) {
+        const bool compact = k & 1;
+        const cudaError_t e =
+            cudaFuncSetAttribute(steps_kernel(compact, k >> 1),
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 int(steps_smem(compact, kStepsMaxThreads)));
+        if (e != cudaSuccess) return int(e);
+    }
+    return 0;
+}
+
 int launch_small_steps(int coll, const DomDesc& d, int parity, int steps, int rows, void* stream)
 {
     if (steps < 2 || small_steps_cols(steps) < 1 || rows < 1 ||
@@ -713,18 +747,8 @@ int launch_small_steps(int coll, const DomDesc& d, int parity, int steps, int ro
         return int(cudaErrorInvalidValue);
     const int threads = small_steps_threads(steps, rows), w = small_steps_cols(steps);
     const dim3 grid((d.nx + w - 1) / w, (d.ny + rows - 1) / rows);
-    const size_t smem = small_smem(d.compact ? SmallKind::Compact : SmallKind::F32, threads / kTX) +
-                        size_t(d.compact ? 9 : 18) * threads * 4;
-    using Kernel = void (*)(DomDesc, int, int, int);
-    const Kernel kernel = d.compact
-        ? (coll ? Kernel(small_steps_kernel<true, true>) : Kernel(small_steps_kernel<false, true>))
-        : (coll ? Kernel(small_steps_kernel<true, false>) : Kernel(small_steps_kernel<false, false>));
-    if (smem > 48 * 1024) {
-        const cudaError_t e =
-            cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
-        if (e != cudaSuccess) return int(e);
-    }
-    kernel<<<grid, threads, smem, static_cast<cudaStream_t>(stream)>>>(d, parity, steps, rows);
+    steps_kernel(d.compact != 0, coll)<<<grid, threads, steps_smem(d.compact != 0, threads),
+                                         static_cast<cudaStream_t>(stream)>>>(d, parity, steps, rows);
     return int(cudaGetLastError());
 }
 

@@ -26,5 +26,7 @@ int launch_small_step(int precision, int coll, const DomDesc& d, const DomDesc* 
 // rows, small_steps_threads(steps, rows) <= kStepsMaxThreads; flips the buffer
 // once.
 int launch_small_steps(int coll, const DomDesc& d, int parity, int steps, int rows, void* stream);
+// Its shared-memory opt-in (once per device, outside any capture).
+int prepare_small_steps();
 
 }  // namespace lbfe
