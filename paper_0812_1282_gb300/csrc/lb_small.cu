@@ -695,7 +695,10 @@ cudaError_t launch_c(int coll, const DomDesc& d, const DomDesc* descs, const Wor
 int launch_small_step(int precision, int coll, const DomDesc& d, const DomDesc* descs,
                       const WorkItem* items, int n_items, int parity, int rows, void* stream)
 {
-    if (rows < 1 || rows > kSmallMaxThreads / kTX) return int(cudaErrorInvalidValue);
+    // FP32 full storage: the threads take the halo in one round (small_steps)
+    const int least = precision == 0 && !d.compact ? 3 : 1;
+    static_assert(3 * kTX >= 2 * kPW + 2 * 3, "a thread for each position");
+    if (rows < least || rows > kSmallMaxThreads / kTX) return int(cudaErrorInvalidValue);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     if (precision != 0 && rows <= kSmallSplitRows)
         return int(launch_c<SmallKind::Split64>(coll, d, descs, items, n_items, parity, rows, s));
@@ -742,8 +745,9 @@ int prepare_small_steps()
 
 int launch_small_steps(int coll, const DomDesc& d, int parity, int steps, int rows, void* stream)
 {
-    if (steps < 2 || small_steps_cols(steps) < 1 || rows < 1 ||
-        small_steps_threads(steps, rows) > kStepsMaxThreads)
+    // a region wraps around the lattice once at most
+    if (steps < 2 || small_steps_cols(steps) < 1 || rows < 1 || d.nx < 2 * steps ||
+        d.ny < 2 * steps || small_steps_threads(steps, rows) > kStepsMaxThreads)
         return int(cudaErrorInvalidValue);
     const int threads = small_steps_threads(steps, rows), w = small_steps_cols(steps);
     const dim3 grid((d.nx + w - 1) / w, (d.ny + rows - 1) / rows);
