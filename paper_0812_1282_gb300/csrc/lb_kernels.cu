@@ -361,12 +361,16 @@ __device__ __forceinline__ void block_reduce(MomAcc v, double& sum, unsigned lon
     }
 }
 
-// j / r to the last bit or so from one reciprocal of r: the product, and its
-// residual's correction.
+// j / r to the last bit or so from one reciprocal of r = 1 + (rho - 1), which is
+// 0 or at least 2^-53: the product, and its residual's correction.  Where that is no
+// finite number the product alone is the quotient: r infinite (0), r zero, j infinite
+// or a quotient that overflows.  (A division there costs 400 -> 690 us a reading of
+// 2048^2, though never taken.)
 __device__ __forceinline__ double div_by(double j, double r, double inv)
 {
     const double q = j * inv;
-    return fma(fma(-q, r, j), inv, q);
+    const double v = fma(fma(-q, r, j), inv, q);
+    return (__double2hiint(v) & 0x7ff00000) == 0x7ff00000 ? q : v;
 }
 
 template <typename Real>
