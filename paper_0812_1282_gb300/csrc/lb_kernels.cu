@@ -551,26 +551,37 @@ __device__ __forceinline__ double phi_at_node(const Real* g, long long P, long l
     return phi_sum<double>(v);
 }
 
-// An estimate of phi that costs no FP64 operation where the storage allows
-// one: the FP32 sum (compact: the word's value).
+// phi without an FP64 operation where the storage allows it: the FP32 sum, with
+// the size of its largest term (eight roundings of at most nine times that);
+// compact: the word's value, to half a bit.  FP64: the sum itself.
 template <typename Real>
-__device__ __forceinline__ Real phi_estimate(const Real* g, long long P, long long o, bool compact)
+struct PhiEstimate {
+    Real phi, size;
+};
+template <typename Real>
+__device__ __forceinline__ PhiEstimate<Real> phi_estimate(const Real* g, long long P, long long o,
+                                                          bool compact)
 {
-    if (sizeof(Real) == 4 && compact) return G0<Real>::value(g[o]);
+    if (sizeof(Real) == 4 && compact) return {G0<Real>::value(g[o]), Real(0)};
     Real v[9];
     for (int i = 0; i < 9; ++i) v[i] = g[i * P + o];
-    return phi_sum<Real>(v);
+    Real size = Real(0);
+    if (sizeof(Real) == 4) {
+        size = 4;  // the word's range
+        for (int i = 1; i < 9; i += 2) size = fmaxf(fmaxf(size, fabsf(v[i])), fabsf(v[i + 1]));
+    }
+    return {phi_sum<Real>(v), size};
 }
 
 // Whether a link whose ends have these estimates surely carries no crossing:
-// both of one sign, far from zero against the estimates' error (nine
-// roundings of numbers below 8: under 1e-5), and of a size phi has.  Only the
-// few links near the interface are evaluated in FP64.
+// both of one sign and farther from zero than 1e-3, against an error below 4e-5.
+// Only the few links near the interface are evaluated in FP64.
 template <typename Real>
-__device__ __forceinline__ bool surely_none(Real a, Real b)
+__device__ __forceinline__ bool surely_none(const PhiEstimate<Real>& a, const PhiEstimate<Real>& b)
 {
-    const Real lo = Real(1e-3), hi = Real(4);
-    return (a > lo && b > lo && a < hi && b < hi) || (a < -lo && b < -lo && a > -hi && b > -hi);
+    const Real lo = Real(1e-3), most = Real(8);
+    return a.size < most && b.size < most &&
+           ((a.phi > lo && b.phi > lo) || (a.phi < -lo && b.phi < -lo));
 }
 
 template <typename Real>
@@ -597,7 +608,7 @@ __global__ void crossings_kernel(DomDesc D, int parity, double* pts, int* count,
         const long long ob = (long long)y * pitch + xp + kXOff, oc = o + pitch;
         const bool right = !cls || cls[y * nx + xp] == 0;
         const bool up = y + 1 < ny && (!cls || cls[k + nx] == 0);
-        const Real ea = phi_estimate(gs, P, o, cmp);
+        const PhiEstimate<Real> ea = phi_estimate(gs, P, o, cmp);
         const bool look_right = right && !surely_none(ea, phi_estimate(gs, P, ob, cmp));
         const bool look_up = up && !surely_none(ea, phi_estimate(gs, P, oc, cmp));
         if (!look_right && !look_up) continue;

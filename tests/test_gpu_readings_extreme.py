@@ -1,5 +1,6 @@
 """Readings of states beyond ordinary numbers: velocities where rho or the
-momentum overflows."""
+momentum overflows, and crossings where the populations are far larger than
+phi."""
 import numpy as np
 import pytest
 
@@ -72,4 +73,45 @@ def test_velocity_that_overflows(lbf):
         with np.errstate(over="ignore"):
             r = rho[3, 7] if want > 0 else rho[1, 9]
             assert u == np.float64(want) / r
+    sim.close()
+
+
+def crossings(phi):
+    """The phi = 0 points on horizontal (periodic) and vertical links."""
+    ny, nx = phi.shape
+    pts = []
+    for y in range(ny):
+        for x in range(nx):
+            a, b = phi[y, x], phi[y, (x + 1) % nx]
+            if a * b < 0:
+                pts.append((x + a / (a - b), y))
+            if y + 1 < ny and a * phi[y + 1, x] < 0:
+                pts.append((x, y + a / (a - phi[y + 1, x])))
+    return pts
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+@pytest.mark.parametrize("big", [2.0 ** 25, 2.0 ** 40])
+def test_crossings_among_large_populations(lbf, oracle_mod, precision, big):
+    """phi = -0.4 in a disc where g_1 = -g_3 = big, so that the sum of the g in
+    FP32 comes out at about +0.5: the disc's edge is an interface."""
+    nx, ny = 64, 48
+    y, x = np.mgrid[0:ny, 0:nx]
+    disc = np.hypot(x - 30.3, y - 20.2) < 11.4
+    g = np.zeros((9, ny, nx))
+    g[0] = np.where(disc, -0.9, 0.5)
+    g[5] = np.where(disc, 0.5, 0.0)
+    g[1] = np.where(disc, big, 0.0)
+    g[3] = np.where(disc, -big, 0.0)
+    sim = lbf.Lattice(lbf.params(precision=precision), nx, ny)
+    sim.set_populations(rest(ny, nx), g)
+    gs = sim.populations()[1]
+    # in the order the library sums in FP64: pairs
+    phi = (((gs[0] + gs[1]) + (gs[2] + gs[3])) + ((gs[4] + gs[5]) + (gs[6] + gs[7]))) + gs[8]
+    assert (phi[disc] < 0).all() and (phi[~disc] > 0).all()
+    assert len(crossings(phi)) > 40
+    got = sim.contact_angle(exclude=0.0)
+    want = oracle_mod.contact_angle(phi, exclude=0.0)
+    for a, b in zip(got, want):
+        assert abs(a - b) <= 1e-9 * max(1.0, abs(b))
     sim.close()
