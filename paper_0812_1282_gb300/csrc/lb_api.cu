@@ -1912,6 +1912,12 @@ int lb_set_geometry(lb_handle* h, int dom, const unsigned char* cls, const doubl
         D.cls = nullptr;
     }
     h->n_geo += (D.cls != nullptr) - int(had);
+    if (had && !cls) {
+        // the obstacle step keeps no periodic ghost columns, the others read them
+        const int e = lbfe::launch_fill_ghosts(h->precision, D, h->parity, h->stream);
+        if (e != 0) return fail(LB_ERR_CUDA, "ghost fill failed: %s", cudaGetErrorString(cudaError_t(e)));
+        h->launches += 1;
+    }
     LB_CUDA(cudaMemcpyAsync(h->d_descs() + dom, &D, sizeof(DomDesc), cudaMemcpyHostToDevice,
                             h->stream));
     LB_CUDA(cudaStreamSynchronize(h->stream));
