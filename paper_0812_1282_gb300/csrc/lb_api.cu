@@ -597,7 +597,7 @@ int build_items(lb_handle* h)
 // fewest iterations over all waves is taken, up to 160 rows (more lose the
 // shared rows between bands in L2), 64-wide CTAs counted 7 % dearer (their
 // halo columns).  Measured, us per step, one step per launch and two: 700^2
-// 13.9 and 12.7, 1024^2 25.3 and 23.0, 2048^2 79.7 and 67.6, 4096^2 272 and
+// 13.9 and 12.7, 1024^2 25.3 and 23.0, 2048^2 79.7 and 66.4, 4096^2 272 and
 // 236, 8192^2 1035 and 880; but 1000 x 500 13.8 and 14.4, and 160 x 5000, whose
 // strips are a third empty, 20.4 and 21.8.
 bool two_step_shape(const lb_handle* h, lb_schedule& s)

@@ -11,12 +11,12 @@ namespace lbfe {
 // Tiles of the per-step form, 32 columns x `rows`: those with a fluid or wall
 // node, the ones whose fluid touches a solid node first and marked by their
 // sign bit (they take longer).  FP32 takes 8 rows while all tiles are
-// resident at once (three to an SM), else 4, of which more fit (us per step:
-// 1000 x 120 channel, 255 tiles of 8 rows, 5.3 with 8 and 6.2 with 4; 2000 x
-// 200, 950 tiles, 13.4 and 10.9).  FP64 takes 4: the FP64 pipe of each SM is
-// the bound and smaller tiles share the work out more evenly (401 x 77: 10.2
-// with 4, 13.9 with 8, 12.6 with 2).  geo_tile_capacity: the most entries a
-// list can have.
+// resident at once (three to an SM), else 4, of which more fit (us per step with 8
+// and 4 rows of channels with so many tiles of 8 rows: 230 (1000 x 120) 3.7 and
+// 5.2, 428 5.0 and 5.4, 482 7.3 and 5.6, 735 8.7 and 8.2, 1011 (2000 x 200) 12.2
+// and 9.8).  FP64 takes 4: the FP64 pipe of each SM is the bound and smaller tiles
+// share the work out more evenly (401 x 77, before the extra warps: 10.2 with 4,
+// 13.9 with 8, 12.6 with 2).  geo_tile_capacity: the most entries a list can have.
 constexpr int kGeoTileIndex = 0x7fffffff;
 struct GeoTiles {
     int rows;

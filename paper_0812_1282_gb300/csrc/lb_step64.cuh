@@ -19,7 +19,7 @@
 //
 // Measured (MRT, 2048^2, best tile, per step): 1828 us with per-warp halos,
 // the phi ring read nine times a node and the plain arithmetic, 828 us so
-// (5.07 G node updates/s, 0.94 of what 112 + 4 operations allow at the
+// (5.07 G node updates/s, 0.925 of what 114.6 operations a node allow at the
 // pipe's 628 G DFMA/s); BGK 900 us.  Wall rows take a copy of the code of
 // their own: their tests and ghost values in the common one cost it 7 %
 // (890 us).  128 x 8 tiles are fastest there, 64 x 16

@@ -34,12 +34,12 @@
 // other compact values two, and B takes A's words from A's own word ring.
 //
 // What bounds it is instruction issue and the latency within an iteration (4096^2:
-// 52 % of issue slots, DRAM at 41 %, 10.3 warp instructions a node
-// update; waits for fixed-latency results, the barrier and the stage in that
-// order), with two CTAs of eight compute warps to an SM, which their shared
+// 62 % of issue slots, DRAM at 46 %, 10.4 warp instructions a node
+// update; waits for fixed-latency results, the barrier, the FMA pipe and the stage
+// in that order), with two CTAs of eight compute warps to an SM, which their shared
 // memory (98 KB at NW = 4) and registers (96) allow.  Two stages: three made
 // no difference.  Measured: 8192^2 1034 -> 880 us a step (64.9 -> 76.3 G node
-// updates/s), 2048^2 79.7 -> 67.6.
+// updates/s), 2048^2 79.7 -> 66.4.
 #pragma once
 
 #include "lb_step_kernels.cuh"
