@@ -264,13 +264,19 @@ __device__ __forceinline__ bool geo_ghost(const DomDesc& D, const GeoConst<Real>
     return true;
 }
 
+// The parts of a node's phi that its collision wants (FP64).
+template <typename Real>
+struct GeoPhi {};
+template <>
+struct GeoPhi<double> : Phi64 {};
+
 // Collision of one fluid node from its pulled f, g, its phi c and the phi of
 // its eight neighbours (ghost values at solid ones), directions 1..8 in nb.
 template <typename Real, bool MRT>
 __device__ __forceinline__ void geo_collide(const DomDesc& D, const GeoConst<Real>& K,
                                             const Real (&f)[9], const Real (&g)[9], Real c,
-                                            const Real (&nb)[9], bool step2, Real (&fo)[9],
-                                            Real (&go)[9])
+                                            const GeoPhi<Real>& s, const Real (&nb)[9],
+                                            bool step2, Real (&fo)[9], Real (&go)[9])
 {
     if constexpr (sizeof(Real) == 8) {
         const Node64& C = K.c;
@@ -281,8 +287,8 @@ __device__ __forceinline__ void geo_collide(const DomDesc& D, const GeoConst<Rea
         const double a = LB64_ADD(LB64_ADD(nb[1], nb[2]), LB64_ADD(nb[3], nb[4]));
         const double d = LB64_ADD(LB64_ADD(nb[5], nb[6]), LB64_ADD(nb[7], nb[8]));
         const double L = __fma_rn(C.m20, c, __fma_rn(C.four, a, d));
-        collide64<MRT>(C, f, c, LB64_MUL(C.sig, X), LB64_MUL(C.sig, Y), LB64_MUL(C.sig, L), step2,
-                       D.step2_relax_j != 0,
+        collide64<MRT>(C, f, c, s, LB64_MUL(C.sig, X), LB64_MUL(C.sig, Y), LB64_MUL(C.sig, L),
+                       step2, D.step2_relax_j != 0,
                        [&](double (&v)[9]) {
 #pragma unroll
                            for (int i = 0; i < 9; ++i) v[i] = g[i];
@@ -299,12 +305,18 @@ __device__ __forceinline__ void geo_collide(const DomDesc& D, const GeoConst<Rea
 
 // phi = sum of the pulled g
 template <typename Real>
-__device__ __forceinline__ Real geo_phi(const GeoConst<Real>& K, const Real (&g)[9])
+__device__ __forceinline__ Real geo_phi(const GeoConst<Real>& K, const Real (&g)[9], GeoPhi<Real>& s)
 {
     if constexpr (sizeof(Real) == 8)
-        return phi64(K.c, g);
+        return phi64(K.c, g, s);
     else
         return phi_sum<Real>(g);
+}
+template <typename Real>
+__device__ __forceinline__ Real geo_phi(const GeoConst<Real>& K, const Real (&g)[9])
+{
+    GeoPhi<Real> s;
+    return geo_phi<Real>(K, g, s);
 }
 
 // Halo position k of a tile, relative to its first node: the one-node ring
@@ -544,8 +556,9 @@ __device__ __forceinline__ void geo_tile_step(const GeoTile<Real, TY, N>& T,
     // a short last tile's threads beyond the lattice take part in the phi array
     // too: their columns and rows are the wrapped ones
     Real c = Real(0);
+    GeoPhi<Real> s;
     if (live) {
-        c = geo_phi<Real>(K, g);
+        c = geo_phi<Real>(K, g, s);
         ph[T.at(x, y)] = c;
     } else if (p.phi_only) {
         pull(gs, p.own, g);
@@ -572,7 +585,7 @@ __device__ __forceinline__ void geo_tile_step(const GeoTile<Real, TY, N>& T,
         Real nb[9];
 #pragma unroll
         for (int i = 1; i < 9; ++i) nb[i] = ph[T.at(x + gex(i), y + gey(i))];
-        geo_collide<Real, MRT>(D, K, f, g, c, nb, D.step2 != 0 && p.next_to_solid, fo, go);
+        geo_collide<Real, MRT>(D, K, f, g, c, s, nb, D.step2 != 0 && p.next_to_solid, fo, go);
     }
     Real* fd = static_cast<Real*>(parity ? D.f[0] : D.f[1]);
     Real* gd = static_cast<Real*>(parity ? D.g[0] : D.g[1]);
@@ -674,8 +687,9 @@ __device__ __forceinline__ void geo_node_update(const DomDesc& D, const GeoConst
             nb[i] = phi_l(qx, qy);
         }
     }
-    geo_collide<Real, MRT>(D, K, f, g, geo_phi<Real>(K, g), nb, D.step2 != 0 && next_to_solid, fo,
-                           go);
+    GeoPhi<Real> s;
+    const Real c = geo_phi<Real>(K, g, s);
+    geo_collide<Real, MRT>(D, K, f, g, c, s, nb, D.step2 != 0 && next_to_solid, fo, go);
 }
 
 template <typename Real>

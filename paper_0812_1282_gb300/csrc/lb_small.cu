@@ -210,14 +210,14 @@ __device__ __forceinline__ void small_step64(const DomDesc& D, int parity, const
     const double wv = tid == 0 ? wet_bottom<double>(D) : (tid == 1 ? wet_top<double>(D) : 0.0);
     load_node64(C, D.c64, tid);
     __syncthreads();
-    auto put = [&](int cx, int cy, const double (&v)[9], double& phi) {
-        phi = phi64(C, v);
-        ph[(cy + 1) * kPW + cx + 1] = LB64_MUL(C.sig, phi);
-    };
-    double c = 0.0, dump;
-    if (live) put(tx, ty, g, c);
+    Phi64 s;
+    double c = 0.0;
+    if (live) {
+        c = phi64(C, g, s);
+        ph[(ty + 1) * kPW + tx + 1] = LB64_MUL(C.sig, c);
+    }
     for (;;) {
-        if (halo) put(hx, hy, gh, dump);
+        if (halo) ph[(hy + 1) * kPW + hx + 1] = LB64_MUL(C.sig, phi64(C, gh));
         k += int(blockDim.x);
         if (k >= nh) break;
         halo = halo_at(k, T.wc, T.hc, hx, hy) && inside(T.y0 + hy);
@@ -232,7 +232,7 @@ __device__ __forceinline__ void small_step64(const DomDesc& D, int parity, const
     double fo[9], go[9];
     double X, Y, L;
     deriv64(C, D, r0, blo, bhi, wet, X, Y, L);
-    collide64<MRT>(C, f, c, X, Y, L, s2, D.step2_relax_j != 0,
+    collide64<MRT>(C, f, c, s, X, Y, L, s2, D.step2_relax_j != 0,
                    [&](double (&v)[9]) {
 #pragma unroll
                        for (int i = 0; i < 9; ++i) v[i] = g[i];
@@ -292,9 +292,10 @@ __device__ __forceinline__ void small_split64(const DomDesc& D, int parity, cons
     __syncthreads();
     double c = 0.0;
     Moments64 m;
+    Phi64 s;
     if (live) {
         if (is_g) {
-            c = phi64(C, v);
+            c = phi64(C, v, s);
             ph[(ty + 1) * kPW + tx + 1] = LB64_MUL(C.sig, c);
             ex[3 * half + node] = c;
         } else {
@@ -325,7 +326,7 @@ __device__ __forceinline__ void small_split64(const DomDesc& D, int parity, cons
         m.jy = ex[2 * half + node];
         velocity64(C, c, s2, m);
         deriv64(C, D, r0, blo, bhi, wet, X, Y, L);
-        collide_g64(C, m, c, LB64_MUL(c, c), L,
+        collide_g64(C, m, c, LB64_MUL(c, c), s, L,
                     [&](double (&g)[9]) {
 #pragma unroll
                         for (int i = 0; i < 9; ++i) g[i] = v[i];

@@ -87,6 +87,7 @@ __device__ __forceinline__ void consume_tile64(const DomDesc& D, const Node64& C
     // row values k, h, m on the scaled phi, and the scaled phi itself
     struct Row {
         double phi, s, k, h, m;
+        Phi64 g;
     };
     auto publish = [&](int p, Row& v, bool blo, bool bhi) {
         const double* sg = stage_ptr(p) + 9 * segw;
@@ -94,7 +95,7 @@ __device__ __forceinline__ void consume_tile64(const DomDesc& D, const Node64& C
         double g[9];
         if (active) {
             read9<double>(sg, segw, col + 4, blo, bhi, g);
-            v.phi = phi64(C, g);
+            v.phi = phi64(C, g, v.g);
             v.s = LB64_MUL(C.sig, v.phi);
             rr[col + 1] = v.s;
         }
@@ -122,7 +123,7 @@ __device__ __forceinline__ void consume_tile64(const DomDesc& D, const Node64& C
     auto wrap_row = [&](int r) { return r < 0 ? r + ny : (r >= ny ? r - ny : r); };
     Row cur, nxt;
     double km = 0.0, mm = 0.0;  // k and m of row y - 1
-    cur.phi = cur.s = cur.k = cur.h = cur.m = 0.0;
+    cur.phi = cur.s = cur.k = cur.h = cur.m = cur.g.g0 = cur.g.tail = 0.0;
     nxt = cur;
     // collide row y (staged at position p) from the row values around it
     auto collide_row = [&](int y, int p, bool blo, bool bhi) {
@@ -132,7 +133,7 @@ __device__ __forceinline__ void consume_tile64(const DomDesc& D, const Node64& C
         const double dy = LB64_SUB(nxt.m, mm);
         const double lap = __fma_rn(C.m20, cur.s, __fma_rn(C.four, cur.h, LB64_ADD(nxt.m, mm)));
         double fo[9], go[9];
-        collide64<MRT>(C, f, cur.phi, dx, dy, lap, D.step2 && (blo || bhi), D.step2_relax_j != 0,
+        collide64<MRT>(C, f, cur.phi, cur.g, dx, dy, lap, D.step2 && (blo || bhi), D.step2_relax_j != 0,
                        [&](double (&g)[9]) {
                            read9<double>(stage_ptr(p) + 9 * segw, segw, col + 4, blo, bhi, g);
                        },
