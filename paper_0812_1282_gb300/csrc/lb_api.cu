@@ -750,7 +750,7 @@ lb_schedule default_schedule(const lb_handle* h)
 // staged and small: FP32 28 x 15 4.0 and 1.4, 200 x 100 4.3 and 1.8, 1000 x 500
 // 15.4 and 13.3, 2000 x 350 20.7 and 20.0, but 900^2 24.4 and 27.4; compact
 // 28 x 15 4.5 and 1.8, 200 x 100 4.8 and 2.2, 512 x 256 7.2 and 5.9, but 700 x
-// 300 7.8 and 8.8; FP64 28 x 15 8.3 and 5.1, 200 x 100 11 and 7.5, 1000 x 500
+// 300 7.8 and 8.8; FP64 28 x 15 8.3 and 5.1, 200 x 100 11 and 7.6, 1000 x 500
 // 115 and 111, but 1200^2 313 and 302 to 317, 2048^2 828 and 850).  In a batch
 // a tile first finds its domain, two loads in series: 6 domains of 22 k nodes
 // FP32 6.6 and 3.3, compact 7.6 and 3.8, FP64 14.3 and 8.7, 8 of 178 k 11.7 and

@@ -47,7 +47,7 @@
 // 1000 x 120 channel FP32 7.6 -> 3.7 (a three-node phi halo in every tile,
 // ghost values formed anew for each fluid neighbour, g pulled twice, tiles of
 // solid nodes launched; then as above), 2000 x 200 FP32 18 -> 9.8, 401 x 77
-// FP64 22 -> 8.9 (with the arithmetic of lb_node64.cuh); a single tile 4.2 ->
+// FP64 22 -> 9.0 (with the arithmetic of lb_node64.cuh); a single tile 4.2 ->
 // 2.5.
 #include <cuda_runtime.h>
 

@@ -17,7 +17,7 @@
 //  - the two reciprocals 1/rho and 1/tau come from one of rho tau;
 //  - constant factors of the stencils (kappa, 1/12, 1/6) are folded into the
 //    node constants, and the stencils into running row values (lb_step64.cuh).
-// 114.6 operations a node (counted, MRT) where the plain form has 203.6.  All products
+// 115.6 operations a node (counted, MRT) where the plain form has 203.6.  All products
 // and sums are explicit fused operations, so every kernel that calls these
 // functions gets the same bits.
 #pragma once

@@ -22,7 +22,7 @@
 //    (small_split64).
 // us a step, staged, one step per launch, and as here: FP32 28 x 15 4.0, 2.3, 1.4,
 // 200 x 100 4.4, 2.7, 1.8; compact 28 x 15 4.5, 3.4, 1.8, 200 x 100 4.9, 3.5, 2.2;
-// FP64 28 x 15 8.3, 6.6, 5.1, 200 x 100 11, 7.5.
+// FP64 28 x 15 8.3, 6.6, 5.1, 200 x 100 11, 7.6.
 // The arithmetic is that of the staged kernels, operation for operation, and
 // so are the stored populations and ghost columns, bit for bit.
 #include <cuda_runtime.h>

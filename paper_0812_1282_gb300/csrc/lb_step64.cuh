@@ -18,9 +18,9 @@
 // the same sequence of barriers whatever its bounded stage waits return.
 //
 // Measured (MRT, 2048^2, best tile, per step): 1828 us with per-warp halos,
-// the phi ring read nine times a node and the plain arithmetic, 828 us so
-// (5.07 G node updates/s, 0.925 of what 114.6 operations a node allow at the
-// pipe's 628 G DFMA/s); BGK 900 us.  Wall rows take a copy of the code of
+// the phi ring read nine times a node and the plain arithmetic, 834 us so
+// (5.03 G node updates/s, 0.925 of what 115.6 operations a node allow at the
+// pipe's 628 G DFMA/s); BGK 907 us.  Wall rows take a copy of the code of
 // their own: their tests and ghost values in the common one cost it 7 %
 // (890 us).  128 x 8 tiles are fastest there, 64 x 16
 // within 1 %; wider tiles leave too few CTAs per SM to hide the barrier.
