@@ -2369,6 +2369,12 @@ int lb_autotune(lb_handle* h, int reps, int* block_x, int* rows, double* best_ms
     const bool plain = h->n_dom == 1 ? h->descs[0].cls == nullptr : h->n_items > 0;
     std::vector<lb_schedule> cands;
     bool small = false;  // candidate 0 is the small-lattice step
+    // a small lattice: launches of a few us, of which at least four are timed, and of
+    // the staged step no tall shapes, whose CTAs march alone (all shapes as graphs of 16
+    // steps and the fastest eight again of 64: 350 ms for 512 x 256 FP64, 44 for 200 x
+    // 100 FP32, and the same choice)
+    const bool brief =
+        h->n_dom == 1 && plain && (long long)h->descs[0].nx * h->descs[0].ny <= 200000;
     if (!plain) {
         cands.push_back(h->sched);
         if (h->n_dom == 1) {
@@ -2394,6 +2400,7 @@ int lb_autotune(lb_handle* h, int reps, int* block_x, int* rows, double* best_ms
             h->descs[0].compact ? std::vector<int>{32, 64, 96, 128, 160, 192, 224, 256, 288}
                                 : std::vector<int>{64, 128, 256};
         std::vector<int> rws = {4, 8, 16, 32, 64, 128};
+        if (brief) rws.resize(3);
         // the shape by size, and the small-lattice step where that is the rule
         lb_schedule def = h->sched;
         const lb_schedule ds = default_schedule(h);
@@ -2438,9 +2445,7 @@ int lb_autotune(lb_handle* h, int reps, int* block_x, int* rows, double* best_ms
     double best = 1e300;
     lb_schedule chosen = old;
     int chosen_small = old_small, rc = LB_OK;
-    // single launches of a small lattice would time the host's launch rate
-    const bool graphs =
-        h->n_dom > 1 || !plain || (long long)h->descs[0].nx * h->descs[0].ny <= 200000;
+    const bool graphs = h->n_dom > 1 || !plain;
     // one timing of candidate k (ms per step); negative on failure
     auto time_candidate = [&](size_t k, int len, int r) -> double {
         if ((rc = set_schedule(h, &cands[k], true)) != LB_OK) return -1.0;
@@ -2450,9 +2455,11 @@ int lb_autotune(lb_handle* h, int reps, int* block_x, int* rows, double* best_ms
         if (graphs) return time_graph_steps(h, len, r, e0, e1);
         // warm-up, then time `r` launches that read the current buffer and
         // write the idle one (the state itself does not advance)
+        if (brief) r = std::max(r, 4);
+        const int per = single_steps(h);
         auto launch = [&]() {
-            return two_step(h) ? launch_several(h, 2, h->parity, h->stream)
-                               : enqueue_step(h, h->parity, h->stream);
+            return per > 1 ? launch_several(h, per, h->parity, h->stream)
+                           : enqueue_step(h, h->parity, h->stream);
         };
         if ((rc = launch()) != LB_OK) return -1.0;
         cudaEventRecord(e0, h->stream);
@@ -2463,10 +2470,10 @@ int lb_autotune(lb_handle* h, int reps, int* block_x, int* rows, double* best_ms
         h->launches += (r + 1) * launches_per_step(h);
         if (cudaEventSynchronize(e1) != cudaSuccess || cudaEventElapsedTime(&t, e0, e1) != cudaSuccess)
             return -1.0;
-        return double(t) / (two_step(h) ? 2 * r : r);
+        return double(t) / (per * r);
     };
-    // a batch or a small lattice: graphs of 16 steps, so that chains and tails
-    // show; then the fastest eight again over graphs of the length the steps run in (the
+    // a batch: graphs of 16 steps, so that chains and tails show; then the
+    // fastest eight again over graphs of the length the steps run in (the
     // leading candidates are within a few percent of each other)
     std::vector<std::pair<double, size_t>> scored;
     for (size_t k = 0; k < cands.size(); ++k) {
