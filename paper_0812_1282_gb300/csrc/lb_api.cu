@@ -1490,11 +1490,9 @@ bool fit_circle(const std::vector<double>& pts, double& xc, double& yc, double& 
 // s + 2d in the directions its ghost value uses.
 int check_geometry(const unsigned char* cls, int nx, int ny, int walls)
 {
-    auto at = [&](int x, int y) {
-        x = ((x % nx) + nx) % nx;
-        y = ((y % ny) + ny) % ny;
-        return int(cls[size_t(y) * nx + x]);
-    };
+    // offsets of up to two nodes of at least three
+    auto wrap = [](int v, int n) { return v < 0 ? v + n : (v >= n ? v - n : v); };
+    auto at = [&](int x, int y) { return int(cls[size_t(wrap(y, ny)) * nx + wrap(x, nx)]); };
     // for the mirror rule a wall node is not fluid (a mirror may not land on one)
     auto solid = [&](int x, int y) {
         if (walls && (y < 0 || y >= ny)) return true;
